@@ -12,30 +12,33 @@
 //
 // Persistent CTAs (one per SM) take work items (request, KV head, key chunk, row group) from a
 // global counter, in the planner's longest-first order.  Warp roles in a CTA:
-//   * warp 6 (item loader) takes the next item just in time (when the K producer is three tiles
+//   * warp 2 (item loader) takes the next item just in time (when the K producer is three tiles
 //     from the end of the current one), publishes it to the other warps through a 4-slot shared
 //     ring, and copies its query rows into one of two shared Q buffers (128-byte-swizzled,
 //     K-major: the B operand of S^T);
-//   * warps 0 and 7 (K and V producers) stream the item's K and V tiles of 128 tokens with TMA
+//   * warps 0 and 3 (K and V producers) stream the item's K and V tiles of 128 tokens with TMA
 //     tiled loads into two rings: one 16 KB box per 64-wide half of the head dim when the tile's
 //     eight 16-token blocks are consecutive in the pool, else one 2 KB box per block; blocks past
 //     the item read as zeros (out-of-range box).  A K stage is free again once S^T of its tile is
 //     done, a V stage once its PV product is;
-//   * warp 1 (one thread) issues tcgen05.mma: S^T into one of two TMEM tiles (key t in TMEM lane
-//     t, query row j in column j), and O^T into the item's TMEM accumulator (head-dim index d in
-//     lane d, row j in column j; two accumulators alternating between items);
-//   * warps 2-5 and 12-15 (softmax): the first group takes rows 0-31 of an item, the second rows
-//     32-63; within a group one warp per TMEM lane quadrant, i.e. 32 keys of each tile per warp: a
-//     thread holds one key's scores for the group's rows.  The rows' reference maxima live in
-//     shared memory; a tile whose scores exceed a reference by more than 2^8 anywhere (the first
-//     tile of an item always does) makes the warps agree on new maxima (exact per-row tile
-//     maxima) and, if O holds earlier tiles, rescale their O^T columns in TMEM.  Each thread
-//     writes its key's part of the P row (bf16, MN-major, swizzled: the B operand of the PV
-//     product) and keeps its share of every row sum;
+//   * warps 1 and 16 (one thread of each) issue tcgen05.mma: warp 1 S^T into one of two TMEM tiles
+//     (key t in TMEM lane t, query row j in column j), warp 16 O^T into the item's TMEM accumulator
+//     (head-dim index d in lane d, row j in column j; two accumulators alternating between items);
+//   * warps 4-7 and 12-15 (softmax): the first group takes the first half of an item's rows, the
+//     second the rest; within a group one warp per TMEM lane quadrant, i.e. 32 keys of each tile per
+//     warp: a thread holds one key's scores for the group's rows.  The rows' reference maxima are
+//     those of the item's first tile and stay fixed.  Each thread writes its key's part of the P row
+//     (bf16, MN-major, swizzled: the B operand of the PV product) and keeps its share of every row sum;
 //   * warps 8-11 (epilogue) add the row-sum shares, read O^T from TMEM and write the normalised
 //     output or, for a split item, the (O, m, l) partials; the last chunk of a split
 //     (request, head, row group) to finish merges all its chunks.  This runs while the softmax
 //     warps are already on the next item.
+// What bounds it: the K and V stream (HBM).  An SM's own limit is the softmax warps' chain per tile
+// (read S^T, P, publish): 0.80 us a 128-key tile at 4 query rows and 1.06 us at 64 with K and V in L2,
+// against the 1.47 us that a tile's 64 KB take at an SM's share of the copy rate (D = 128).  With one
+// thread issuing both products, a vote of the softmax warps per tile and the barrier pointers in local
+// memory those were 1.42 and 1.78 us.
+//
 // Every mbarrier wait is bounded in time; an expired wait records WISP_DEV_TIMEOUT and the CTA
 // drains.  No named barrier is used: a warp that gives up cannot leave the others blocked, and the
 // TMEM is freed once every warp has arrived on a final mbarrier.
@@ -53,14 +56,17 @@ namespace {
 
 constexpr int kBT = 128;            // KV tokens per tile (the M of S^T)
 constexpr int kNR = kTcRowsPerItem; // query rows per item at most (64: the planner cuts larger sets)
-constexpr int kThreads = 512;       // warp 0 K producer, warp 1 MMA, warps 2-5 softmax (rows 0-31), warp 6
-                                    // item loader, warp 7 V producer, warps 8-11 epilogue, warps 12-15
-                                    // softmax (rows 32-63)
+constexpr int kThreads = 640;       // warps 0-3 K producer, S^T issuer, item loader and V producer; 4-7 softmax
+                                    // (first half of the rows); 8-11 epilogue; 12-15 softmax (second half);
+                                    // 16 PV issuer (17-19 have no work: registers are allotted per four warps)
 constexpr int kSoftmaxWarps = 8;
 constexpr uint32_t kTmemCols = 256; // S^T[2] at columns 0 / 64, O^T[2] at 128 / 192
 constexpr long long kWaitCycles = 4000000000LL;  // about two seconds: a wait that long is a failure
-constexpr float kTau = 8.0f;        // lazy rescale threshold (log2 units)
-constexpr float kExpTau = 256.0f;   // 2^kTau
+// Largest P = 2^(s - m) an item may hold: m is the maximum of a row's first tile, so later scores may
+// exceed it.  P (bf16), its row sums and O (fp32) keep their relative precision at any exponent; up to
+// 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it is
+// computed again by its epilogue warps (item_exact).
+constexpr float kMaxP = 0x1p64f;
 static_assert(kNR == 64, "TMEM and shared-memory layout assume 64 rows per item");
 
 template <int D>
@@ -82,26 +88,61 @@ struct Cfg {
   static constexpr int OFF_P = OFF_V + NSV * KV_TILE;
   static constexpr int OFF_BAR = OFF_P + NP * P_BYTES;
   static constexpr int N_BAR = 2 * NSK + 2 * NSV + 8 + 2 * NP + 6 + 1 + 2 * RING + 5;
-  static constexpr int OFF_MW = (OFF_BAR + N_BAR * 8 + 15) / 16 * 16;  // float [8][32] per-warp row maxima
-  static constexpr int OFF_FW = OFF_MW + kSoftmaxWarps * 32 * 4;       // float [8][32] per-warp rescale factors
-  static constexpr int OFF_RED = OFF_FW + kSoftmaxWarps * 32 * 4;      // float [4][64] tile maxima per quadrant
-  static constexpr int OFF_FLAG = OFF_RED + 4 * kNR * 4;               // uint32 [2][8] exceed votes per warp
-  static constexpr int OFF_HL = OFF_FLAG + 64;                         // float [2][4][64] row-sum shares per quadrant
+  static constexpr int OFF_MW = (OFF_BAR + N_BAR * 8 + 15) / 16 * 16;  // float [8][32] per warp: minus the rows' references
+  static constexpr int OFF_RED = OFF_MW + kSoftmaxWarps * 32 * 4;      // float [2][4][64] first-tile maxima per quadrant
+  static constexpr int OFF_HL = OFF_RED + 2 * 4 * kNR * 4;             // float [2][4][64] row-sum shares per quadrant
   static constexpr int OFF_HM = OFF_HL + 2 * 4 * kNR * 4;              // float [2][64] row reference maxima
-  static constexpr int OFF_EM = OFF_HM + 2 * kNR * 4;                  // float [2][64] merge: max, 1 / sum
-  static constexpr int OFF_MISC = OFF_EM + 2 * kNR * 4;                // tmem base, flags
+  static constexpr int OFF_EX = OFF_HM + 2 * kNR * 4;                  // float [128 + 4] item_exact: a block's weights
+  static constexpr int OFF_MISC = OFF_EX + (kBT + 4) * 4;              // tmem base, flags
   static constexpr int OFF_RING = OFF_MISC + 64;                       // RING x (index, WorkItem)
   static constexpr int SMEM = OFF_RING + RING * 64 + 1024;             // + slack to align the base to 1024
   static_assert(SMEM <= 227 * 1024, "shared memory of one CTA on sm_103a");
   static_assert(OFF_K % 1024 == 0 && OFF_V % 1024 == 0 && OFF_P % 1024 == 0, "swizzled buffers need 1 KB alignment");
 };
 
+// The CTA's mbarriers: shared-memory addresses at constant offsets from one base.
+template <int D>
 struct Bars {
-  uint64_t *k_full, *k_empty, *v_full, *v_empty, *q_full, *q_empty, *s_full, *s_empty, *p_full, *o_full;
-  uint64_t *o_empty, *o_done, *ep_full, *mma_done, *it_full, *it_empty, *egrp, *sm_sync, *sm_sync2, *fin, *claim;
+  using C = Cfg<D>;
+  uint32_t base;
+  __device__ __forceinline__ uint32_t at(int i) const { return base + 8 * i; }
+  static constexpr int K_FULL = 0, K_EMPTY = C::NSK, V_FULL = 2 * C::NSK, V_EMPTY = V_FULL + C::NSV;
+  static constexpr int Q_FULL = V_EMPTY + C::NSV, Q_EMPTY = Q_FULL + 2, S_FULL = Q_EMPTY + 2, S_EMPTY = S_FULL + 2;
+  static constexpr int P_FULL = S_EMPTY + 2;      // [NP] per P buffer
+  static constexpr int O_FULL = P_FULL + C::NP;   // [NP] per P buffer: PV of tiles n with n % NP == b
+  static constexpr int O_EMPTY = O_FULL + C::NP;  // [2] per O buffer: its epilogue is done
+  static constexpr int O_DONE = O_EMPTY + 2;      // [2] per O buffer: the item's last PV is done
+  static constexpr int EP_FULL = O_DONE + 2;      // [2] per O buffer: the softmax warps handed the item over
+  static constexpr int MMA_DONE = EP_FULL + 2;    // the two MMA issuers, at the end
+  static constexpr int IT_FULL = MMA_DONE + 1, IT_EMPTY = IT_FULL + C::RING;
+  static constexpr int EGRP = IT_EMPTY + C::RING; // the epilogue warps
+  static constexpr int RED = EGRP + 1;            // [2] per softmax group: its four warps, once per item (first-tile maxima)
+  static constexpr int FIN = RED + 2;             // every warp, once: its last access to TMEM is done
+  static constexpr int CLAIM = FIN + 1;           // the K producer, once per item, a few tiles before the item's end
+  static_assert(CLAIM + 1 <= C::N_BAR, "barrier count");
+  __device__ __forceinline__ uint32_t k_full(int i) const { return at(K_FULL + i); }
+  __device__ __forceinline__ uint32_t k_empty(int i) const { return at(K_EMPTY + i); }
+  __device__ __forceinline__ uint32_t v_full(int i) const { return at(V_FULL + i); }
+  __device__ __forceinline__ uint32_t v_empty(int i) const { return at(V_EMPTY + i); }
+  __device__ __forceinline__ uint32_t q_full(int i) const { return at(Q_FULL + i); }
+  __device__ __forceinline__ uint32_t q_empty(int i) const { return at(Q_EMPTY + i); }
+  __device__ __forceinline__ uint32_t s_full(int i) const { return at(S_FULL + i); }
+  __device__ __forceinline__ uint32_t s_empty(int i) const { return at(S_EMPTY + i); }
+  __device__ __forceinline__ uint32_t p_full(int i) const { return at(P_FULL + i); }
+  __device__ __forceinline__ uint32_t o_full(int i) const { return at(O_FULL + i); }
+  __device__ __forceinline__ uint32_t o_empty(int i) const { return at(O_EMPTY + i); }
+  __device__ __forceinline__ uint32_t o_done(int i) const { return at(O_DONE + i); }
+  __device__ __forceinline__ uint32_t ep_full(int i) const { return at(EP_FULL + i); }
+  __device__ __forceinline__ uint32_t it_full(int i) const { return at(IT_FULL + i); }
+  __device__ __forceinline__ uint32_t it_empty(int i) const { return at(IT_EMPTY + i); }
+  __device__ __forceinline__ uint32_t red(int i) const { return at(RED + i); }
+  __device__ __forceinline__ uint32_t mma_done() const { return at(MMA_DONE); }
+  __device__ __forceinline__ uint32_t egrp() const { return at(EGRP); }
+  __device__ __forceinline__ uint32_t fin() const { return at(FIN); }
+  __device__ __forceinline__ uint32_t claim() const { return at(CLAIM); }
 };
 
-__device__ __forceinline__ bool wait_bar(uint64_t *b, uint32_t parity, volatile int *abort) {
+__device__ __forceinline__ bool wait_bar(uint32_t b, uint32_t parity, volatile int *abort) {
   if (ptx::mbar_try_wait(b, parity)) return true;
   const long long t0 = clock64();
   while (true) {
@@ -124,10 +165,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// Transposing reductions over the 32 lanes of a warp (v is consumed): on return lane i holds the
-// sum (max) over all lanes of v[i].  31 shuffles for 32 values.
-template <bool MAX>
-__device__ __forceinline__ float warp_transpose_reduce(float (&v)[32], int lane) {
+// Transposing sum over the 32 lanes of a warp (v is consumed): on return lane i holds the sum over all
+// lanes of v[i].  31 shuffles for 32 values.
+__device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
 #pragma unroll
   for (int w = 16; w >= 1; w >>= 1) {
     const bool up = (lane & w) != 0;
@@ -135,11 +175,118 @@ __device__ __forceinline__ float warp_transpose_reduce(float (&v)[32], int lane)
     for (int i = 0; i < w; ++i) {
       const float keep = up ? v[i + w] : v[i];
       const float send = up ? v[i] : v[i + w];
-      const float got = __shfl_xor_sync(0xffffffffu, send, w);
-      v[i] = MAX ? fmaxf(keep, got) : keep + got;
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
     }
   }
   return v[0];
+}
+
+// CPL (2 or 4) consecutive floats of a partial, and as many outputs scaled by inv and rounded to bf16.
+template <int CPL>
+__device__ __forceinline__ void ld_cols(const float *src, float (&v)[CPL]) {
+  if (CPL == 4) {
+    const float4 t = __ldcg(reinterpret_cast<const float4 *>(src));
+    v[0] = t.x;
+    v[1] = t.y;
+    v[CPL - 2] = t.z;
+    v[CPL - 1] = t.w;
+  } else {
+    const float2 t = __ldcg(reinterpret_cast<const float2 *>(src));
+    v[0] = t.x;
+    v[1] = t.y;
+  }
+}
+template <int CPL>
+__device__ __forceinline__ void st_cols(uint16_t *dst, const float (&v)[CPL], float inv) {
+  if (CPL == 4)
+    *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[CPL - 2] * inv, v[CPL - 1] * inv));
+  else
+    *reinterpret_cast<uint32_t *>(dst) = pack_bf16(v[0] * inv, v[1] * inv);
+}
+
+__device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b) {  // NaN never wins
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+
+// The whole item again, by the four epilogue warps on the CUDA cores with a running row maximum: the
+// way out for an item whose scores grow past kMaxP times its first tile's maximum (no input of an
+// ordinary model does; one such item takes about a millisecond).  Same output or partials as the main
+// path; a key whose block id is invalid reads as zero, as in the TMA loads.  s_p: kBT + 4 floats.
+// `bar`, `ph`: the epilogue warps' barrier and its phase count; returns the new count, or -1 if a wait
+// gave up.
+template <int D>
+__device__ __noinline__ int item_exact(const AttnParams &p, int it, float *s_p, uint32_t bar, int ph,
+                                       volatile int *abort) {
+  const WorkItem w = p.items[it];
+  const int g = p.Hq / p.Hkv;
+  auto sync = [&]() -> bool {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
+    return wait_bar(bar, (ph++) & 1, abort);
+  };
+  const int tid = threadIdx.x & 127, lane = tid & 31, wq = tid >> 5;
+  float *s_w = s_p + kBT;
+  const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
+  const uint16_t *kc = static_cast<const uint16_t *>(p.k_cache), *vc = static_cast<const uint16_t *>(p.v_cache);
+  const int32_t *bt = p.block_tables + (int64_t)w.r * p.max_blocks_per_seq;
+  auto key_at = [&](int t) -> int64_t {
+    const int32_t b = __ldg(bt + t / 16);
+    return b < 0 || b >= p.num_blocks ? -1 : (((int64_t)b * p.Hkv + w.h) * 16 + t % 16) * D;
+  };
+  for (int jr = 0; jr < w.rows; ++jr) {
+    const int rj = w.row0 + jr, jq = rj / g, hh = rj % g;
+    const int64_t o_at = ((int64_t)(w.q0 + jq) * p.Hq + w.h * g + hh) * D;
+    const uint16_t *qr = static_cast<const uint16_t *>(p.q) + o_at;
+    const int end = min(w.t1, w.ctx + jq + 1);
+    float m = -INFINITY, l = 0.0f, acc = 0.0f;
+    for (int t0 = w.t0; t0 < end; t0 += kBT) {
+      float s = -INFINITY;
+      if (t0 + tid < end) {
+        const int64_t at = key_at(t0 + tid);
+        float a = 0.0f;
+        if (at >= 0)
+          for (int d = 0; d < D; ++d) a = fmaf(bf16_bits_to_float(__ldg(qr + d)), bf16_bits_to_float(__ldg(kc + at + d)), a);
+        s = a * scale_log2;
+      }
+      float mx = s;
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      if (lane == 0) s_w[wq] = mx;
+      if (!sync()) return -1;
+      mx = fmaxf(m, fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3])));
+      const float f = m == mx ? 1.0f : ptx::ex2(m - mx);
+      const float e = t0 + tid < end ? ptx::ex2(s - mx) : 0.0f;
+      m = mx;
+      l = fmaf(l, f, e);
+      s_p[tid] = e;
+      if (!sync()) return -1;
+      acc *= f;
+      if (tid < D) {
+        for (int i = 0; i < kBT && t0 + i < end; ++i) {
+          const int64_t at = key_at(t0 + i);
+          if (at >= 0) acc = fmaf(s_p[i], bf16_bits_to_float(__ldg(vc + at + tid)), acc);
+        }
+      }
+      if (!sync()) return -1;
+    }
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) s_w[wq] = l;
+    if (!sync()) return -1;
+    l = s_w[0] + s_w[1] + s_w[2] + s_w[3];
+    if (!sync()) return -1;
+    if (tid < D) {
+      if (w.poff < 0)
+        static_cast<uint16_t *>(p.out)[o_at + tid] = __bfloat16_as_ushort(__float2bfloat16_rn(acc / l));
+      else
+        __stcg(p.partials + w.poff + (int64_t)jr * D + tid, acc);
+    }
+    if (w.poff >= 0 && tid == 0) {
+      __stcg(p.partials + w.poff + w.rows * D + jr, m);
+      __stcg(p.partials + w.poff + w.rows * D + w.rows + jr, l);
+    }
+  }
+  return ph;
 }
 
 }  // namespace
@@ -151,42 +298,19 @@ __global__ void __launch_bounds__(kThreads, 1)
                    const __grid_constant__ CUtensorMap tmv8) {
   using C = Cfg<D>;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  // aligned by an offset, not through an integer: the compiler then still knows the address space
+  uint8_t *smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   const uint32_t sbase = ptx::smem_u32(smem);
-  uint64_t *bar = reinterpret_cast<uint64_t *>(smem + C::OFF_BAR);
-  Bars B;
-  B.k_full = bar;
-  B.k_empty = B.k_full + C::NSK;
-  B.v_full = B.k_empty + C::NSK;
-  B.v_empty = B.v_full + C::NSV;
-  B.q_full = B.v_empty + C::NSV;
-  B.q_empty = B.q_full + 2;
-  B.s_full = B.q_empty + 2;
-  B.s_empty = B.s_full + 2;
-  B.p_full = B.s_empty + 2;     // [NP] per P buffer
-  B.o_full = B.p_full + C::NP;  // [NP] per P buffer: PV of tiles n with n % NP == b
-  B.o_empty = B.o_full + C::NP; // [2] per O buffer: its epilogue is done
-  B.o_done = B.o_empty + 2;     // [2] per O buffer: the item's last PV is done
-  B.ep_full = B.o_done + 2;     // [2] per O buffer: the softmax warps handed the item over
-  B.mma_done = B.ep_full + 2;
-  B.it_full = B.mma_done + 1;
-  B.it_empty = B.it_full + C::RING;
-  B.egrp = B.it_empty + C::RING;
-  B.sm_sync = B.egrp + 1;       // the softmax warps, once per tile
-  B.sm_sync2 = B.sm_sync + 1;   // the softmax warps, once per tile that moves a reference max
-  B.fin = B.sm_sync2 + 1;       // every warp, once: its last access to TMEM is done
-  B.claim = B.fin + 1;          // the K producer, once per item, a few tiles before the item's end
-  static_assert(2 * C::NSK + 2 * C::NSV + 8 + 2 * C::NP + 6 + 1 + 2 * C::RING + 5 <= C::N_BAR, "barrier count");
+  const Bars<D> B{sbase + C::OFF_BAR};
   float *s_mw = reinterpret_cast<float *>(smem + C::OFF_MW);
-  float *s_fw = reinterpret_cast<float *>(smem + C::OFF_FW);
   float *s_red = reinterpret_cast<float *>(smem + C::OFF_RED);
-  volatile uint32_t *s_flag = reinterpret_cast<volatile uint32_t *>(smem + C::OFF_FLAG);
-  float *s_em = reinterpret_cast<float *>(smem + C::OFF_EM);
+  float *s_ex = reinterpret_cast<float *>(smem + C::OFF_EX);
   float *s_hl = reinterpret_cast<float *>(smem + C::OFF_HL);
   float *s_hm = reinterpret_cast<float *>(smem + C::OFF_HM);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + C::OFF_MISC);
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 4);
   volatile int *s_last = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 8);
+  volatile int *s_ovf = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 16);  // [2] per O buffer: P past kMaxP
   struct RingSlot {
     int it;
     int pad[3];
@@ -198,39 +322,40 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::NSK; ++s) {
-      ptx::mbar_init(B.k_full + s, 1);
-      ptx::mbar_init(B.k_empty + s, 1);
+      ptx::mbar_init(B.k_full(s), 1);
+      ptx::mbar_init(B.k_empty(s), 1);
     }
     for (int s = 0; s < C::NSV; ++s) {
-      ptx::mbar_init(B.v_full + s, 1);
-      ptx::mbar_init(B.v_empty + s, 1);
+      ptx::mbar_init(B.v_full(s), 1);
+      ptx::mbar_init(B.v_empty(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      ptx::mbar_init(B.q_full + b, 1);
-      ptx::mbar_init(B.q_empty + b, 1);
-      ptx::mbar_init(B.s_full + b, 1);
-      ptx::mbar_init(B.s_empty + b, kSoftmaxWarps);
+      ptx::mbar_init(B.q_full(b), 1);
+      ptx::mbar_init(B.q_empty(b), 1);
+      ptx::mbar_init(B.s_full(b), 1);
+      ptx::mbar_init(B.s_empty(b), kSoftmaxWarps);
     }
     for (int b = 0; b < C::NP; ++b) {
-      ptx::mbar_init(B.p_full + b, kSoftmaxWarps);
-      ptx::mbar_init(B.o_full + b, 1);
+      ptx::mbar_init(B.p_full(b), kSoftmaxWarps);
+      ptx::mbar_init(B.o_full(b), 1);
     }
     for (int b = 0; b < 2; ++b) {
-      ptx::mbar_init(B.o_empty + b, 4);  // the four epilogue warps
-      ptx::mbar_init(B.o_done + b, 1);
-      ptx::mbar_init(B.ep_full + b, kSoftmaxWarps);
+      ptx::mbar_init(B.o_empty(b), 4);  // the four epilogue warps
+      ptx::mbar_init(B.o_done(b), 1);
+      ptx::mbar_init(B.ep_full(b), kSoftmaxWarps);
     }
-    ptx::mbar_init(B.mma_done, 1);
+    ptx::mbar_init(B.mma_done(), 2);  // the two MMA issuers
     for (int i = 0; i < C::RING; ++i) {
-      ptx::mbar_init(B.it_full + i, 1);
-      ptx::mbar_init(B.it_empty + i, 3 + kSoftmaxWarps + 4);  // KV producers, MMA, softmax and epilogue warps
+      ptx::mbar_init(B.it_full(i), 1);
+      ptx::mbar_init(B.it_empty(i), 4 + kSoftmaxWarps + 4);  // KV producers, MMA issuers, softmax and epilogue warps
     }
-    ptx::mbar_init(B.egrp, 4);      // the four epilogue warps
-    ptx::mbar_init(B.sm_sync, kSoftmaxWarps);
-    ptx::mbar_init(B.sm_sync2, kSoftmaxWarps);
-    ptx::mbar_init(B.fin, kThreads / 32);
-    ptx::mbar_init(B.claim, 1);
+    ptx::mbar_init(B.egrp(), 4);      // the four epilogue warps
+    ptx::mbar_init(B.red(0), 4);
+    ptx::mbar_init(B.red(1), 4);
+    ptx::mbar_init(B.fin(), kThreads / 32);
+    ptx::mbar_init(B.claim(), 1);
     *s_abort = 0;
+    s_ovf[0] = s_ovf[1] = 0;
     ptx::fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -260,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   const int g = p.Hq / p.Hkv;
 
-  if (warp == 0 || warp == 7) {
+  if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------------ K / V producers
     // K and V have rings of their own: a K stage is free again once S^T of its tile is done, a V
     // stage once PV is, so each tensor is fetched about as many tiles ahead of its use as its ring
@@ -270,17 +395,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const CUtensorMap *tm1 = is_k ? &tmk : &tmv;
     const CUtensorMap *tm8 = is_k ? &tmk8 : &tmv8;
     const uint32_t off_t = sbase + (is_k ? C::OFF_K : C::OFF_V);
-    uint64_t *full = is_k ? B.k_full : B.v_full;
-    uint64_t *empty = is_k ? B.k_empty : B.v_empty;
+    const uint32_t full = is_k ? B.k_full(0) : B.v_full(0), empty = is_k ? B.k_empty(0) : B.v_empty(0);
     uint32_t tile_n = 0;
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
       const int slot = j % C::RING;
-      if (!wait_bar(B.it_full + slot, (j / C::RING) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const WorkItem w = s_ring[slot].w;
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.it_empty + slot);
+      if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
       const int32_t *bt = p.block_tables + (int64_t)w.r * p.max_blocks_per_seq + w.t0 / 16;
       const int nblk = (w.t1 - w.t0 + 15) / 16;
@@ -294,15 +418,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int t = 0; t < ntiles; ++t, ++tile_n) {
         // a few tiles before this item's end the loader may take the next one (items are taken
         // just in time, so the work counter balances the CTAs to the end)
-        if (is_k && t == t_claim && lane == 0) ptx::mbar_arrive(B.claim);
+        if (is_k && t == t_claim && lane == 0) ptx::mbar_arrive(B.claim());
         if (t > 0 && (t & 3) == 0) {
           cur = nxt;
           nxt = fetch(32 * ((t >> 2) + 1));
         }
         const int s = (int)(tile_n % ns);
         const uint32_t round = tile_n / ns;
-        if (!wait_bar(empty + s, (round & 1) ^ 1, s_abort)) { ok = false; break; }
-        if (lane == 0) ptx::mbar_arrive_expect_tx(full + s, C::KV_TILE);
+        if (!wait_bar(empty + 8 * s, (round & 1) ^ 1, s_abort)) { ok = false; break; }
+        if (lane == 0) ptx::mbar_arrive_expect_tx(full + 8 * s, C::KV_TILE);
         __syncwarp();
         const int bi = lane & 7;  // block of the tile this lane looks after
         int bid = __shfl_sync(0xffffffffu, cur, (8 * t + bi) & 31);
@@ -316,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (lane == 0) {
 #pragma unroll
             for (int hf = 0; hf < C::HALVES; ++hf) {
-              ptx::tma_load_4d(off_t + s * C::KV_TILE + hf * C::HALF, tm8, full + s, hf * 64, 0, w.h, b0);
+              ptx::tma_load_4d(off_t + s * C::KV_TILE + hf * C::HALF, tm8, full + 8 * s, hf * 64, 0, w.h, b0);
             }
           }
         } else if (lane < 8) {
@@ -324,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int hf = 0; hf < C::HALVES; ++hf) {
             const uint32_t off = s * C::KV_TILE + hf * C::HALF + lane * (16 * 128);
-            ptx::tma_load_4d(off_t + off, tm1, full + s, hf * 64, 0, w.h, bid);
+            ptx::tma_load_4d(off_t + off, tm1, full + 8 * s, hf * 64, 0, w.h, bid);
           }
         }
       }
@@ -335,11 +459,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (uint32_t k = 0; k < ns && k < tile_n; ++k) {
         const uint32_t n = tile_n - 1 - k;
         const long long t0 = clock64();
-        while (!ptx::mbar_try_wait(full + n % ns, (n / ns) & 1) && clock64() - t0 < kWaitCycles) {
+        while (!ptx::mbar_try_wait(full + 8 * (n % ns), (n / ns) & 1) && clock64() - t0 < kWaitCycles) {
         }
       }
     }
-  } else if (warp == 6) {
+  } else if (warp == 2) {
     // ------------------------------------------------------------------ item loader
     int li = 0;
     bool ok = true;
@@ -349,8 +473,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       // per item, and the producer cannot pass item j - 1 before item j is published: the parity
       // is exact).
       const int slot = j % C::RING;
-      if (j > 0 && !wait_bar(B.claim, (j - 1) & 1, s_abort)) { ok = false; break; }
-      if (!wait_bar(B.it_empty + slot, ((j / C::RING) & 1) ^ 1, s_abort)) { ok = false; break; }
+      if (j > 0 && !wait_bar(B.claim(), (j - 1) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.it_empty(slot), ((j / C::RING) & 1) ^ 1, s_abort)) { ok = false; break; }
       int it = -1;
       if (lane == 0) {
         while (true) {
@@ -361,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         s_ring[slot].it = it;
         if (it >= 0) s_ring[slot].w = p.items[it];
-        ptx::mbar_arrive(B.it_full + slot);
+        ptx::mbar_arrive(B.it_full(slot));
       }
       it = __shfl_sync(0xffffffffu, it, 0);
       if (it < 0) {
@@ -372,7 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const WorkItem w = p.items[it];
       const int qb = li % C::NQ;
-      if (!wait_bar(B.q_empty + qb, ((li / C::NQ) & 1) ^ 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.q_empty(qb), ((li / C::NQ) & 1) ^ 1, s_abort)) { ok = false; break; }
       ++li;
       // the item's query rows -> Q[qb], row rho (query row row0 + rho = j*g + hh) at MMA row rho.
       // Loads are issued QBATCH at a time per lane before any store.  Rows past `rows` up to the
@@ -405,120 +529,91 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       ptx::fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.q_full + qb);
+      if (lane == 0) ptx::mbar_arrive(B.q_full(qb));
     }
     if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    // One thread polls two queues: S^T(n) is issued as soon as tile n's K has landed, its Q is
-    // loaded and its TMEM buffer has been read; PV(m) as soon as P(m) is published and V(m) has
-    // landed (and, for an item's first tile, the previous item's O has been read).  S^T therefore
-    // runs ahead of PV instead of waiting behind it.
-    if (lane == 0) {
-      uint32_t n_s = 0, n_pv = 0, j = 0;
-      int li = 0, s_t = 0, s_nt = 0, s_qb = 0, s_li = 0;
-      uint32_t s_idesc = 0, s_pvdesc = 0;
-      bool s_have = false, items_done = false, ok = true;
-      uint8_t tflag[4];     // per issued S^T tile: bit 0 first tile of its item, bit 1 its last
-      int tli[4];           // item number of the tile (O buffer, o_empty parity)
-      uint32_t tpv[4];      // instruction descriptor of the tile's PV product
-      long long last = clock64();
-      while (true) {
-        bool prog = false;
-        if (!s_have && !items_done) {
-          const int slot = j % C::RING;
-          if (ptx::mbar_test_wait(B.it_full + slot, (j / C::RING) & 1)) {
-            const int it = s_ring[slot].it;
-            const WorkItem w = s_ring[slot].w;
-            ptx::mbar_arrive(B.it_empty + slot);
-            ++j;
-            if (it < 0) {
-              items_done = true;
-            } else {
-              const int nrow = (w.rows + 15) / 16 * 16;  // the MMA's N: rows rounded up to 16
-              s_idesc = ptx::idesc_bf16_f32(kBT, nrow, false, false);
-              s_pvdesc = ptx::idesc_bf16_f32(128, nrow, true, true);
-              s_have = true;
-              s_t = 0;
-              s_nt = (w.t1 - w.t0 + kBT - 1) / kBT;
-              s_qb = li % C::NQ;
-              s_li = li;
-              ++li;
-            }
-            prog = true;
-          }
-        }
-        if (s_have && n_s < n_pv + 4) {
-          const int st = (int)(n_s % C::NSK), sb = n_s & 1;
-          if ((s_t > 0 || ptx::mbar_test_wait(B.q_full + s_qb, (s_li / C::NQ) & 1)) &&
-              ptx::mbar_test_wait(B.k_full + st, (n_s / C::NSK) & 1) &&
-              ptx::mbar_test_wait(B.s_empty + sb, ((n_s >> 1) & 1) ^ 1)) {
-            ptx::tc_fence_after();
-            const uint32_t qa = sbase + C::OFF_Q + s_qb * C::Q_BYTES;
-            const uint32_t ka = sbase + C::OFF_K + st * C::KV_TILE;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-              const uint32_t koff = (ks >> 2) * C::HALF + (ks & 3) * 32;
-              const uint32_t qoff = (ks >> 2) * C::QHALF + (ks & 3) * 32;
-              ptx::umma_f16(tmem + sb * kNR, ptx::sdesc_sw128(ka + koff, 16, 1024),
-                            ptx::sdesc_sw128(qa + qoff, 16, 1024), s_idesc, ks > 0);
-            }
-            ptx::umma_commit(B.s_full + sb);
-            ptx::umma_commit(B.k_empty + st);
-            if (s_t == s_nt - 1) ptx::umma_commit(B.q_empty + s_qb);
-            tflag[n_s & 3] = (s_t == 0 ? 1 : 0) | (s_t == s_nt - 1 ? 2 : 0);
-            tli[n_s & 3] = s_li;
-            tpv[n_s & 3] = s_pvdesc;
-            ++n_s;
-            if (++s_t == s_nt) s_have = false;
-            prog = true;
-          }
-        }
-        if (n_pv < n_s) {
-          const int pb = (int)(n_pv % C::NP);
-          const bool first = tflag[n_pv & 3] & 1, last = tflag[n_pv & 3] & 2;
-          const int tl = tli[n_pv & 3], ob = tl & 1;  // the item's O buffer
-          const int st = (int)(n_pv % C::NSV);
-          if (ptx::mbar_test_wait(B.p_full + pb, (n_pv / C::NP) & 1) &&
-              ptx::mbar_test_wait(B.v_full + st, (n_pv / C::NSV) & 1) &&
-              (!first || ptx::mbar_test_wait(B.o_empty + ob, ((tl >> 1) & 1) ^ 1))) {
-            ptx::tc_fence_after();
-            const uint32_t pa = sbase + C::OFF_P + pb * C::P_BYTES;
-            const uint32_t va = sbase + C::OFF_V + st * C::KV_TILE;
-            // A = V^T, MN-major: the head dim's 64-wide halves are HALF apart (for D = 64 both MMA
-            // halves read the same half, so O^T lanes 64..127 repeat lanes 0..63 and are not used)
-            constexpr uint32_t lbo_v = D == 128 ? C::HALF : 0;
-#pragma unroll
-            for (int ks = 0; ks < kBT / 16; ++ks) {
-              const uint64_t a = ptx::sdesc_sw128(va + ks * 16 * 128, lbo_v, 1024);
-              const uint64_t b = ptx::sdesc_sw128(pa + ks * 16 * 128, C::P_BYTES, 1024);
-              ptx::umma_f16(tmem + 128 + ob * kNR, a, b, tpv[n_pv & 3], (!first || ks > 0) ? 1u : 0u);
-            }
-            ptx::umma_commit(B.o_full + pb);
-            ptx::umma_commit(B.v_empty + st);
-            if (last) ptx::umma_commit(B.o_done + ob);
-            ++n_pv;
-            prog = true;
-          }
-        }
-        if (items_done && !s_have && n_pv == n_s) break;
-        if (prog) {
-          last = clock64();
-        } else {
-          if (*s_abort) { ok = false; break; }
-          if (clock64() - last > kWaitCycles) {
-            *s_abort = 1;
+  } else if (warp == 1 || warp == 16) {
+    // ------------------------------------------------------------------ MMA issuers
+    // One warp issues S^T, another PV, so that neither waits behind the other's barriers: one thread
+    // for both took 2400-2900 cycles a tile (about 45-90 per MMA, 100 per commit, and the polling of
+    // both queues), which bounded every item whatever its rows; the two run side by side.
+    const bool is_s = warp == 1;
+    uint32_t n = 0;
+    int li = 0;
+    bool ok = true;
+    for (uint32_t j = 0; ok; ++j, ++li) {
+      const int slot = j % C::RING;
+      if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
+      const int it = s_ring[slot].it;
+      const int rows = s_ring[slot].w.rows, ntok = s_ring[slot].w.t1 - s_ring[slot].w.t0;
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
+      if (it < 0) break;
+      const int nt = (ntok + kBT - 1) / kBT;
+      const int nrow = (rows + 15) / 16 * 16;  // the MMA's N: rows rounded up to 16
+      if (is_s) {
+        // S^T(n): K(n) has landed, the item's Q is loaded, the TMEM tile has been read
+        const uint32_t idesc = ptx::idesc_bf16_f32(kBT, nrow, false, false);
+        const int qb = li % C::NQ;
+        if (!wait_bar(B.q_full(qb), (li / C::NQ) & 1, s_abort)) { ok = false; break; }
+        const uint64_t qd = ptx::sdesc_sw128(sbase + C::OFF_Q + qb * C::Q_BYTES, 16, 1024);
+        for (int t = 0; t < nt; ++t, ++n) {
+          const int st = (int)(n % C::NSK), sb = n & 1;
+          if (!wait_bar(B.k_full(st), (n / C::NSK) & 1, s_abort) ||
+              !wait_bar(B.s_empty(sb), ((n >> 1) & 1) ^ 1, s_abort)) {
             ok = false;
             break;
           }
-          __nanosleep(20);
+          if (lane == 0) {
+            ptx::tc_fence_after();
+            const uint64_t kd = ptx::sdesc_sw128(sbase + C::OFF_K + st * C::KV_TILE, 16, 1024);
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks)  // descriptor addresses are in units of 16 bytes
+              ptx::umma_f16(tmem + sb * kNR, kd + (((ks >> 2) * C::HALF + (ks & 3) * 32) >> 4),
+                            qd + (((ks >> 2) * C::QHALF + (ks & 3) * 32) >> 4), idesc, ks > 0);
+            ptx::umma_commit(B.s_full(sb));
+            ptx::umma_commit(B.k_empty(st));
+            if (t == nt - 1) ptx::umma_commit(B.q_empty(qb));
+          }
+          __syncwarp();
+        }
+      } else {
+        // PV(n): P(n) is published, V(n) has landed and, for an item's first tile, the O buffer has
+        // been read.  A = V^T, MN-major: the head dim's 64-wide halves are HALF apart (for D = 64 both
+        // MMA halves read the same half, so O^T lanes 64..127 repeat lanes 0..63 and are not used)
+        const uint32_t idesc = ptx::idesc_bf16_f32(128, nrow, true, true);
+        const int ob = li & 1;  // the item's O buffer
+        constexpr uint32_t lbo_v = D == 128 ? C::HALF : 0;
+        for (int t = 0; t < nt; ++t, ++n) {
+          const int st = (int)(n % C::NSV), pb = (int)(n % C::NP);
+          if ((t == 0 && !wait_bar(B.o_empty(ob), ((li >> 1) & 1) ^ 1, s_abort)) ||
+              !wait_bar(B.v_full(st), (n / C::NSV) & 1, s_abort) ||
+              !wait_bar(B.p_full(pb), (n / C::NP) & 1, s_abort)) {
+            ok = false;
+            break;
+          }
+          if (lane == 0) {
+            ptx::tc_fence_after();
+            const uint64_t vd = ptx::sdesc_sw128(sbase + C::OFF_V + st * C::KV_TILE, lbo_v, 1024);
+            const uint64_t pd = ptx::sdesc_sw128(sbase + C::OFF_P + pb * C::P_BYTES, C::P_BYTES, 1024);
+#pragma unroll
+            for (int ks = 0; ks < kBT / 16; ++ks)
+              ptx::umma_f16(tmem + 128 + ob * kNR, vd + ((ks * 16 * 128) >> 4), pd + ((ks * 16 * 128) >> 4), idesc,
+                            (t > 0 || ks > 0) ? 1u : 0u);
+            ptx::umma_commit(B.o_full(pb));
+            ptx::umma_commit(B.v_empty(st));
+            if (t == nt - 1) ptx::umma_commit(B.o_done(ob));
+          }
+          __syncwarp();
         }
       }
+    }
+    if (lane == 0) {
       if (!ok) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
-      // every MMA this thread issued must finish before the TMEM is released
-      ptx::umma_commit(B.mma_done);
+      // every MMA the issuers issued must finish before the TMEM is released
+      ptx::umma_commit(B.mma_done());
       const long long t0 = clock64();
-      while (!ptx::mbar_try_wait(B.mma_done, 0) && clock64() - t0 < kWaitCycles) {
+      while (!ptx::mbar_try_wait(B.mma_done(), 0) && clock64() - t0 < kWaitCycles) {
       }
     }
   } else if (warp >= 8 && warp < 12) {
@@ -538,26 +633,33 @@ __global__ void __launch_bounds__(kThreads, 1)
     // barrier of the four epilogue warps (an mbarrier, so that the wait is bounded)
     auto group_sync = [&]() -> bool {
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.egrp);
-      return wait_bar(B.egrp, (gph++) & 1, s_abort);
+      if (lane == 0) ptx::mbar_arrive(B.egrp());
+      return wait_bar(B.egrp(), (gph++) & 1, s_abort);
     };
     for (uint32_t j = 0; ok; ++j) {
       const int slot = j % C::RING;
-      if (!wait_bar(B.it_full + slot, (j / C::RING) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const WorkItem w = s_ring[slot].w;
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.it_empty + slot);
+      if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
       const int ob = li & 1;
       const uint32_t o_col = 128 + ob * kNR;
       // the softmax warps' hand-over and the item's last PV
-      if (!wait_bar(B.ep_full + ob, (li >> 1) & 1, s_abort)) { ok = false; break; }
-      if (!wait_bar(B.o_done + ob, (li >> 1) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.ep_full(ob), (li >> 1) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.o_done(ob), (li >> 1) & 1, s_abort)) { ok = false; break; }
       ++li;
       ptx::tc_fence_after();
       const int nc = (w.rows + 31) / 32;
-      for (int c = 0; c < nc; ++c) {
+      const bool ovf = s_ovf[ob] != 0;
+      if (ovf) {  // (uniform over the four warps: set before the hand-over, cleared below)
+        const int ph = item_exact<D>(p, it, s_ex, B.egrp(), (int)(gph & 1), s_abort);
+        if (ph < 0) { ok = false; break; }
+        gph = (uint32_t)ph;
+        if (warp == 8 && lane == 0) s_ovf[ob] = 0;
+      }
+      for (int c = 0; c < nc && !ovf; ++c) {
         uint32_t x[32];  // O^T[d][rows 32c..]
         ptx::tmem_ld32(tmem + lane_addr + o_col + 32 * c, x);
         ptx::tmem_wait_ld();
@@ -593,7 +695,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.o_empty + ob);
+      if (lane == 0) ptx::mbar_arrive(B.o_empty(ob));
 
       // ---- split item: the last chunk of this (request, head, row group) to finish merges all ----
       if (w.poff >= 0) {
@@ -608,262 +710,227 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!group_sync()) { ok = false; break; }
         const int chunks = *s_last;
         if (chunks > 0) {
+          // The chunks' partials of this (head, row group) lie a fixed stride apart.  A warp takes two
+          // rows at a time: a lane holds one chunk's (m, l) of each, the warp reduces the rows' maximum
+          // and denominator, and then every lane adds its columns of the chunks' O with the chunk's
+          // weight broadcast by a shuffle, four chunks of both rows in flight.  (With one thread per
+          // row walking the chunks' (m, l), this merge took about 90 us of a request's 114 us at 16
+          // chunks: serial chains of L2 loads.)
           const WorkItem *ci = p.items + p.req_item_begin[w.r] + (w.h * w.nrg + w.rg) * chunks;
-          // thread jr < rows: row jr's overall max and 1 / sum over the chunks
-          if (d < w.rows) {
-            float mstar = -INFINITY;
-            for (int c = 0; c < chunks; ++c) mstar = fmaxf(mstar, __ldcg(p.partials + ci[c].poff + w.rows * D + d));
-            float den = 0.0f;
-            for (int c = 0; c < chunks; ++c) {
-              const float *part = p.partials + ci[c].poff;
-              const float mc = __ldcg(part + w.rows * D + d);
-              if (mc != -INFINITY) den = fmaf(__ldcg(part + w.rows * D + w.rows + d), ptx::ex2(mc - mstar), den);
+          const float *base = p.partials + ci[0].poff;
+          const int64_t stride = ci[1].poff - ci[0].poff;
+          constexpr int CPL = D / 32;  // columns per lane
+          uint16_t *og = static_cast<uint16_t *>(p.out);
+          for (int j0 = 2 * qd; j0 < w.rows; j0 += 8) {
+            const int j1 = min(j0 + 1, w.rows - 1);  // an odd last row is merged twice, alike
+            float m0 = -INFINITY, m1 = -INFINITY;
+            for (int c = lane; c < chunks; c += 32) {
+              const float *pm = base + c * stride + w.rows * D;
+              m0 = fmaxf(m0, __ldcg(pm + j0));
+              m1 = fmaxf(m1, __ldcg(pm + j1));
             }
-            s_em[d] = mstar;
-            s_em[kNR + d] = 1.0f / den;
-          }
-          if (!group_sync()) { ok = false; break; }
-          // thread d: column d of every row, eight rows at a time (independent loads in flight)
-          if (dval) {
-            uint16_t *og = static_cast<uint16_t *>(p.out);
-            for (int j0 = 0; j0 < w.rows; j0 += 8) {
-              float acc[8];
 #pragma unroll
-              for (int q = 0; q < 8; ++q) acc[q] = 0.0f;
-#pragma unroll 4
-              for (int c = 0; c < chunks; ++c) {
-                const float *part = p.partials + ci[c].poff;
+            for (int o = 16; o > 0; o >>= 1) {
+              m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+              m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+            }
+            float den0 = 0.0f, den1 = 0.0f, a0[CPL], a1[CPL];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                  const int jr = j0 + q;
-                  if (jr < w.rows) {
-                    const float mc = __ldcg(part + w.rows * D + jr);
-                    const float ov = __ldcg(part + (int64_t)jr * D + d);
-                    if (mc != -INFINITY) acc[q] = fmaf(ov, ptx::ex2(mc - s_em[jr]), acc[q]);
+            for (int q = 0; q < CPL; ++q) a0[q] = a1[q] = 0.0f;
+            for (int c0 = 0; c0 < chunks; c0 += 32) {
+              float w0 = 0.0f, w1 = 0.0f;  // lane: chunk c0 + lane
+              if (c0 + lane < chunks) {
+                const float *pm = base + (c0 + lane) * stride + w.rows * D;
+                const float mc0 = __ldcg(pm + j0), mc1 = __ldcg(pm + j1);
+                w0 = mc0 == -INFINITY ? 0.0f : ptx::ex2(mc0 - m0);
+                w1 = mc1 == -INFINITY ? 0.0f : ptx::ex2(mc1 - m1);
+                den0 = fmaf(__ldcg(pm + w.rows + j0), w0, den0);
+                den1 = fmaf(__ldcg(pm + w.rows + j1), w1, den1);
+              }
+              const int nc8 = min(32, chunks - c0);
+#pragma unroll 1
+              for (int c = 0; c < nc8; c += 4) {
+                float v0[4][CPL], v1[4][CPL];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const float *po = base + (c0 + min(c + u, nc8 - 1)) * stride + lane * CPL;
+                  ld_cols<CPL>(po + (int64_t)j0 * D, v0[u]);
+                  ld_cols<CPL>(po + (int64_t)j1 * D, v1[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  // a chunk with weight zero (none of its keys visible to the row) adds nothing
+                  const float x0 = __shfl_sync(0xffffffffu, w0, (c + u) & 31);
+                  const float x1 = __shfl_sync(0xffffffffu, w1, (c + u) & 31);
+                  const bool in = c + u < nc8;
+#pragma unroll
+                  for (int q = 0; q < CPL; ++q) {
+                    if (in && x0 != 0.0f) a0[q] = fmaf(v0[u][q], x0, a0[q]);
+                    if (in && x1 != 0.0f) a1[q] = fmaf(v1[u][q], x1, a1[q]);
                   }
                 }
               }
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const int jr = j0 + q;
-                if (jr < w.rows) {
-                  const int rj = w.row0 + jr, jq = rj / g, hh = rj % g;
-                  og[((int64_t)(w.q0 + jq) * p.Hq + w.h * g + hh) * D + d] =
-                      __bfloat16_as_ushort(__float2bfloat16_rn(acc[q] * s_em[kNR + jr]));
-                }
-              }
             }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+              den0 += __shfl_xor_sync(0xffffffffu, den0, o);
+              den1 += __shfl_xor_sync(0xffffffffu, den1, o);
+            }
+            const float i0 = 1.0f / den0, i1 = 1.0f / den1;
+            const int rj0 = w.row0 + j0, rj1 = w.row0 + j1;
+            st_cols<CPL>(og + ((int64_t)(w.q0 + rj0 / g) * p.Hq + w.h * g + rj0 % g) * D + lane * CPL, a0, i0);
+            st_cols<CPL>(og + ((int64_t)(w.q0 + rj1 / g) * p.Hq + w.h * g + rj1 % g) * D + lane * CPL, a1, i1);
           }
-          // s_em is read above until every warp is past this point
-          if (!group_sync()) { ok = false; break; }
         }
       }
     }
     if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
-  } else {
+  } else if (warp < 16) {
     // ------------------------------------------------------------------ softmax warps
-    // Two groups of four: warps 2-5 take rows 0-31 of every item, warps 12-15 rows 32-63 (and only
-    // keep in step for items of at most 32 rows).  Within a group, one warp per TMEM lane quadrant,
-    // i.e. 32 keys of each tile: a thread holds one key's scores for the group's 32 rows.
+    // Two groups of four: warps 4-7 take the first half of an item's rows, warps 12-15 the second (the
+    // MMA's N is a multiple of 16, so both halves are whole 8-row units and both groups always have
+    // work).  Within a group, one warp per TMEM lane quadrant, i.e. 32 keys of each tile: a thread holds
+    // one key's scores for the group's rows.  The rows' reference maxima are those of the item's first
+    // tile (its four warps exchange them once per item): a key of the item that a row can see at all is
+    // preceded by one in the first tile, and later tiles then need no agreement between warps.  (A vote
+    // of the eight warps on every tile, with a second pass over tiles that moved a reference, took
+    // 700-1000 of about 2900 cycles a tile.)
     const int qd = warp & 3;                  // TMEM lane quadrant: keys 32*qd .. 32*qd + 31 of a tile
-    const int grp = warp >= 12 ? 1 : 0;       // row chunk: rows 32*grp .. 32*grp + 31
-    const int sw8 = grp * 4 + qd;             // index of this warp among the eight
+    const int grp = warp >= 12 ? 1 : 0;
     const uint32_t lane_addr = (uint32_t)(qd * 32) << 16;
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
-    float *mw = s_mw + sw8 * 32;              // this warp's copy of its rows' reference maxima
-    float *fw = s_fw + sw8 * 32;              // this warp's copy of its rows' rescale factors
-    const int r0 = 32 * grp;                  // first row of the chunk
-    uint32_t n = 0, nf = 0;                   // tiles so far; tiles that moved a reference max
+    const float2 scale2 = make_float2(scale_log2, scale_log2);
+    float *mw = s_mw + (grp * 4 + qd) * 32;   // minus the rows' references, this warp's copy
+    uint32_t n = 0;                           // tiles so far
     int li = 0;                               // items so far: item li accumulates into O buffer li & 1
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
       const int slot = j % C::RING;
-      if (!wait_bar(B.it_full + slot, (j / C::RING) & 1, s_abort)) { ok = false; break; }
+      if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
-      const WorkItem w = s_ring[slot].w;
+      const int t0 = s_ring[slot].w.t0, t1 = s_ring[slot].w.t1, rows = s_ring[slot].w.rows;
+      const int ctx = s_ring[slot].w.ctx, row0 = s_ring[slot].w.row0;
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.it_empty + slot);
+      if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
       const int ob = li & 1;
-      const uint32_t o_col = 128 + ob * kNR;
-      const int ntiles = (w.t1 - w.t0 + kBT - 1) / kBT;
-      // 8-row units of this chunk that the MMA reads (its N / 8 minus the chunk's offset)
-      const int nu = min(4, max(0, (w.rows + 15) / 16 * 2 - 4 * grp));
-      const bool active = nu > 0;
-      const int jmax = w.rows - r0;          // rows of the item in this chunk (may be <= 0)
-      mw[lane] = -INFINITY;
-      __syncwarp();
-      float lp[32];  // this thread's (key's) share of every row sum of the chunk
+      const int ntiles = (t1 - t0 + kBT - 1) / kBT;
+      const int nfull = (max(t0, min(t1, ctx + 1)) - t0) / kBT;  // tiles whose keys every row sees
+      const int half = (rows + 15) / 16 * 8;  // rows per group
+      const int nu = half / 8;                // its 8-row units, 1 to 4
+      const int r0 = grp * half;              // the group's first row
+      float2 lp[16];  // this thread's (key's) share of every row sum of the group
 #pragma unroll
-      for (int i = 0; i < 32; ++i) lp[i] = 0.0f;
+      for (int i = 0; i < 16; ++i) lp[i] = make_float2(0.0f, 0.0f);
+      uint32_t pmax = 0;        // largest P so far (two bf16 lanes)
+      float mref = -INFINITY;   // lane i: row r0 + i's reference (-inf: no key visible)
       for (int t = 0; t < ntiles && ok; ++t, ++n) {
         const int sb = n & 1;
-        if (!wait_bar(B.s_full + sb, (n >> 1) & 1, s_abort)) { ok = false; break; }
+        if (!wait_bar(B.s_full(sb), (n >> 1) & 1, s_abort)) { ok = false; break; }
         ptx::tc_fence_after();
-        const int pbuf = (int)(n % C::NP);
-        uint8_t *prow = smem + C::OFF_P + pbuf * C::P_BYTES + (qd * 32 + lane) * 128;
-        const int sw = lane & 7;
+        uint32_t x[2][16];
+        ptx::tmem_ld16(tmem + lane_addr + sb * kNR + r0, x[0]);
+        if (nu > 2) ptx::tmem_ld16(tmem + lane_addr + sb * kNR + r0 + 16, x[1]);
+        ptx::tmem_wait_ld();
+        // S^T(n) is in registers: its TMEM tile may be overwritten by S^T(n + 2)
+        ptx::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(B.s_empty(sb));
         // causal mask: key tok is visible to row jr iff tok <= ctx + (row0 + jr) / g, i.e.
-        // row0 + jr >= g * (tok - ctx); keys past the item and rows past `rows` are masked too
-        const int tok = w.t0 + t * kBT + qd * 32 + lane;
-        const int jmin = (tok >= w.t1 ? kNR : max(0, g * (tok - w.ctx) - w.row0)) - r0;
-        float emax = 0.0f;
-        if (active) {
-          // P buffer n % NP is free again once PV(n - NP) is done: the other group's wait or this
-          // warp's own one covered PV(n - 2NP), and PV(n) needs the P(n) about to be published,
-          // so the parity is exact
-          if (n >= (uint32_t)C::NP && !wait_bar(B.o_full + pbuf, ((n - C::NP) / C::NP) & 1, s_abort)) {
-            ok = false;
-            break;
-          }
-          // P = 2^(s - m) against the current reference maxima (masked: 0), written straight to the
-          // P buffer and added to the row-sum shares; the vote asks whether any P exceeds 2^kTau
-          // (then the tile is redone below with new references)
-          uint32_t x[32];
-          ptx::tmem_ld32(tmem + lane_addr + sb * kNR + r0, x);
-          ptx::tmem_wait_ld();
+        // row0 + jr >= g * (tok - ctx); keys past the item are masked too.  Only an item's last tiles
+        // (from nfull on) have such keys.
+        if (t >= nfull) {
+          const int tok = t0 + t * kBT + qd * 32 + lane;
+          const int jmin = tok >= t1 ? 32 : max(0, min(32, g * (tok - ctx) - row0 - r0));
+          const uint32_t seen = (uint32_t)(0xffffffffull << jmin);
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (!(seen & (1u << i))) x[i >> 4][i & 15] = 0xff800000u;
+        }
+        if (t == 0) {
+          // references: exact row maxima of the tile, over this warp's 32 keys, then over the group's
+          // four quadrants.  Padding rows get +inf (P = 0), rows without a visible key 0 (P = 0: all
+          // their scores are -inf).  s_red alternates between items: a warp that writes it for item
+          // li + 2 has passed the barrier of item li + 1, where every reader of item li has arrived.
+          float wm = -INFINITY;  // lane i: row r0 + i's maximum over this warp's keys
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             if (u < nu) {
-              uint32_t pk[4];
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int i0 = 8 * u + 4 * h;
-                const float4 m4 = reinterpret_cast<const float4 *>(mw + i0)[0];
-                const float mm[4] = {m4.x, m4.y, m4.z, m4.w};
-                float e[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                  const int jr = i0 + q;
-                  const float v = ptx::ex2(fmaf(__uint_as_float(x[i0 + q]), scale_log2, -mm[q]));
-                  e[q] = (jr >= jmin && jr < jmax) ? v : 0.0f;
-                  emax = fmaxf(emax, e[q]);
-                  lp[i0 + q] += e[q];
-                }
-                pk[2 * h] = pack_bf16(e[0], e[1]);
-                pk[2 * h + 1] = pack_bf16(e[2], e[3]);
+              for (int i = 8 * u; i < 8 * u + 8; ++i) {
+                const float rm = ptx::warp_max(__uint_as_float(x[i >> 4][i & 15]));
+                if (lane == i) wm = rm;
               }
-              *reinterpret_cast<uint4 *>(prow + (((4 * grp + u) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             }
           }
-        }
-        // the eight warps' votes, double-buffered by tile parity (NaN never wins fmaxf, and a
-        // visible key of a row without a reference yet gives +inf)
-        const uint32_t vote = __ballot_sync(0xffffffffu, !(emax <= kExpTau));
-        if (lane == 0) {
-          s_flag[(n & 1) * 8 + sw8] = vote;
-          ptx::mbar_arrive(B.sm_sync);
-        }
-        if (!wait_bar(B.sm_sync, n & 1, s_abort)) { ok = false; break; }
-        uint32_t anyv = 0;
-#pragma unroll
-        for (int k8 = 0; k8 < 8; ++k8) anyv |= s_flag[(n & 1) * 8 + k8];
-        if (anyv != 0) {
-          // new references: exact tile maxima per row (over this warp's 32 keys, then over the
-          // group's four quadrants), from the scores read again
-          if (active) {
-            uint32_t x[32];
-            ptx::tmem_ld32(tmem + lane_addr + sb * kNR + r0, x);
-            ptx::tmem_wait_ld();
-            float sv[32];
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              sv[i] = (i >= jmin && i < jmax) ? __uint_as_float(x[i]) * scale_log2 : -INFINITY;  // scale > 0
-            s_red[qd * kNR + r0 + lane] = warp_transpose_reduce<true>(sv, lane);
-          }
+          float *red = s_red + (li & 1) * 4 * kNR + r0 + lane;
+          if (lane < half) red[qd * kNR] = wm;
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(B.sm_sync2);
-          if (!wait_bar(B.sm_sync2, nf & 1, s_abort)) { ok = false; break; }
-          ++nf;
-          if (active) {
-            // this tile's P leaves the shares (a row without a reference had nothing yet)
-            {
-              uint32_t x[32];
-              ptx::tmem_ld32(tmem + lane_addr + sb * kNR + r0, x);
-              ptx::tmem_wait_ld();
+          if (lane == 0) ptx::mbar_arrive(B.red(grp));
+          if (!wait_bar(B.red(grp), li & 1, s_abort)) { ok = false; break; }
+          if (lane < half)
+            mref = fmaxf(fmaxf(red[0], red[kNR]), fmaxf(red[2 * kNR], red[3 * kNR])) * scale_log2;
+          mw[lane] = r0 + lane >= rows || lane >= half ? -INFINITY : mref == -INFINITY ? 0.0f : -mref;
+          __syncwarp();
+        }
+        // P buffer n % NP is free again once PV(n - NP) is done; PV(n) needs the P(n) about to be
+        // published, so the parity is exact
+        const int pbuf = (int)(n % C::NP);
+        if (n >= (uint32_t)C::NP && !wait_bar(B.o_full(pbuf), ((n - C::NP) / C::NP) & 1, s_abort)) {
+          ok = false;
+          break;
+        }
+        uint8_t *prow = smem + C::OFF_P + pbuf * C::P_BYTES + (qd * 32 + lane) * 128;
+        const int sw = lane & 7;
+        // P = 2^(s - m) (masked: 0), two rows at a time in packed fp32x2 arithmetic, written straight to
+        // the P buffer and added to the row-sum shares
 #pragma unroll
-              for (int i = 0; i < 32; ++i) {
-                const float mo = mw[i];
-                const float v = ptx::ex2(fmaf(__uint_as_float(x[i]), scale_log2, -mo));
-                const float eo = (i >= jmin && i < jmax) ? v : 0.0f;
-                lp[i] = mo == -INFINITY ? 0.0f : lp[i] - eo;
+        for (int u = 0; u < 4; ++u) {
+          if (u < nu) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const float4 m4 = reinterpret_cast<const float4 *>(mw + 8 * u + 4 * h)[0];
+#pragma unroll
+              for (int q = 0; q < 2; ++q) {
+                const int i = 8 * u + 4 * h + 2 * q;
+                const float2 s2 = make_float2(__uint_as_float(x[i >> 4][i & 15]), __uint_as_float(x[i >> 4][(i & 15) + 1]));
+                const float2 a = __ffma2_rn(s2, scale2, q == 0 ? make_float2(m4.x, m4.y) : make_float2(m4.z, m4.w));
+                const float2 e = make_float2(ptx::ex2(a.x), ptx::ex2(a.y));
+                lp[i >> 1] = __fadd2_rn(lp[i >> 1], e);
+                const uint32_t pe = pack_bf16(e.x, e.y);
+                pmax = bmax2(pmax, pe);
+                pk[2 * h + q] = pe;
               }
             }
-            __syncwarp();
-            // every warp of the group derives the same new maxima and factors from the same values
-            const int jl = r0 + lane;
-            const float tmax = fmaxf(fmaxf(s_red[jl], s_red[kNR + jl]), fmaxf(s_red[2 * kNR + jl], s_red[3 * kNR + jl]));
-            const float mo = mw[lane];
-            const float mn = tmax > mo + kTau ? tmax : mo;
-            fw[lane] = mn == mo ? 1.0f : (mo == -INFINITY ? 0.0f : ptx::ex2(mo - mn));
-            const bool moved = mn != mo && mo != -INFINITY;
-            mw[lane] = mn;
-            __syncwarp();
-            // P again against the new references: shares rescaled, P rewritten
-            {
-              uint32_t x[32];
-              ptx::tmem_ld32(tmem + lane_addr + sb * kNR + r0, x);
-              ptx::tmem_wait_ld();
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                uint32_t pk[4];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  float e[4];
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const int i = 8 * u + 4 * h + q;
-                    const float v = ptx::ex2(fmaf(__uint_as_float(x[i]), scale_log2, -mw[i]));
-                    e[q] = (i >= jmin && i < jmax) ? v : 0.0f;
-                    lp[i] = fmaf(lp[i], fw[i], e[q]);
-                  }
-                  pk[2 * h] = pack_bf16(e[0], e[1]);
-                  pk[2 * h + 1] = pack_bf16(e[2], e[3]);
-                }
-                if (u < nu)
-                  *reinterpret_cast<uint4 *>(prow + (((4 * grp + u) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-              }
-            }
-            // this chunk's O^T columns, if they hold earlier tiles of the item, move to the new
-            // references; the rescale needs PV(n-1) complete and precedes PV(n)
-            if (t > 0 && __any_sync(0xffffffffu, moved)) {
-              // PV(m) completes barrier o_full[m % NP] for the (m / NP)-th time; PV(n-1-NP) was
-              // waited for (by this warp or, through the tile votes, by the other group) and
-              // PV(n-1+NP) needs P(n-1+NP), so the parity names PV(n-1)
-              if (!wait_bar(B.o_full + (n - 1) % C::NP, ((n - 1) / C::NP) & 1, s_abort)) { ok = false; break; }
-              ptx::tc_fence_after();
-#pragma unroll
-              for (int c = 0; c < 2; ++c) {
-                uint32_t y[16];
-                ptx::tmem_ld16(tmem + lane_addr + o_col + r0 + 16 * c, y);
-                ptx::tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) y[i] = __float_as_uint(__uint_as_float(y[i]) * fw[16 * c + i]);
-                ptx::tmem_st16(tmem + lane_addr + o_col + r0 + 16 * c, y);
-              }
-              ptx::tmem_wait_st();
-            }
+            *reinterpret_cast<uint4 *>(prow + (((r0 / 8 + u) ^ sw) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
           }
         }
-        // S^T(n) has been read: its TMEM buffer may be overwritten by S^T(n+2); P(n) is published
-        ptx::tc_fence_before();
+        // P(n) is published
         ptx::fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) {
-          ptx::mbar_arrive(B.s_empty + sb);
-          ptx::mbar_arrive(B.p_full + pbuf);
-        }
+        if (lane == 0) ptx::mbar_arrive(B.p_full(pbuf));
       }
       if (!ok) break;
       // ---- hand the item over to the epilogue warps: this quadrant's share of each row sum of
-      // the chunk, and the reference maxima.  The epilogue of item li - 2 (same buffers) must be
+      // the group, and the references.  The epilogue of item li - 2 (same buffers) must be
       // done with them.
-      const float lsh = warp_transpose_reduce<false>(lp, lane);
-      if (!wait_bar(B.o_empty + ob, ((li >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
-      s_hl[(ob * 4 + qd) * kNR + r0 + lane] = lsh;
-      if (qd == 0) s_hm[ob * kNR + r0 + lane] = mw[lane];
+      float ls[32];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        ls[2 * i] = lp[i].x;
+        ls[2 * i + 1] = lp[i].y;
+      }
+      const float lsh = warp_transpose_sum(ls, lane);
+      const bool ovf = __any_sync(0xffffffffu, fmaxf(__uint_as_float(pmax << 16), __uint_as_float(pmax & 0xffff0000u)) > kMaxP);
+      if (!wait_bar(B.o_empty(ob), ((li >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
+      if (lane < half) {
+        s_hl[(ob * 4 + qd) * kNR + r0 + lane] = lsh;
+        if (qd == 0) s_hm[ob * kNR + r0 + lane] = mref;
+      }
+      if (ovf && lane == 0) s_ovf[ob] = 1;
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(B.ep_full + ob);
+      if (lane == 0) ptx::mbar_arrive(B.ep_full(ob));
       ++li;
     }
     if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
@@ -873,10 +940,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   // TMEM once all have (a bounded wait; the warps' shared memory stays until the last one exits).
   __syncwarp();
   ptx::tc_fence_before();
-  if (lane == 0) ptx::mbar_arrive(B.fin);
+  if (lane == 0) ptx::mbar_arrive(B.fin());
   if (warp == 1) {
     const long long t0 = clock64();
-    while (!ptx::mbar_try_wait(B.fin, 0) && clock64() - t0 < kWaitCycles) {
+    while (!ptx::mbar_try_wait(B.fin(), 0) && clock64() - t0 < kWaitCycles) {
     }
     __syncwarp();
     ptx::tc_fence_after();
