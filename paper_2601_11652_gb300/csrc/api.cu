@@ -70,7 +70,7 @@ wisp_status device_setup(int *dev_out, int *sms_out) {
   if (!d.attrs_done) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return WISP_ERR_CUDA;
-    cudaError_t e = attn_simt_setup();
+    cudaError_t e = attn_f32_setup();
     if (e == cudaSuccess) e = attn_tc_setup();
     if (e == cudaSuccess) e = accept_setup();
     if (e != cudaSuccess) return WISP_ERR_CUDA;
@@ -191,14 +191,14 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
   L.plan_header = take(sizeof(PlanHeader));
   if (a) {
     L.target_items = sms * kItemsPerSM;
-    // the tensor-core kernel takes at most kTcRowsPerItem query rows per item: a (request, head)
-    // with more is cut into two row groups, which at most doubles the item count
-    const int64_t rg = a->qkv_dtype == WISP_BF16 ? 2 : 1;
-    L.max_items = rg * ((int64_t)L.target_items + (int64_t)B * a->Hkv);
-    L.partial_cap = (int64_t)2 * L.target_items * kMaxRowsPerHead * (a->D + 2);
+    // the kernels take at most so many query rows per item: a (request, head) with more is cut into
+    // row groups of equal size, which multiplies the item count at most as often
+    L.row_groups = kMaxRowsPerHead / (a->qkv_dtype == WISP_BF16 ? kTcRowsPerItem : kF32RowsPerItem);
+    L.max_items = L.row_groups * ((int64_t)L.target_items + (int64_t)B * a->Hkv);
+    L.partial_cap = (int64_t)2 * L.target_items * (kMaxRowsPerHead * (a->D + 2) + 4 * L.row_groups);
     L.req_item_begin = take(sizeof(int32_t) * (size_t)B);
     L.req_chunks = take(sizeof(int32_t) * (size_t)B);
-    L.pair_done = take(sizeof(int32_t) * (size_t)B * a->Hkv * 2);
+    L.pair_done = take(sizeof(int32_t) * (size_t)B * a->Hkv * L.row_groups);
     L.items = take(sizeof(WorkItem) * (size_t)L.max_items);
     L.order = take(sizeof(int32_t) * (size_t)L.max_items);
     L.partials = take(sizeof(float) * (size_t)L.partial_cap);
@@ -260,7 +260,9 @@ PlanParams plan_params(const wisp_attn_args *a, const wisp_accept_args *c, void 
     pp.context_lens = a->context_lens;
     pp.with_attention = 1;
     pp.target_items = L.target_items;
-    pp.max_rows_item = a->qkv_dtype == WISP_BF16 ? kTcRowsPerItem : kMaxRowsPerHead;
+    pp.max_rows_item = a->qkv_dtype == WISP_BF16 ? kTcRowsPerItem : kF32RowsPerItem;
+    pp.row_groups = L.row_groups;
+    pp.kv_f32 = a->qkv_dtype == WISP_F32;
     pp.max_items = L.max_items;
     pp.partial_cap = L.partial_cap;
     pp.req_item_begin = at<int32_t>(ws, L.req_item_begin);
@@ -315,16 +317,12 @@ wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L,
   ap.order = at<int32_t>(ws, L.order);
   ap.partials = at<float>(ws, L.partials);
   ap.pair_done = at<int32_t>(ws, L.pair_done);
-  const bool bf = a->qkv_dtype == WISP_BF16;
-  if (bf) {
-    // persistent tensor-core kernel: one CTA per SM
-    const int grid = (int)(L.max_items < L.target_items / kItemsPerSM ? L.max_items : L.target_items / kItemsPerSM);
-    // the work counter lives in the plan header written by the planner on this stream
-    // split items are merged inside the kernel by the last chunk to finish
-    return attn_tc_launch(ap, grid, s, pdl) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
-  }
-  if (attn_simt_launch(ap, bf, (int)L.max_items, s) != cudaSuccess) return WISP_ERR_CUDA;
-  return attn_combine_launch(ap, bf, s) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
+  ap.row_groups = L.row_groups;
+  // persistent kernels, one CTA per SM: the work counter lives in the plan header written by the planner
+  // on this stream, and split items are merged inside the kernel by the last chunk to finish
+  const int grid = (int)(L.max_items < L.target_items / kItemsPerSM ? L.max_items : L.target_items / kItemsPerSM);
+  const cudaError_t e = a->qkv_dtype == WISP_BF16 ? attn_tc_launch(ap, grid, s, pdl) : attn_f32_launch(ap, grid, s, pdl);
+  return e == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
 }
 
 AcceptParams accept_params(const wisp_accept_args *c, void *ws, const Layout &L, int sms,

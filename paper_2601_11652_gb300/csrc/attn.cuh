@@ -18,13 +18,15 @@ struct AttnParams {
   const WorkItem *items;
   const int32_t *order;  // dispatch order of the persistent kernel: item index per counter value
   float *partials;
-  int32_t *pair_done;  // [B * Hkv] finished chunks of each split (request, head), zeroed by the planner
+  int row_groups;      // row groups per (request, head) at most
+  int32_t *pair_done;  // [B * Hkv * row_groups] finished chunks of each split (request, head, row group), zeroed
+                       // by the planner
 };
 
 // Host launchers (defined next to their kernels).
-cudaError_t attn_simt_setup();  // once per device: shared-memory attributes
-cudaError_t attn_simt_launch(const AttnParams &p, bool bf16, int grid, cudaStream_t s);
-cudaError_t attn_combine_launch(const AttnParams &p, bool bf16, cudaStream_t s);
+// CUDA-core kernel for fp32 KV, D in {64, 128}; `grid` persistent CTAs
+cudaError_t attn_f32_setup();  // once per device: shared-memory attributes
+cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s, bool pdl);
 // tcgen05 / TMA kernel for bf16 KV, D in {64, 128}; `grid` persistent CTAs
 cudaError_t attn_tc_setup();
 // pdl: programmatic dependent launch (the CTAs' set-up overlaps the previous kernel on `s`, which

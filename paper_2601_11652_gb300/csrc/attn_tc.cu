@@ -42,7 +42,7 @@
 // Every mbarrier wait is bounded in time; an expired wait records WISP_DEV_TIMEOUT and the CTA
 // drains.  No named barrier is used: a warp that gives up cannot leave the others blocked, and the
 // TMEM is freed once every warp has arrived on a final mbarrier.
-#include "attn.cuh"
+#include "attn_merge.cuh"
 #include "sm100_ptx.cuh"
 
 #include <cudaTypedefs.h>
@@ -157,12 +157,7 @@ __device__ __forceinline__ bool wait_bar(uint32_t b, uint32_t parity, volatile i
 
 __device__ __forceinline__ bool item_ok(const AttnParams &p, const WorkItem &w) {
   return w.r >= 0 && w.r < p.B && p.req_flag[w.r] == REQ_OK && w.t1 > w.t0 && w.rows > 0 && w.rows <= kNR &&
-         w.row0 >= 0 && (w.nrg == 1 || w.nrg == 2) && w.rg >= 0 && w.rg < w.nrg;
-}
-
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t *>(&v);
+         w.row0 >= 0 && w.nrg >= 1 && w.nrg <= p.row_groups && w.rg >= 0 && w.rg < w.nrg;
 }
 
 // Transposing sum over the 32 lanes of a warp (v is consumed): on return lane i holds the sum over all
@@ -179,29 +174,6 @@ __device__ __forceinline__ float warp_transpose_sum(float (&v)[32], int lane) {
     }
   }
   return v[0];
-}
-
-// CPL (2 or 4) consecutive floats of a partial, and as many outputs scaled by inv and rounded to bf16.
-template <int CPL>
-__device__ __forceinline__ void ld_cols(const float *src, float (&v)[CPL]) {
-  if (CPL == 4) {
-    const float4 t = __ldcg(reinterpret_cast<const float4 *>(src));
-    v[0] = t.x;
-    v[1] = t.y;
-    v[CPL - 2] = t.z;
-    v[CPL - 1] = t.w;
-  } else {
-    const float2 t = __ldcg(reinterpret_cast<const float2 *>(src));
-    v[0] = t.x;
-    v[1] = t.y;
-  }
-}
-template <int CPL>
-__device__ __forceinline__ void st_cols(uint16_t *dst, const float (&v)[CPL], float inv) {
-  if (CPL == 4)
-    *reinterpret_cast<uint2 *>(dst) = make_uint2(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[CPL - 2] * inv, v[CPL - 1] * inv));
-  else
-    *reinterpret_cast<uint32_t *>(dst) = pack_bf16(v[0] * inv, v[1] * inv);
 }
 
 __device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b) {  // NaN never wins
@@ -703,84 +675,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!group_sync()) { ok = false; break; }
         if (warp == 8 && lane == 0) {
           const int chunks = p.req_chunks[w.r];
-          const int done = atomicAdd(p.pair_done + ((int64_t)w.r * p.Hkv + w.h) * 2 + w.rg, 1);
+          const int done = atomicAdd(p.pair_done + ((int64_t)w.r * p.Hkv + w.h) * p.row_groups + w.rg, 1);
           *s_last = done == chunks - 1 ? chunks : 0;
           __threadfence();
         }
         if (!group_sync()) { ok = false; break; }
         const int chunks = *s_last;
         if (chunks > 0) {
-          // The chunks' partials of this (head, row group) lie a fixed stride apart.  A warp takes two
-          // rows at a time: a lane holds one chunk's (m, l) of each, the warp reduces the rows' maximum
-          // and denominator, and then every lane adds its columns of the chunks' O with the chunk's
-          // weight broadcast by a shuffle, four chunks of both rows in flight.  (With one thread per
-          // row walking the chunks' (m, l), this merge took about 90 us of a request's 114 us at 16
-          // chunks: serial chains of L2 loads.)
-          const WorkItem *ci = p.items + p.req_item_begin[w.r] + (w.h * w.nrg + w.rg) * chunks;
-          const float *base = p.partials + ci[0].poff;
-          const int64_t stride = ci[1].poff - ci[0].poff;
-          constexpr int CPL = D / 32;  // columns per lane
-          uint16_t *og = static_cast<uint16_t *>(p.out);
-          for (int j0 = 2 * qd; j0 < w.rows; j0 += 8) {
-            const int j1 = min(j0 + 1, w.rows - 1);  // an odd last row is merged twice, alike
-            float m0 = -INFINITY, m1 = -INFINITY;
-            for (int c = lane; c < chunks; c += 32) {
-              const float *pm = base + c * stride + w.rows * D;
-              m0 = fmaxf(m0, __ldcg(pm + j0));
-              m1 = fmaxf(m1, __ldcg(pm + j1));
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-              m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-            }
-            float den0 = 0.0f, den1 = 0.0f, a0[CPL], a1[CPL];
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) a0[q] = a1[q] = 0.0f;
-            for (int c0 = 0; c0 < chunks; c0 += 32) {
-              float w0 = 0.0f, w1 = 0.0f;  // lane: chunk c0 + lane
-              if (c0 + lane < chunks) {
-                const float *pm = base + (c0 + lane) * stride + w.rows * D;
-                const float mc0 = __ldcg(pm + j0), mc1 = __ldcg(pm + j1);
-                w0 = mc0 == -INFINITY ? 0.0f : ptx::ex2(mc0 - m0);
-                w1 = mc1 == -INFINITY ? 0.0f : ptx::ex2(mc1 - m1);
-                den0 = fmaf(__ldcg(pm + w.rows + j0), w0, den0);
-                den1 = fmaf(__ldcg(pm + w.rows + j1), w1, den1);
-              }
-              const int nc8 = min(32, chunks - c0);
-#pragma unroll 1
-              for (int c = 0; c < nc8; c += 4) {
-                float v0[4][CPL], v1[4][CPL];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  const float *po = base + (c0 + min(c + u, nc8 - 1)) * stride + lane * CPL;
-                  ld_cols<CPL>(po + (int64_t)j0 * D, v0[u]);
-                  ld_cols<CPL>(po + (int64_t)j1 * D, v1[u]);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                  // a chunk with weight zero (none of its keys visible to the row) adds nothing
-                  const float x0 = __shfl_sync(0xffffffffu, w0, (c + u) & 31);
-                  const float x1 = __shfl_sync(0xffffffffu, w1, (c + u) & 31);
-                  const bool in = c + u < nc8;
-#pragma unroll
-                  for (int q = 0; q < CPL; ++q) {
-                    if (in && x0 != 0.0f) a0[q] = fmaf(v0[u][q], x0, a0[q]);
-                    if (in && x1 != 0.0f) a1[q] = fmaf(v1[u][q], x1, a1[q]);
-                  }
-                }
-              }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              den0 += __shfl_xor_sync(0xffffffffu, den0, o);
-              den1 += __shfl_xor_sync(0xffffffffu, den1, o);
-            }
-            const float i0 = 1.0f / den0, i1 = 1.0f / den1;
-            const int rj0 = w.row0 + j0, rj1 = w.row0 + j1;
-            st_cols<CPL>(og + ((int64_t)(w.q0 + rj0 / g) * p.Hq + w.h * g + rj0 % g) * D + lane * CPL, a0, i0);
-            st_cols<CPL>(og + ((int64_t)(w.q0 + rj1 / g) * p.Hq + w.h * g + rj1 % g) * D + lane * CPL, a1, i1);
-          }
+          merge_chunks<D, uint16_t>(p, w, g, chunks, qd, 4);
         }
       }
     }

@@ -281,14 +281,13 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
       n = (int64_t)ctx_r + k_r + 1;
       chunks = (n + chunk - 1) / chunk;
       rows = (int64_t)g * (k_r + 1);
-      nrg = rows > p.max_rows_item ? 2 : 1;
-      rows0 = (rows + nrg - 1) / nrg;  // rows <= 2 * max_rows_item: both groups fit
+      nrg = (rows + p.max_rows_item - 1) / p.max_rows_item;
+      rows0 = (rows + nrg - 1) / nrg;  // every group but the last; rows <= row_groups * max_rows_item
     }
     const int64_t nitems = chunks * p.Hkv * nrg;
     // each split item's partials start on a 16-byte boundary (vector stores)
-    const int64_t slot_a = (rows0 * (p.D + 2) + 3) / 4 * 4;
-    const int64_t slot_b = nrg == 2 ? ((rows - rows0) * (p.D + 2) + 3) / 4 * 4 : 0;
-    const int64_t pfl = chunks > 1 ? chunks * p.Hkv * (slot_a + slot_b) : 0;
+    const int64_t slot = (rows0 * (p.D + 2) + 3) / 4 * 4;
+    const int64_t pfl = chunks > 1 ? nitems * slot : 0;
     int64_t sv[2] = {nitems, pfl}, st[2];
     block_scan_n<2>(sv, s_warp4, st);
     const int64_t ii = sv[0], ip = sv[1], ti = st[0], tp = st[1];
@@ -315,8 +314,8 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
     s_q0[tid] = r < p.B ? (one ? my_q0 : p.q_row_start[r]) : 0;
     s_nn[tid] = (int32_t)n;
     // per (request, head, row group) finished-chunk counters of the chunk's requests: zeroed, coalesced
-    const int64_t pd0 = (int64_t)base * p.Hkv * 2;
-    const int64_t pd1 = (int64_t)min(p.B, base + kThreads) * p.Hkv * 2;
+    const int64_t pd0 = (int64_t)base * p.Hkv * p.row_groups;
+    const int64_t pd1 = (int64_t)min(p.B, base + kThreads) * p.Hkv * p.row_groups;
     for (int64_t x = pd0 + tid; x < pd1; x += kThreads) p.pair_done[x] = 0;
     __syncthreads();
     for (int64_t i = tid; i < ti; i += kThreads) {
@@ -331,23 +330,22 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
       const int ch = s_ch[lo];
       if (ch == 0 || rr >= p.B) continue;  // a refused request (its scan slot is empty)
       const int rws = s_rows[lo];
-      const int ng = rws > p.max_rows_item ? 2 : 1;
+      const int ng = (rws + p.max_rows_item - 1) / p.max_rows_item;
       const int r0 = (rws + ng - 1) / ng;
       const int j = (int)(i - s_first[lo]);  // (head, row group, chunk) in that order
       const int hg = j / ch, c = j - hg * ch;
-      const int h = ng == 2 ? hg >> 1 : hg, rg = ng == 2 ? hg & 1 : 0;
-      const int sa = (r0 * (p.D + 2) + 3) / 4 * 4;
-      const int sb = ng == 2 ? ((rws - r0) * (p.D + 2) + 3) / 4 * 4 : 0;
+      const int h = hg / ng, rg = hg - h * ng;
+      const int slot = (r0 * (p.D + 2) + 3) / 4 * 4;
       WorkItem it;
       it.r = rr;
       it.h = h;
       it.t0 = (int32_t)(c * chunk);
       it.t1 = (int32_t)min64(s_nn[lo], (c + 1) * chunk);
-      it.row0 = rg ? r0 : 0;
-      it.rows = rg ? rws - r0 : r0;
+      it.row0 = rg * r0;
+      it.rows = min(r0, rws - rg * r0);
       it.rg = rg;
       it.nrg = ng;
-      it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)(h * ch + c) * (sa + sb) + (rg ? sa : 0)) : -1;
+      it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)j * slot) : -1;
       it.q0 = s_q0[lo];
       it.ctx = s_ctx[lo];
       it.pad = 0;
@@ -419,11 +417,12 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
     // CTAs of 152); with more it is bound by each SM's streaming rate, and only a few SMs (an
     // eighth) pay off by starting the acceptance early (2-3% at 256-512 requests; a quarter or
     // more is slower).  When the acceptance has little vocabulary work per KV tile (under 50
-    // elements: a few requests with long contexts) every SM stays with the attention.
+    // elements: a few requests with long contexts) every SM stays with the attention.  The fp32
+    // kernel is bound by arithmetic, so every SM taken from it costs.
     const int sms = p.target_items / kItemsPerSM;
     int na = sms;
     if (p.with_accept && p.split_sms && tiles > 0 && (int64_t)p.B * p.V >= 50 * tiles)
-      na = tiles < (int64_t)200 * sms ? sms / 2 + 4 : sms - sms / 8;
+      na = !p.kv_f32 && tiles < (int64_t)200 * sms ? sms / 2 + 4 : sms - sms / 8;
     PlanHeader hd;
     hd.n_items = (int32_t)n_items;
     hd.chunk_len = (int32_t)chunk;

@@ -17,7 +17,7 @@ struct alignas(16) WorkItem {  // 48 bytes: written and read as three 16-byte ve
   int32_t ctx;    // c_r
   int32_t row0;   // first query row of the item within its (request, head)
   int32_t rg;     // row group of the item
-  int32_t nrg;    // row groups of its (request, head): 1 or 2
+  int32_t nrg;    // row groups of its (request, head)
   int32_t pad;
 };
 static_assert(sizeof(WorkItem) == 48, "work item layout");
@@ -68,7 +68,7 @@ struct Layout {
   size_t plan_header = 0;     // PlanHeader
   size_t req_item_begin = 0;  // int32 [B]  first item of request r
   size_t req_chunks = 0;      // int32 [B]  chunks per KV head of request r
-  size_t pair_done = 0;       // int32 [B * Hkv * 2] finished chunks per split (request, head, row group)
+  size_t pair_done = 0;       // int32 [B * Hkv * row_groups] finished chunks per split (request, head, row group)
   size_t items = 0;           // WorkItem [max_items]
   size_t order = 0;           // int32 [max_items]  dispatch order of the items (largest first)
   size_t partials = 0;        // float [partial_cap]
@@ -89,14 +89,17 @@ struct Layout {
   int64_t max_items = 0;
   int64_t partial_cap = 0;    // floats
   int target_items = 0;
+  int row_groups = 0;         // row groups per (request, head) at most
 };
 
 struct PlanParams {
   int B, Hq, Hkv, D, max_blocks_per_seq, block_size;
   int total_q_rows, total_draft;  // total_draft < 0: not checked (attention-only call)
+  int kv_f32;                  // 1: fp32 queries and cache (the CUDA-core attention kernel)
   int with_attention;          // 0: offsets and validation only
   int target_items;
-  int max_rows_item;           // row groups of at most this many rows (rows per head <= 2 * this)
+  int max_rows_item;           // row groups of at most this many rows
+  int row_groups;              // row groups per (request, head) at most
   int64_t max_items, partial_cap;
   const int32_t *draft_lens, *context_lens;
   const int64_t *request_ids;
