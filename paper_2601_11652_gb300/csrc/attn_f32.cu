@@ -21,9 +21,11 @@
 // the chunks' partials.
 //
 // What bounds it: fp32 multiply-adds at 32 rows (two per key, row and head-dim element; about 74 TFLOP/s
-// on 152 SMs), the K / V stream below about 12 rows.  With the previous kernel (32-token tiles staged
-// through scalar loads, one warp shuffle per key and row, accumulators in shared memory) 32 requests of
-// 512-4096 tokens, 32 query and 8 KV heads, D = 128 took 5870 us; now @F32US@ us.
+// on 152 SMs), of which it reaches half: the scores read RL + 2 floats per lane for 2 RL products, and
+// shared memory delivers one float a lane per four multiply-adds.  Below about 8 rows, the K / V stream
+// (4.7 TB/s at 4 rows).  With the previous kernel (32-token tiles staged through scalar loads, one warp
+// shuffle per key and row, accumulators in shared memory) 32 requests of 512-4096 tokens, 32 query and 8
+// KV heads, D = 128 took 5870 us; now 290 us.
 #include "attn_merge.cuh"
 
 #include <cstring>
@@ -275,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_f32_kernel(const __grid_cons
     if (it < 0 || *(volatile int *)&sh.abort_) break;
     const WorkItem w = p.items[it];
     // the item's query rows (rows past `rows` up to the lanes' share read as zero)
-    const int rl = w.rows <= 4 ? 1 : w.rows <= 8 ? 2 : w.rows <= 16 ? 4 : w.rows <= 24 ? 6 : 8;
+    const int rl = (w.rows + 3) / 4;
     const float *qg = static_cast<const float *>(p.q);
     for (int c = tid; c < 4 * rl * (D / 4); c += kThreads) {
       const int row = c / (D / 4), cc = c % (D / 4), rj = w.row0 + row;
@@ -288,8 +290,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_f32_kernel(const __grid_cons
     switch (rl) {
       case 1: item_rows<D, 1>(p, w, g, smem, sh, warp, nk, nv); break;
       case 2: item_rows<D, 2>(p, w, g, smem, sh, warp, nk, nv); break;
+      case 3: item_rows<D, 3>(p, w, g, smem, sh, warp, nk, nv); break;
       case 4: item_rows<D, 4>(p, w, g, smem, sh, warp, nk, nv); break;
+      case 5: item_rows<D, 5>(p, w, g, smem, sh, warp, nk, nv); break;
       case 6: item_rows<D, 6>(p, w, g, smem, sh, warp, nk, nv); break;
+      case 7: item_rows<D, 7>(p, w, g, smem, sh, warp, nk, nv); break;
       default: item_rows<D, 8>(p, w, g, smem, sh, warp, nk, nv); break;
     }
     __syncthreads();
