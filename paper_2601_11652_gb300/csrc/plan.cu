@@ -20,65 +20,33 @@ constexpr int kOrderTile = 64;       // tokens per KV tile of the attention kern
 __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 __device__ __forceinline__ int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
 
-// Inclusive block scan of one int64 per thread; returns the inclusive value, *total the block sum.
-__device__ int64_t block_scan(int64_t v, int64_t *s_warp, int64_t *total) {
+// Inclusive block scan of one int per thread; returns the inclusive value, *total the block sum.  One
+// barrier: every warp scans the warps' sums itself.  s_w (32 values) may be written again only after
+// another barrier.
+__device__ int block_scan(int v, int *s_w, int *total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    int64_t o = __shfl_up_sync(0xffffffffu, v, d);
+    const int o = __shfl_up_sync(0xffffffffu, v, d);
     if (lane >= d) v += o;
   }
-  if (lane == 31) s_warp[w] = v;
+  if (lane == 31) s_w[w] = v;
   __syncthreads();
-  if (w == 0) {
-    int64_t t = s_warp[lane];
-    for (int d = 1; d < 32; d <<= 1) {
-      int64_t o = __shfl_up_sync(0xffffffffu, t, d);
-      if (lane >= d) t += o;
-    }
-    s_warp[lane] = t;
+  int t = s_w[lane];
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, t, d);
+    if (lane >= d) t += o;
   }
-  __syncthreads();
-  int64_t res = v + (w > 0 ? s_warp[w - 1] : 0);
-  *total = s_warp[31];
-  __syncthreads();
-  return res;
+  const int before = __shfl_sync(0xffffffffu, t, (w + 31) & 31);
+  *total = __shfl_sync(0xffffffffu, t, 31);
+  return v + (w > 0 ? before : 0);
 }
 
-// Inclusive block scans of N int64 per thread at once (one set of barriers for all N): v is replaced
-// by its inclusive values, total[] receives the block sums.  s_w holds N x 32 values.
-template <int N>
-__device__ void block_scan_n(int64_t (&v)[N], int64_t (*s_w)[32], int64_t (&total)[N]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int d = 1; d < 32; d <<= 1) {
-#pragma unroll
-    for (int x = 0; x < N; ++x) {
-      const int64_t o = __shfl_up_sync(0xffffffffu, v[x], d);
-      if (lane >= d) v[x] += o;
-    }
-  }
-  if (lane == 31) {
-#pragma unroll
-    for (int x = 0; x < N; ++x) s_w[x][w] = v[x];
-  }
-  __syncthreads();
-  if (w == 0) {
-#pragma unroll
-    for (int x = 0; x < N; ++x) {
-      int64_t t = s_w[x][lane];
-      for (int d = 1; d < 32; d <<= 1) {
-        const int64_t o = __shfl_up_sync(0xffffffffu, t, d);
-        if (lane >= d) t += o;
-      }
-      s_w[x][lane] = t;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int x = 0; x < N; ++x) {
-    v[x] += w > 0 ? s_w[x][w - 1] : 0;
-    total[x] = s_w[x][31];
-  }
-  __syncthreads();
+// a / b rounded up, b > 0 (the 64-bit division only where 32 bits do not hold a)
+__device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) {
+  const int64_t x = a + b - 1;
+  return x <= 0xffffffffll && b <= 0xffffffffll ? (int64_t)((uint32_t)x / (uint32_t)b) : x / b;
 }
 
 // The acceptance pass's dispatch order and state.  Rows are listed level-major: row index 0 of
@@ -87,10 +55,11 @@ __device__ void block_scan_n(int64_t (&v)[N], int64_t (*s_w)[32], int64_t (&tota
 // of a request is then usually known before its row i + 1 comes up, and the acceptance kernel skips
 // rows past a rejection.  Also clears the per-row and per-request state of the launch and gives the
 // requests this planner refused -1 outputs.
-__device__ void plan_accept(const PlanParams &p, int64_t *s_warp) {
+__device__ void plan_accept(const PlanParams &p) {
   constexpr int KB = kMaxDraft + 1;  // draft lengths 0..kMaxDraft
   __shared__ int32_t s_n[KB + 1];    // level sizes n_i = #{valid r : k_r >= i}, then cursors
   __shared__ int32_t s_ls[KB + 1];   // level starts
+  __shared__ int s_w[2][32];
   const int tid = threadIdx.x;
   __syncthreads();  // pass 1's flags and offsets are visible to every thread
   for (int b = tid; b <= KB; b += kThreads) s_n[b] = 0;
@@ -117,30 +86,29 @@ __device__ void plan_accept(const PlanParams &p, int64_t *s_warp) {
   __shared__ int32_t s_nvalid;
   if (tid == 0) s_nvalid = 0;
   __syncthreads();
-  for (int o = 16; o > 0; o >>= 1) nv += __shfl_xor_sync(0xffffffffu, nv, o);
+  nv = __reduce_add_sync(0xffffffffu, nv);
   if ((tid & 31) == 0 && nv) atomicAdd(&s_nvalid, nv);
-  __syncthreads();
-  const int64_t nvalid = s_nvalid;
   static_assert(KB + 1 <= 2 * kThreads, "two histogram buckets per thread");
   // n_i: suffix sums of the histogram (buckets in decreasing order, two per thread)
   {
     const int b0 = KB - 1 - 2 * tid, b1 = b0 - 1;
-    const int64_t h0 = b0 >= 0 ? s_n[b0] : 0, h1 = b1 >= 0 ? s_n[b1] : 0;
-    int64_t tot;
-    const int64_t incl = block_scan(h0 + h1, s_warp, &tot);
-    if (b0 >= 0) s_n[b0] = (int32_t)(incl - h1);
-    if (b1 >= 0) s_n[b1] = (int32_t)incl;
+    const int h0 = b0 >= 0 ? s_n[b0] : 0, h1 = b1 >= 0 ? s_n[b1] : 0;
+    int tot;
+    const int incl = block_scan(h0 + h1, s_w[0], &tot);
+    if (b0 >= 0) s_n[b0] = incl - h1;
+    if (b1 >= 0) s_n[b1] = incl;
   }
   if (tid == 0) s_n[KB] = 0;
   __syncthreads();
+  const int nvalid = s_nvalid;
   // level starts: exclusive prefix sums of n_i (two per thread)
-  int64_t rows_valid;
+  int rows_valid;
   {
     const int b0 = 2 * tid, b1 = b0 + 1;
-    const int64_t c0 = b0 <= KB ? s_n[b0] : 0, c1 = b1 <= KB ? s_n[b1] : 0;
-    const int64_t incl = block_scan(c0 + c1, s_warp, &rows_valid);
-    if (b0 <= KB) s_ls[b0] = (int32_t)(incl - c0 - c1);
-    if (b1 <= KB) s_ls[b1] = (int32_t)(incl - c1);
+    const int c0 = b0 <= KB ? s_n[b0] : 0, c1 = b1 <= KB ? s_n[b1] : 0;
+    const int incl = block_scan(c0 + c1, s_w[1], &rows_valid);
+    if (b0 <= KB) s_ls[b0] = incl - c0 - c1;
+    if (b1 <= KB) s_ls[b1] = incl - c1;
   }
   __syncthreads();
   // cursors: in every level, the requests with a larger k come first; bucket k starts at n_{k+1}
@@ -162,8 +130,8 @@ __device__ void plan_accept(const PlanParams &p, int64_t *s_warp) {
     for (int i = 0; i <= k; ++i) p.row_order[s_ls[i] + pos] = make_int2(r, i);
   }
   if (tid == 0) {
-    p.acc_ctr->n_items = (int32_t)(rows_valid * p.sslices);
-    p.acc_ctr->n_valid = (int32_t)nvalid;
+    p.acc_ctr->n_items = rows_valid * p.sslices;
+    p.acc_ctr->n_valid = nvalid;
     p.acc_ctr->q_reserve = 0;
     p.acc_ctr->q_head = 0;
     p.acc_ctr->n_claimed = 0;
@@ -177,28 +145,40 @@ __device__ void plan_accept(const PlanParams &p, int64_t *s_warp) {
 
 }  // namespace
 
+// One CTA, bound by latency: global loads of the lengths, then barriers.  So: 32-bit scans with one barrier
+// each, each item's bucket kept from the pass that writes it, and no 64-bit division where 32 bits hold the
+// operands.  With 64-bit scans of three barriers, separate passes and a binary search per pass, one request
+// took 9.7 us here and 256 requests 18.4 us (cold caches, launch included); now 8.6 and 15 us.
 __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
   // a kernel launched after this one with programmatic stream serialization (the attention) may
   // start its own set-up now; it reads the plan only after waiting for this grid to complete
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __shared__ int64_t s_warp[32];
-  __shared__ int64_t s_warp4[4][32];
-  const int tid = threadIdx.x;
+  constexpr int kKeep = 4;  // items per thread whose bucket is kept in registers
+  __shared__ int s_w[6][32];
+  __shared__ unsigned long long s_sum[2];  // keys of the valid requests; KV tiles of the items
+  __shared__ int32_t s_valid;
+  __shared__ int32_t s_hist[kOrderBuckets];
+  const int tid = threadIdx.x, lane = tid & 31;
   // the launch's status word starts clear (every kernel of the call reports into it)
   if (tid == 0) {
     p.status->code = 0;
     p.status->pad = 0;
     p.status->request_id = 0;
+    s_sum[0] = s_sum[1] = 0;
+    s_valid = 0;
   }
-  __syncthreads();
+  s_hist[tid] = 0;
+  static_assert(kOrderBuckets == kThreads, "one bucket per thread");
   const int g = p.Hq > 0 && p.Hkv > 0 ? p.Hq / p.Hkv : 1;
   const int64_t cap_tokens = (int64_t)p.max_blocks_per_seq * p.block_size;
-
-  // pass 1: offsets (negative lengths count as 0) and validation
-  int64_t carry_q = 0, carry_d = 0, carry_n = 0, carry_v = 0;
   // with at most kThreads requests, pass 3 reuses what this thread read and decided here
+  const bool one = p.B <= kThreads;
   int32_t my_k = 0, my_ctx = 0, my_q0 = 0;
   bool my_ok = false;
+
+  // pass 1: offsets (negative lengths count as 0) and validation.  A request's first query row is its
+  // first draft row plus its index, so one scan gives both.
+  int64_t carry_d = 0;
   for (int base = 0; base < p.B; base += kThreads) {
     const int r = base + tid;
     int64_t k = 0, n = 0;
@@ -206,21 +186,39 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
     if (r < p.B) {
       k = p.draft_lens[r];
       my_k = (int32_t)k;
+      const int64_t c = p.with_attention ? p.context_lens[r] : 0;
+      my_ctx = (int32_t)c;
       if (k < 0) { bad = WISP_DEV_BAD_LENGTH; k = 0; }
       if (!bad && k > kMaxDraft) bad = WISP_DEV_UNSUPPORTED;
       if (p.with_attention) {
-        const int64_t c = p.context_lens[r];
-        my_ctx = (int32_t)c;
         if (!bad && (c < 0 || c + k + 1 > cap_tokens)) bad = WISP_DEV_BAD_LENGTH;
         if (!bad && (int64_t)g * (k + 1) > kMaxRowsPerHead) bad = WISP_DEV_UNSUPPORTED;
         n = bad ? 0 : c + k + 1;
       }
     }
-    int64_t sv[4] = {r < p.B ? k + 1 : 0, r < p.B ? k : 0, n, n > 0 ? 1 : 0}, st[4];
-    block_scan_n<4>(sv, s_warp4, st);
-    const int64_t iq = sv[0], id = sv[1], tq = st[0], td = st[1], tn = st[2], tv = st[3];
+    // the scan in 32 bits (no sum of 1024 lengths up to 2^20 overflows), or in two parts of 16 bits when a
+    // length, refused itself but counted in the offsets, is longer.  (The first barrier is also what makes
+    // the cleared shared and status words visible.)
+    int64_t incl, td;
+    if (!__syncthreads_or(k > (1 << 20))) {
+      int t;
+      incl = block_scan((int)k, s_w[base / kThreads % 2], &t);
+      td = t;
+    } else {
+      int tl, th;
+      const int lo = block_scan((int)k & 0xffff, s_w[2], &tl);
+      const int hi = block_scan((int)(k >> 16), s_w[base / kThreads % 2], &th);
+      incl = lo + ((int64_t)hi << 16);
+      td = tl + ((int64_t)th << 16);
+    }
+    const unsigned vm = __ballot_sync(0xffffffffu, n > 0);
+    const unsigned n_lo = __reduce_add_sync(0xffffffffu, (unsigned)n & 0xffffu), n_hi = __reduce_add_sync(0xffffffffu, (unsigned)n >> 16);
+    if (lane == 0 && vm) {
+      atomicAdd(&s_sum[0], (unsigned long long)n_lo + ((unsigned long long)n_hi << 16));
+      atomicAdd(&s_valid, __popc(vm));
+    }
     if (r < p.B) {
-      const int64_t q0 = carry_q + iq - (k + 1), d0 = carry_d + id - k;
+      const int64_t d0 = carry_d + incl - k, q0 = d0 + r;
       // a request whose rows fall outside the caller's buffers is never touched
       if (!bad && (q0 + k + 1 > p.total_q_rows || (p.total_draft >= 0 && d0 + k > p.total_draft)))
         bad = WISP_DEV_BAD_LENGTH;
@@ -231,20 +229,18 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
       my_ok = !bad;
       if (bad) report(p.status, bad, p.request_ids, r);
     }
-    carry_q += tq;
     carry_d += td;
-    carry_n += tn;
-    carry_v += tv;
   }
+  if (p.B == 0) __syncthreads();
   if (tid == 0) {
-    p.q_row_start[p.B] = (int32_t)min64(carry_q, INT32_MAX);
+    p.q_row_start[p.B] = (int32_t)min64(carry_d + p.B, INT32_MAX);
     p.draft_start[p.B] = (int32_t)min64(carry_d, INT32_MAX);
-    if (carry_q != p.total_q_rows || (p.total_draft >= 0 && carry_d != p.total_draft)) {
+    if (carry_d + p.B != p.total_q_rows || (p.total_draft >= 0 && carry_d != p.total_draft)) {
       // the caller sized its buffers with other totals: flag it (requests that still fit run)
       atomicCAS(&p.status->code, 0, (int32_t)WISP_DEV_BAD_LENGTH);
     }
   }
-  if (p.with_accept && !p.accept_apart) plan_accept(p, s_warp);
+  if (p.with_accept && !p.accept_apart) plan_accept(p);
   if (!p.with_attention) return;
   __syncthreads();
 
@@ -254,45 +250,50 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
   // into about kItemsPerSM items per SM.  The fp32 kernel's time also grows with the item's rows, which
   // the order does not see, so it gets items of at most 2/3 of the average (32 requests of 512-4096
   // tokens: 307 us at 5/4, 290 at 2/3, 302 at 1/2; the tensor-core kernel there: 68, 80, 83 us).
-  const int64_t work = carry_n * p.Hkv;
+  const int64_t work = (int64_t)s_sum[0] * p.Hkv;
   const int64_t sms = max(1, p.target_items / kItemsPerSM);
-  const bool many_pairs = carry_v * p.Hkv >= sms;
+  const bool many_pairs = (int64_t)s_valid * p.Hkv >= sms;
   const int64_t goal = many_pairs ? sms : (int64_t)p.target_items;
-  int64_t chunk = (work + goal - 1) / goal;
+  int64_t chunk = ceil_div(work, goal);
   if (many_pairs) chunk = p.kv_f32 ? chunk - chunk / 3 : chunk + chunk / 4;
   chunk = max64(chunk, kMinChunk);
-  chunk = (chunk + kChunkAlign - 1) / kChunkAlign * kChunkAlign;
+  chunk = min64((chunk + kChunkAlign - 1) / kChunkAlign * kChunkAlign, (int64_t)1 << 30);  // (a sequence is shorter)
 
-  // pass 3: items and partial slots (request-major, then KV head, then row group, then chunk).
-  // Per chunk of kThreads requests: one thread per request sizes its items (block scans), then the
-  // chunk's items are written by consecutive threads (item i by thread i mod kThreads, its request
-  // found by binary search over the chunk's first items), so that the stores coalesce.
+  // pass 3: items and partial slots (request-major, then KV head, then row group, then chunk), and the
+  // histogram of their lengths.  Per chunk of kThreads requests: one thread per request sizes its items
+  // (block scans), then the chunk's items are written by consecutive threads (item i by thread
+  // i mod kThreads, its request found by binary search over the chunk's first items), so that the stores
+  // coalesce.
   __shared__ int32_t s_first[kThreads + 1];  // the chunk's requests' first items, relative
   // per request of the chunk: query rows, chunks (0: no items), first partial, context, first
   // query row, keys
   __shared__ int32_t s_rows[kThreads], s_ch[kThreads], s_pf[kThreads], s_ctx[kThreads], s_q0[kThreads], s_nn[kThreads];
+  auto bucket_of = [&](int tokens) -> int {  // bucket 0: the longest
+    return kOrderBuckets - 1 - min((tokens + kOrderTile - 1) / kOrderTile, kOrderBuckets - 1);
+  };
   int64_t item_carry = 0, poff_carry = 0;
+  int keep[kKeep];
+#pragma unroll
+  for (int x = 0; x < kKeep; ++x) keep[x] = 0;
+  unsigned long long my_tiles = 0;  // KV tiles (kOrderTile tokens) of this thread's items
   for (int base = 0; base < p.B; base += kThreads) {
     const int r = base + tid;
-    int64_t n = 0, chunks = 0, rows = 0, nrg = 1, rows0 = 0;
-    int32_t ctx_r = 0;
-    const bool one = p.B <= kThreads;  // this thread's request of pass 1
+    int n = 0, chunks = 0, rows = 0, nrg = 1, rows0 = 0, ctx_r = 0;
     if (r < p.B && (one ? my_ok : p.req_flag[r] == REQ_OK)) {
       const int32_t k_r = one ? my_k : p.draft_lens[r];
       ctx_r = one ? my_ctx : p.context_lens[r];
-      n = (int64_t)ctx_r + k_r + 1;
-      chunks = (n + chunk - 1) / chunk;
-      rows = (int64_t)g * (k_r + 1);
+      n = ctx_r + k_r + 1;
+      chunks = (int)(((unsigned)n + (unsigned)chunk - 1) / (unsigned)chunk);
+      rows = g * (k_r + 1);
       nrg = (rows + p.max_rows_item - 1) / p.max_rows_item;
       rows0 = (rows + nrg - 1) / nrg;  // every group but the last; rows <= row_groups * max_rows_item
     }
-    const int64_t nitems = chunks * p.Hkv * nrg;
+    const int nitems = chunks * p.Hkv * nrg;
     // each split item's partials start on a 16-byte boundary (vector stores)
-    const int64_t slot = (rows0 * (p.D + 2) + 3) / 4 * 4;
-    const int64_t pfl = chunks > 1 ? nitems * slot : 0;
-    int64_t sv[2] = {nitems, pfl}, st[2];
-    block_scan_n<2>(sv, s_warp4, st);
-    const int64_t ii = sv[0], ip = sv[1], ti = st[0], tp = st[1];
+    const int slot = (rows0 * (p.D + 2) + 3) / 4 * 4;
+    const int pfl = chunks > 1 ? nitems * slot : 0;
+    int ti, tp;  // (a batch's items and partials are bounded by max_items and partial_cap: 32 bits hold them)
+    const int ii = block_scan(nitems, s_w[3], &ti), ip = block_scan(pfl, s_w[4], &tp);
     bool fits = false;
     if (r < p.B) {
       const int64_t first = item_carry + ii - nitems;
@@ -304,23 +305,23 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
         report(p.status, WISP_DEV_UNSUPPORTED, p.request_ids, r);
       }
       p.req_item_begin[r] = (int32_t)first;
-      p.req_chunks[r] = fits ? (int32_t)chunks : 0;
+      p.req_chunks[r] = fits ? chunks : 0;
     }
-    // the chunk's requests in shared memory: first item (relative), rows, chunks (0: no items)
-    s_first[tid] = (int32_t)(ii - nitems);
-    if (tid == kThreads - 1) s_first[kThreads] = (int32_t)ti;
-    s_rows[tid] = (int32_t)rows;
-    s_ch[tid] = fits ? (int32_t)chunks : 0;
+    s_first[tid] = ii - nitems;
+    if (tid == kThreads - 1) s_first[kThreads] = ti;
+    s_rows[tid] = rows;
+    s_ch[tid] = fits ? chunks : 0;
     s_pf[tid] = (int32_t)min64(poff_carry + ip - pfl, INT32_MAX);
     s_ctx[tid] = ctx_r;
     s_q0[tid] = r < p.B ? (one ? my_q0 : p.q_row_start[r]) : 0;
-    s_nn[tid] = (int32_t)n;
+    s_nn[tid] = n;
     // per (request, head, row group) finished-chunk counters of the chunk's requests: zeroed, coalesced
     const int64_t pd0 = (int64_t)base * p.Hkv * p.row_groups;
     const int64_t pd1 = (int64_t)min(p.B, base + kThreads) * p.Hkv * p.row_groups;
     for (int64_t x = pd0 + tid; x < pd1; x += kThreads) p.pair_done[x] = 0;
     __syncthreads();
-    for (int64_t i = tid; i < ti; i += kThreads) {
+    int x = 0;
+    for (int i = tid; i < ti; i += kThreads, ++x) {
       // the request of item i: the last one whose first item is <= i
       int lo = 0, hi = kThreads - 1;
       while (lo < hi) {
@@ -330,87 +331,86 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
       }
       const int rr = base + lo;
       const int ch = s_ch[lo];
-      if (ch == 0 || rr >= p.B) continue;  // a refused request (its scan slot is empty)
-      const int rws = s_rows[lo];
-      const int ng = (rws + p.max_rows_item - 1) / p.max_rows_item;
-      const int r0 = (rws + ng - 1) / ng;
-      const int j = (int)(i - s_first[lo]);  // (head, row group, chunk) in that order
-      const int hg = j / ch, c = j - hg * ch;
-      const int h = hg / ng, rg = hg - h * ng;
-      const int slot = (r0 * (p.D + 2) + 3) / 4 * 4;
-      WorkItem it;
-      it.r = rr;
-      it.h = h;
-      it.t0 = (int32_t)(c * chunk);
-      it.t1 = (int32_t)min64(s_nn[lo], (c + 1) * chunk);
-      it.row0 = rg * r0;
-      it.rows = min(r0, rws - rg * r0);
-      it.rg = rg;
-      it.nrg = ng;
-      it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)j * slot) : -1;
-      it.q0 = s_q0[lo];
-      it.ctx = s_ctx[lo];
-      it.pad = 0;
-      p.items[item_carry + i] = it;
+      if (item_carry + i >= p.max_items) continue;  // (a request refused for want of room)
+      int bucket = kOrderBuckets - 1;
+      if (ch == 0) {  // a refused request's slot: an empty item, listed last; the kernels skip it
+        WorkItem it = {};
+        it.r = rr;
+        p.items[item_carry + i] = it;
+      } else {
+        const int rws = s_rows[lo];
+        const int ng = (rws + p.max_rows_item - 1) / p.max_rows_item;
+        const int r0 = (rws + ng - 1) / ng;
+        const int j = i - s_first[lo];  // (head, row group, chunk) in that order
+        const int hg = j / ch, c = j - hg * ch;
+        const int h = hg / ng, rg = hg - h * ng;
+        const int slot_r = (r0 * (p.D + 2) + 3) / 4 * 4;
+        WorkItem it;
+        it.r = rr;
+        it.h = h;
+        it.t0 = (int32_t)(c * chunk);
+        it.t1 = (int32_t)min64(s_nn[lo], (c + 1) * chunk);
+        it.row0 = rg * r0;
+        it.rows = min(r0, rws - rg * r0);
+        it.rg = rg;
+        it.nrg = ng;
+        it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)j * slot_r) : -1;
+        it.q0 = s_q0[lo];
+        it.ctx = s_ctx[lo];
+        it.pad = 0;
+        p.items[item_carry + i] = it;
+        bucket = bucket_of(it.t1 - it.t0);
+        my_tiles += (unsigned)(it.t1 - it.t0 + kOrderTile - 1) / kOrderTile;
+      }
+      atomicAdd(&s_hist[bucket], 1);
+#pragma unroll
+      for (int y = 0; y < kKeep; ++y)
+        if (y == x) keep[y] = bucket;
     }
     item_carry += ti;
     poff_carry += tp;
-    __syncthreads();  // s_first / s_rq are rewritten by the next chunk
+    __syncthreads();  // the shared arrays are rewritten by the next chunk; the histogram is complete after the last
   }
   // pass 4: dispatch order, longest items first (counting sort on the tile count), so that the
   // persistent kernel ends with its shortest items and its CTAs finish close together
-  __shared__ int32_t s_hist[kOrderBuckets];
-  const int64_t n_items = min64(item_carry, p.max_items);
-  for (int b = tid; b < kOrderBuckets; b += kThreads) s_hist[b] = 0;
-  __syncthreads();  // also makes pass 3's items visible to every thread of the block
-  // an item's KV tiles: with one chunk of requests (B <= kThreads) from pass 3's shared arrays,
-  // which still describe every request (no global read of the items just written), else from the
-  // item itself
-  const bool one_chunk = p.B <= kThreads;
-  auto item_tiles = [&](int64_t i) -> int64_t {
-    int64_t t0, t1;
-    if (one_chunk) {
+  const int n_items = (int)min64(item_carry, p.max_items);
+  for (int o = 16; o > 0; o >>= 1) my_tiles += __shfl_xor_sync(0xffffffffu, my_tiles, o);
+  if (lane == 0 && my_tiles) atomicAdd(&s_sum[1], my_tiles);
+  {
+    const int h = s_hist[tid];
+    int tot;
+    s_hist[tid] = block_scan(h, s_w[5], &tot) - h;
+  }
+  __syncthreads();
+  int x = 0;
+  for (int i = tid; i < n_items; i += kThreads, ++x) {
+    int bucket = 0;
+    if (one && x < kKeep) {
+#pragma unroll
+      for (int y = 0; y < kKeep; ++y)
+        if (y == x) bucket = keep[y];
+    } else if (one) {  // from the shared arrays, which still describe every request
       int lo = 0, hi = kThreads - 1;
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (s_first[mid] <= i) lo = mid;
         else hi = mid - 1;
       }
-      const int ch = max(1, s_ch[lo]);
-      const int c = (int)(i - s_first[lo]) % ch;  // item = (head, row group) * ch + chunk
-      t0 = (int64_t)c * chunk;
-      t1 = min64(s_nn[lo], t0 + chunk);
+      const int ch = s_ch[lo];
+      bucket = kOrderBuckets - 1;
+      if (ch > 0) {
+        const int64_t t0 = (int64_t)((i - s_first[lo]) % ch) * chunk;
+        bucket = bucket_of((int)(min64(s_nn[lo], t0 + chunk) - t0));
+      }
     } else {
       const WorkItem &w = p.items[i];
-      t0 = w.t0;
-      t1 = w.t1;
+      bucket = bucket_of(w.t1 - w.t0);  // (an empty item: the last bucket)
     }
-    return (t1 - t0 + kOrderTile - 1) / kOrderTile;
-  };
-  auto bucket_of = [&](int64_t tiles) -> int {
-    return kOrderBuckets - 1 - (int)max64(0, min64(tiles, kOrderBuckets - 1));  // bucket 0: the longest
-  };
-  int64_t my_tiles = 0;  // KV tile passes of the attention (kOrderTile tokens), this thread's items
-  for (int64_t i = tid; i < n_items; i += kThreads) {
-    const int64_t t = item_tiles(i);
-    atomicAdd(&s_hist[bucket_of(t)], 1);
-    my_tiles += t;
+    p.order[atomicAdd(&s_hist[bucket], 1)] = i;
   }
-  __syncthreads();
-  {
-    static_assert(kOrderBuckets == kThreads, "one bucket per thread in the scan");
-    int64_t tot;
-    const int64_t incl = block_scan(s_hist[tid], s_warp, &tot);
-    const int32_t excl = (int32_t)(incl - s_hist[tid]);
-    __syncthreads();
-    s_hist[tid] = excl;
-    __syncthreads();
-  }
-  for (int64_t i = tid; i < n_items; i += kThreads) p.order[atomicAdd(&s_hist[bucket_of(item_tiles(i))], 1)] = (int32_t)i;
-  int64_t tiles = 0;
-  block_scan(my_tiles, s_warp, &tiles);
 
   if (tid == 0) {
+    const int64_t tiles = (int64_t)s_sum[1];
     // SMs for the attention in a step whose acceptance pass runs beside it.  Both kernels are
     // persistent and each fills an SM's shared memory, so the acceptance CTAs start on the SMs the
     // attention leaves.  Measured on GB300 (bf16, D = 128): with few KV tiles per SM (under ~200
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
     if (p.with_accept && p.split_sms && tiles > 0 && (int64_t)p.B * p.V >= 50 * tiles)
       na = !p.kv_f32 && tiles < (int64_t)200 * sms ? sms / 2 + 4 : sms - sms / 8;
     PlanHeader hd;
-    hd.n_items = (int32_t)n_items;
+    hd.n_items = n_items;
     hd.chunk_len = (int32_t)chunk;
     hd.partial_floats = (int32_t)min64(poff_carry, p.partial_cap);
     hd.next_item = 0;
@@ -440,8 +440,7 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
 // that the attention, which waits for the whole planner grid, does not wait for it).  Reads what
 // plan_kernel's first pass wrote (flags and offsets).
 __global__ void __launch_bounds__(kThreads) plan_accept_kernel(const PlanParams p) {
-  __shared__ int64_t s_warp[32];
-  plan_accept(p, s_warp);
+  plan_accept(p);
 }
 
 }  // namespace wisp
