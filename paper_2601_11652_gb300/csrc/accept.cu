@@ -1669,12 +1669,61 @@ __global__ void __launch_bounds__(kCtaThreads, kAcceptCtasPerSM) accept_kernel(c
 // ---- greedy (temperature 0) acceptance -----------------------------------------------------
 // Sampling at temperature 0 takes the most likely token, so the rule of Eq. 1-3 becomes: accept
 // y_i iff y_i is the argmax of logit row i-1 (the lowest token id among equal maxima), stop at the
-// first mismatch, and emit the argmax of row L.  row_argmax_kernel: one warp per (row, slice), every
-// row in parallel; greedy_walk_kernel: one warp per request merges the slices of its rows in order.
+// first mismatch, and emit the argmax of row L.
+//
+// Two forms (greedy_level_major in api.cu):
+//   * a batch whose rows take longer to read than to decide: greedy_kernel, one persistent kernel of
+//     independent warps.  A warp claims (row, slice) items in the planner's level-major row order (row 0 of
+//     every request, then row 1, ...) and skips rows past a mismatch already known for their request; the
+//     warp that finishes a row's last slice merges the slices, scores the row and, once rows 0..L of the
+//     request are scored, writes its outputs.  A row is cut so that one level of the batch keeps every
+//     resident warp busy: then a level is decided while the next one is claimed, and few rows past a
+//     mismatch are read.  Bound by the latency of an item's chain of loads, then by HBM: 256 requests of
+//     1-16 draft tokens, V = 128256, take 77 us for 321 MB (173 MB are needed, 625 MB with every row);
+//   * a smaller one: row_argmax_kernel reads every row at once (one warp per row and slice), then
+//     greedy_walk_kernel walks.  The same 256 requests take 115 us (96% of the copy rate), but 32 requests of
+//     1-8 tokens 26 us against 30.
 struct RowArg {
   float m;  // max of the slice (-inf if none)
   int idx;  // lowest token id attaining it
 };
+__device__ __forceinline__ RowArg warp_argmax(RowArg a) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float om = __shfl_xor_sync(0xffffffffu, a.m, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, a.idx, o);
+    if (om > a.m || (om == a.m && oi < a.idx)) {
+      a.m = om;
+      a.idx = oi;
+    }
+  }
+  return a;
+}
+
+// Writes request r's outputs if its rows 0..L are scored (row codes as in the sampling rule; a scored row's
+// argmax is in row_rec[].m as int bits).  By the warp that has just scored a row.
+__device__ void greedy_determine(const AcceptParams &p, int r, int k, int64_t Q0) {
+  const int lane = threadIdx.x & 31;
+  for (int j0 = 0; j0 <= k; j0 += 32) {
+    const int j = j0 + lane;
+    const int c = j <= k ? ld_vol(p.row_code + Q0 + j) : ROW_ACCEPT;
+    const unsigned stop = __ballot_sync(0xffffffffu, c != ROW_ACCEPT);
+    if (stop == 0) continue;
+    const int l0 = __ffs(stop) - 1;
+    const int c0 = __shfl_sync(0xffffffffu, c, l0);
+    if (c0 == ROW_UNKNOWN || lane != 0 || atomicCAS(p.req_claim + r, 0, 1) != 0) return;
+    if (c0 == ROW_REJECT || c0 == ROW_BONUS) {
+      __threadfence();
+      p.accepted_len[r] = j0 + l0;
+      p.next_token[r] = ld_vol(reinterpret_cast<const int32_t *>(&p.row_rec[Q0 + j0 + l0].m));
+    } else {
+      report(p.status, c0 == ROW_BAD_TOKEN ? WISP_DEV_BAD_TOKEN : WISP_DEV_BAD_PROB, p.request_ids, r);
+      p.accepted_len[r] = -1;
+      p.next_token[r] = -1;
+    }
+    return;
+  }
+}
 
 template <typename LT>
 __global__ void __launch_bounds__(NT) row_argmax_kernel(const __grid_constant__ AcceptParams p) {
@@ -1712,15 +1761,8 @@ __global__ void __launch_bounds__(NT) row_argmax_kernel(const __grid_constant__ 
       }
     }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const float om = __shfl_xor_sync(0xffffffffu, m, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-    if (om > m || (om == m && oi < idx)) {
-      m = om;
-      idx = oi;
-    }
-  }
-  if (lane == 0) reinterpret_cast<RowArg *>(p.parts)[unit] = RowArg{m, idx};
+  const RowArg a = warp_argmax(RowArg{m, idx});
+  if (lane == 0) reinterpret_cast<RowArg *>(p.parts)[unit] = a;
 }
 
 template <typename LT>
@@ -1735,14 +1777,7 @@ __global__ void __launch_bounds__(NT) greedy_walk_kernel(const __grid_constant__
   for (int i = 0; i <= k; ++i) {
     RowArg a{-INFINITY, INT32_MAX};
     if (lane < S) a = parts[(Q0 + i) * S + lane];
-    for (int o = 16; o > 0; o >>= 1) {
-      const float om = __shfl_xor_sync(0xffffffffu, a.m, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, a.idx, o);
-      if (om > a.m || (om == a.m && oi < a.idx)) {
-        a.m = om;
-        a.idx = oi;
-      }
-    }
+    a = warp_argmax(a);
     if (!(a.m > -INFINITY) || a.idx >= V) {  // no finite logit in the row
       err = WISP_DEV_BAD_PROB;
       break;
@@ -1771,6 +1806,94 @@ __global__ void __launch_bounds__(NT) greedy_walk_kernel(const __grid_constant__
       p.accepted_len[r] = L;
       p.next_token[r] = tok;
     }
+  }
+}
+
+template <typename LT>
+__global__ void __launch_bounds__(NT, kGreedyCtasPerSM) greedy_kernel(const __grid_constant__ AcceptParams p) {
+  constexpr int E = LTraits<LT>::E;
+  constexpr int U = 8;  // vectors in flight per lane (4 / 6 / 8 with three CTAs per SM: 86 / 81 / 80 us on the case above)
+  // launched as a programmatic dependent of the planner: read nothing of its before it has completed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int lane = threadIdx.x & 31;
+  const int V = p.V, S = p.slices;
+  const int64_t nvec = (V + E - 1) / E;
+  const int n_items = p.ctr->n_items / p.sslices * S;  // rows of valid requests x slices
+  const int warps = gridDim.x * NW;  // the first item of a warp is its own number
+  auto claim = [&]() { return lane == 0 ? warps + atomicAdd(&p.ctr->stats_next, 1) : 0; };
+  auto entry = [&](int t) { return t < n_items ? __ldg(p.row_order + t / S) : make_int2(0, 0); };
+  int t = blockIdx.x * NW + (threadIdx.x >> 5);
+  int2 ent = entry(t);
+  while (t < n_items) {
+    const int next = claim();  // the next item is looked up while this one is finished
+    int tn = 0;
+    int2 ent_n = make_int2(0, 0);
+    const int r = ent.x, i = ent.y, sl = t % S;
+    if (i <= ld_vol(p.req_rej + r)) {
+      const int k = __ldg(p.draft_lens + r);
+      const int64_t Q0 = __ldg(p.q_row_start + r), D0 = __ldg(p.draft_start + r), R = Q0 + i;
+      const int32_t y = i < k ? __ldg(p.draft_tokens + D0 + i) : 0;
+      const LT *rowp = static_cast<const LT *>(p.logits) + R * (int64_t)V;
+      const int64_t vlo = min(nvec, (int64_t)sl * p.vps), vhi = min(nvec, vlo + p.vps);
+      RowArg a{-INFINITY, INT32_MAX};
+      // a lane visits its elements in increasing token order, so a strict ">" keeps the first maximum
+      for (int64_t v0 = vlo + lane; v0 < vhi; v0 += U * 32) {
+        uint4 w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (v0 + u * 32 < vhi) w[u] = load_vec<LT>(rowp, v0 + u * 32, V, p.vec_z != 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t vi = v0 + u * 32;
+          if (vi >= vhi) break;
+#pragma unroll
+          for (int x = 0; x < E; ++x) {
+            const float z = vec_elem<LT>(w[u], x);
+            if (z > a.m) {
+              a.m = z;
+              a.idx = (int)(vi * E + x);
+            }
+          }
+        }
+      }
+      tn = __shfl_sync(0xffffffffu, next, 0);
+      ent_n = entry(tn);
+      a = warp_argmax(a);
+      RowArg *parts = reinterpret_cast<RowArg *>(p.parts) + R * S;
+      int last = 1;
+      if (S > 1) {
+        if (lane == 0) {
+          __stcg(reinterpret_cast<float2 *>(parts + sl), make_float2(a.m, __int_as_float(a.idx)));
+          __threadfence();
+          last = atomicAdd(&p.row_cnt[R], 1) == S - 1;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+      }
+      if (last) {
+        if (S > 1) {
+          __threadfence();
+          float2 v = make_float2(-INFINITY, __int_as_float(INT32_MAX));
+          if (lane < S) v = __ldcg(reinterpret_cast<const float2 *>(parts + lane));
+          a = warp_argmax(RowArg{v.x, __float_as_int(v.y)});
+        }
+        const bool ok = a.m > -INFINITY && a.idx < V;  // a finite logit in the row
+        const int code = !ok ? ROW_BAD_PROB : i == k ? ROW_BONUS : y < 0 || y >= V ? ROW_BAD_TOKEN : y == a.idx ? ROW_ACCEPT : ROW_REJECT;
+        if (lane == 0) {
+          st_vol(reinterpret_cast<int32_t *>(&p.row_rec[R].m), a.idx);
+          if (code != ROW_ACCEPT) atomicMin(p.req_rej + r, i);
+          __threadfence();
+          st_vol(p.row_code + R, code);
+        }
+        __syncwarp();
+        fence_sc();  // this code before the codes read next (against the warp that scores another row)
+        greedy_determine(p, r, k, Q0);
+      }
+    } else {
+      tn = __shfl_sync(0xffffffffu, next, 0);
+      ent_n = entry(tn);
+    }
+    t = tn;
+    ent = ent_n;
   }
 }
 
@@ -1842,16 +1965,29 @@ cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_
   return bf16 ? launch_t<uint16_t>(p, sms, s, pdl) : launch_t<float>(p, sms, s, pdl);
 }
 
-cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, cudaStream_t s) {
-  const unsigned g1 = (unsigned)((p.total_rows * p.slices + NW - 1) / NW), g2 = (unsigned)((p.B + NW - 1) / NW);
-  if (bf16) {
-    row_argmax_kernel<uint16_t><<<g1, NT, 0, s>>>(p);
-    greedy_walk_kernel<uint16_t><<<g2, NT, 0, s>>>(p);
-  } else {
-    row_argmax_kernel<float><<<g1, NT, 0, s>>>(p);
-    greedy_walk_kernel<float><<<g2, NT, 0, s>>>(p);
+cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, bool level_major, int sms, cudaStream_t s) {
+  if (!level_major) {
+    const unsigned g1 = (unsigned)((p.total_rows * p.slices + NW - 1) / NW), g2 = (unsigned)((p.B + NW - 1) / NW);
+    if (bf16) {
+      row_argmax_kernel<uint16_t><<<g1, NT, 0, s>>>(p);
+      greedy_walk_kernel<uint16_t><<<g2, NT, 0, s>>>(p);
+    } else {
+      row_argmax_kernel<float><<<g1, NT, 0, s>>>(p);
+      greedy_walk_kernel<float><<<g2, NT, 0, s>>>(p);
+    }
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3((unsigned)(sms * kGreedyCtasPerSM));
+  cfg.blockDim = dim3(NT);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return bf16 ? cudaLaunchKernelEx(&cfg, greedy_kernel<uint16_t>, p) : cudaLaunchKernelEx(&cfg, greedy_kernel<float>, p);
 }
 
 }  // namespace wisp

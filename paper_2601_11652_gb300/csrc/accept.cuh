@@ -10,6 +10,7 @@ constexpr int kAcceptCtasPerSM = 2;  // resident CTAs per SM of the persistent a
 constexpr int kStatsChunkVecs = 3;   // 16-byte vectors per consumer thread in one chunk of the statistics stream
 constexpr int kAmbPerSlice = 8;      // residual elements per draw slice whose sign is left to the finisher
 constexpr int kMaxSlices = 32;       // warp slices per row of the greedy variant
+constexpr int kGreedyCtasPerSM = 3;  // resident CTAs (of kAcceptThreads) per SM of the greedy variant
 
 // Per-CTA table of exp(u - m) for the bf16 values u with 2^-16 <= |u| < 2^6 (exponent fields
 // kExpTabLo .. kExpTabLo + kExpTabBinades - 1, both signs): 64-bit fixed-point values of the draw.
@@ -126,7 +127,8 @@ struct AcceptParams {
 cudaError_t accept_setup();  // once per device: kernel attributes, the exp table of the draw
 // the acceptance pass (one persistent kernel; needs the planner's offsets and dispatch order)
 cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_t s, bool pdl);
-// greedy (temperature 0) variant: argmax partials of every row, then the walk (two launches)
-cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, cudaStream_t s);
+// greedy (temperature 0) variant: one persistent kernel in the planner's dispatch order, or argmax partials of
+// every row and then the walk (two launches; needs only the planner's offsets)
+cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, bool level_major, int sms, cudaStream_t s);
 
 }  // namespace wisp

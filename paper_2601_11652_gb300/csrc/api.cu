@@ -100,13 +100,24 @@ wisp_status check_attn(const wisp_attn_args *a) {
   return WISP_OK;
 }
 
-// Vocabulary slices per logit row for the row-statistics kernel (one warp each): enough warps to
-// keep every SM streaming (48 per SM), slices of at least 256 vectors (4 KB), at most kMaxSlices.
-void accept_slices(const wisp_accept_args *c, int sms, int *slices, int *vps) {
+// The greedy variant skips rows past a mismatch (level-major order) when reading every row would take well
+// longer than the planner's ordering and the claims cost (about 3 us and a few us of latency per level):
+// above 128 MiB of logits, 20 us at the copy rate.  Measured: 50 MB 26 us with every row, 30 us in
+// level-major order; 460 MB 88 and 83 us; 625 MB 115 and 77 us.
+bool greedy_level_major(const wisp_accept_args *c) {
+  return (int64_t)c->total_q_rows * c->V * (c->logits_dtype == WISP_BF16 ? 2 : 4) > ((int64_t)128 << 20);
+}
+
+// Vocabulary slices per logit row of the greedy variant (one warp each): enough warps to keep every SM
+// streaming, over one level of the batch (one row per request) in level-major order, else over all rows;
+// slices of at least 256 vectors (4 KB), at most kMaxSlices.
+void greedy_slices(const wisp_accept_args *c, int sms, int *slices, int *vps) {
   const int E = c->logits_dtype == WISP_BF16 ? 8 : 4;
   const int64_t nvec = ((int64_t)c->V + E - 1) / E;
-  const int64_t rows = c->total_q_rows > 0 ? c->total_q_rows : 1;
-  int64_t S = ((int64_t)48 * sms + rows - 1) / rows;
+  const bool lm = greedy_level_major(c);
+  const int64_t rows = lm ? c->B : c->total_q_rows > 0 ? c->total_q_rows : 1;
+  const int64_t warps = lm ? (int64_t)sms * kGreedyCtasPerSM * (kAcceptThreads / 32) : (int64_t)48 * sms;
+  int64_t S = (warps + rows - 1) / rows;
   const int64_t by_size = (nvec + 255) / 256;
   if (S > by_size) S = by_size;
   if (S > kMaxSlices) S = kMaxSlices;
@@ -219,7 +230,7 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
     // the greedy variant's argmax partials (8 bytes per row and warp slice) share the statistics'
     // space when they fit, else get their own
     int S = 1, vps = 0;
-    accept_slices(c, sms, &S, &vps);
+    greedy_slices(c, sms, &S, &vps);
     const size_t gbytes = 8 * T * S;
     L.row_parts = gbytes <= sizeof(SlicePart) * T * sh.sslices ? L.sparts : take(gbytes);
   }
@@ -344,7 +355,7 @@ AcceptParams accept_params(const wisp_accept_args *c, void *ws, const Layout &L,
   ap.ntiles = sh.ntiles;
   ap.tiles = at<TileRec>(ws, L.tiles);
   ap.total_rows = c->total_q_rows;
-  accept_slices(c, sms, &ap.slices, &ap.vps);
+  greedy_slices(c, sms, &ap.slices, &ap.vps);
   ap.parts = at<void>(ws, L.row_parts);
   ap.row_order = at<int2>(ws, L.row_order);
   ap.row_cnt = at<int32_t>(ws, L.row_cnt);
@@ -475,10 +486,11 @@ wisp_status wisp_verify_accept_greedy(const wisp_accept_args *acc, void *ws, siz
   const Layout L = make_layout(nullptr, acc, sms);
   if ((st = check_ws(ws, ws_bytes, L)) != WISP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if ((st = launch_plan(nullptr, acc, ws, L, sms, false, s)) != WISP_OK) return st;
+  const bool lm = greedy_level_major(acc);
+  if ((st = launch_plan(nullptr, acc, ws, L, sms, lm, s)) != WISP_OK) return st;
   if (acc->B == 0) return WISP_OK;
   const AcceptParams ap = accept_params(acc, ws, L, sms);
-  return accept_greedy_launch(ap, acc->logits_dtype == WISP_BF16, s) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
+  return accept_greedy_launch(ap, acc->logits_dtype == WISP_BF16, lm, sms, s) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
 }
 
 wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args *acc, void *ws, size_t ws_bytes,

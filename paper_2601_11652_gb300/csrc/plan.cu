@@ -55,79 +55,66 @@ __device__ __forceinline__ int64_t ceil_div(int64_t a, int64_t b) {
 // of a request is then usually known before its row i + 1 comes up, and the acceptance kernel skips
 // rows past a rejection.  Also clears the per-row and per-request state of the launch and gives the
 // requests this planner refused -1 outputs.
-__device__ void plan_accept(const PlanParams &p) {
-  constexpr int KB = kMaxDraft + 1;  // draft lengths 0..kMaxDraft
-  __shared__ int32_t s_n[KB + 1];    // level sizes n_i = #{valid r : k_r >= i}, then cursors
-  __shared__ int32_t s_ls[KB + 1];   // level starts
-  __shared__ int s_w[2][32];
+// The caller has cleared sh.n and sh.nvalid before a barrier; one: at most kThreads requests, thread r holds
+// request r's k and whether it is valid.
+struct AcceptPlan {
+  static constexpr int KB = kMaxDraft + 1;  // draft lengths 0..kMaxDraft
+  int32_t n[2 * kThreads];                  // histogram of k, then the buckets' cursors
+  int32_t ls[2 * kThreads];                 // level starts
+  int w[2][32];
+  int32_t nvalid;
+};
+static_assert(AcceptPlan::KB + 1 <= 2 * kThreads, "two buckets per thread");
+
+__device__ __forceinline__ void plan_accept_clear(AcceptPlan &sh) {
+  sh.n[threadIdx.x] = sh.n[threadIdx.x + kThreads] = 0;
+  if (threadIdx.x == 0) sh.nvalid = 0;
+}
+
+__device__ void plan_accept(const PlanParams &p, AcceptPlan &sh, bool one, int my_k, bool my_ok) {
   const int tid = threadIdx.x;
-  __syncthreads();  // pass 1's flags and offsets are visible to every thread
-  for (int b = tid; b <= KB; b += kThreads) s_n[b] = 0;
-  __syncthreads();
   int nv = 0;
   for (int r = tid; r < p.B; r += kThreads) {
     p.req_rej[r] = INT32_MAX;
     p.req_claim[r] = 0;
     p.req_dcnt[r] = 0;
     p.queue[r] = -1;
-    if (p.req_flag[r] == REQ_OK) {
-      atomicAdd(&s_n[p.draft_lens[r]], 1);  // histogram of k
+    if (one ? my_ok : p.req_flag[r] == REQ_OK) {
+      atomicAdd(&sh.n[one ? my_k : p.draft_lens[r]], 1);  // histogram of k
       ++nv;
     } else {
       p.accepted_len[r] = -1;
       p.next_token[r] = -1;
     }
   }
+  // valid requests: a warp sum per warp, added into a shared counter
+  nv = __reduce_add_sync(0xffffffffu, nv);
+  if ((tid & 31) == 0 && nv) atomicAdd(&sh.nvalid, nv);
   for (int64_t j = tid; j < p.total_q_rows; j += kThreads) {
     p.row_cnt[j] = 0;
     p.row_code[j] = 0;
   }
-  // valid requests: a warp sum per warp, added into a shared counter
-  __shared__ int32_t s_nvalid;
-  if (tid == 0) s_nvalid = 0;
-  __syncthreads();
-  nv = __reduce_add_sync(0xffffffffu, nv);
-  if ((tid & 31) == 0 && nv) atomicAdd(&s_nvalid, nv);
-  static_assert(KB + 1 <= 2 * kThreads, "two histogram buckets per thread");
-  // n_i: suffix sums of the histogram (buckets in decreasing order, two per thread)
-  {
-    const int b0 = KB - 1 - 2 * tid, b1 = b0 - 1;
-    const int h0 = b0 >= 0 ? s_n[b0] : 0, h1 = b1 >= 0 ? s_n[b1] : 0;
-    int tot;
-    const int incl = block_scan(h0 + h1, s_w[0], &tot);
-    if (b0 >= 0) s_n[b0] = incl - h1;
-    if (b1 >= 0) s_n[b1] = incl;
-  }
-  if (tid == 0) s_n[KB] = 0;
-  __syncthreads();
-  const int nvalid = s_nvalid;
-  // level starts: exclusive prefix sums of n_i (two per thread)
-  int rows_valid;
-  {
-    const int b0 = 2 * tid, b1 = b0 + 1;
-    const int c0 = b0 <= KB ? s_n[b0] : 0, c1 = b1 <= KB ? s_n[b1] : 0;
-    const int incl = block_scan(c0 + c1, s_w[1], &rows_valid);
-    if (b0 <= KB) s_ls[b0] = incl - c0 - c1;
-    if (b1 <= KB) s_ls[b1] = incl - c1;
+  for (int j = tid; j < kTabCacheSlots; j += kThreads) {
+    p.acc_ctr->tab_state[j] = 0;
+    p.acc_ctr->tab_m[j] = 0;
   }
   __syncthreads();
-  // cursors: in every level, the requests with a larger k come first; bucket k starts at n_{k+1}
-  int32_t nxt[2];
-  for (int j = 0; j < 2; ++j) {
-    const int b = j * kThreads + tid;
-    nxt[j] = b < KB ? s_n[b + 1] : 0;
-  }
-  __syncthreads();
-  for (int j = 0; j < 2; ++j) {
-    const int b = j * kThreads + tid;
-    if (b < KB) s_n[b] = nxt[j];
-  }
+  // per bucket b (two per thread): level size n_b = #{k >= b}, its start (the sum of the levels before), and
+  // the bucket's cursor n_{b+1} (in every level the requests with a larger k come first)
+  const int nvalid = sh.nvalid, h0 = sh.n[2 * tid], h1 = sh.n[2 * tid + 1];
+  int tot, rows_valid;
+  const int n0 = nvalid - (block_scan(h0 + h1, sh.w[0], &tot) - h0 - h1), n1 = n0 - h0;
+  const int l0 = block_scan(n0 + n1, sh.w[1], &rows_valid) - n0 - n1;
+  sh.ls[2 * tid] = l0;
+  sh.ls[2 * tid + 1] = l0 + n0;
+  sh.n[2 * tid] = n0 - h0;
+  sh.n[2 * tid + 1] = n1 - h1;
   __syncthreads();
   for (int r = tid; r < p.B; r += kThreads) {
-    if (p.req_flag[r] != REQ_OK) continue;
-    const int k = p.draft_lens[r];
-    const int pos = atomicAdd(&s_n[k], 1);
-    for (int i = 0; i <= k; ++i) p.row_order[s_ls[i] + pos] = make_int2(r, i);
+    if (!(one ? my_ok : p.req_flag[r] == REQ_OK)) continue;
+    const int k = one ? my_k : p.draft_lens[r];
+    const int pos = atomicAdd(&sh.n[k], 1);
+    for (int i = 0; i <= k; ++i) p.row_order[sh.ls[i] + pos] = make_int2(r, i);
   }
   if (tid == 0) {
     p.acc_ctr->n_items = rows_valid * p.sslices;
@@ -137,10 +124,6 @@ __device__ void plan_accept(const PlanParams &p) {
     p.acc_ctr->n_claimed = 0;
     p.acc_ctr->stats_next = 0;
   }
-  for (int j = tid; j < kTabCacheSlots; j += kThreads) {
-    p.acc_ctr->tab_state[j] = 0;
-    p.acc_ctr->tab_m[j] = 0;
-  }
 }
 
 }  // namespace
@@ -149,7 +132,7 @@ __device__ void plan_accept(const PlanParams &p) {
 // each, each item's bucket kept from the pass that writes it, and no 64-bit division where 32 bits hold the
 // operands.  With 64-bit scans of three barriers, separate passes and a binary search per pass, one request
 // took 9.7 us here and 256 requests 18.4 us (cold caches, launch included); now 8.6 and 15 us.
-__global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
+__global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // a kernel launched after this one with programmatic stream serialization (the attention) may
   // start its own set-up now; it reads the plan only after waiting for this grid to complete
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -158,7 +141,16 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
   __shared__ unsigned long long s_sum[2];  // keys of the valid requests; KV tiles of the items
   __shared__ int32_t s_valid;
   __shared__ int32_t s_hist[kOrderBuckets];
+  // the attention's per-request arrays (pass 3) come after the acceptance part is done with its own
+  union Shared {
+    AcceptPlan acc;
+    struct {
+      int32_t first[kThreads + 1], rows[kThreads], ch[kThreads], pf[kThreads], ctx[kThreads], q0[kThreads], nn[kThreads];
+    } att;
+  };
+  __shared__ Shared sh;
   const int tid = threadIdx.x, lane = tid & 31;
+  if (p.with_accept && !p.accept_apart) plan_accept_clear(sh.acc);
   // the launch's status word starts clear (every kernel of the call reports into it)
   if (tid == 0) {
     p.status->code = 0;
@@ -240,7 +232,7 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
       atomicCAS(&p.status->code, 0, (int32_t)WISP_DEV_BAD_LENGTH);
     }
   }
-  if (p.with_accept && !p.accept_apart) plan_accept(p);
+  if (p.with_accept && !p.accept_apart) plan_accept(p, sh.acc, one, my_k, my_ok);
   if (!p.with_attention) return;
   __syncthreads();
 
@@ -264,10 +256,10 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
   // (block scans), then the chunk's items are written by consecutive threads (item i by thread
   // i mod kThreads, its request found by binary search over the chunk's first items), so that the stores
   // coalesce.
-  __shared__ int32_t s_first[kThreads + 1];  // the chunk's requests' first items, relative
+  int32_t *s_first = sh.att.first;  // the chunk's requests' first items, relative
   // per request of the chunk: query rows, chunks (0: no items), first partial, context, first
   // query row, keys
-  __shared__ int32_t s_rows[kThreads], s_ch[kThreads], s_pf[kThreads], s_ctx[kThreads], s_q0[kThreads], s_nn[kThreads];
+  int32_t *s_rows = sh.att.rows, *s_ch = sh.att.ch, *s_pf = sh.att.pf, *s_ctx = sh.att.ctx, *s_q0 = sh.att.q0, *s_nn = sh.att.nn;
   auto bucket_of = [&](int tokens) -> int {  // bucket 0: the longest
     return kOrderBuckets - 1 - min((tokens + kOrderTile - 1) / kOrderTile, kOrderBuckets - 1);
   };
@@ -439,8 +431,15 @@ __global__ void __launch_bounds__(kThreads) plan_kernel(const PlanParams p) {
 // The acceptance part of the plan on its own (a step: it runs on the acceptance pass's stream, so
 // that the attention, which waits for the whole planner grid, does not wait for it).  Reads what
 // plan_kernel's first pass wrote (flags and offsets).
-__global__ void __launch_bounds__(kThreads) plan_accept_kernel(const PlanParams p) {
-  plan_accept(p);
+__global__ void __launch_bounds__(kThreads, 1) plan_accept_kernel(const PlanParams p) {
+  __shared__ AcceptPlan sh;
+  plan_accept_clear(sh);
+  const int r = threadIdx.x;
+  const bool one = p.B <= kThreads, mine = one && r < p.B;
+  const int k = mine ? p.draft_lens[r] : 0;
+  const bool ok = mine && p.req_flag[r] == REQ_OK;
+  __syncthreads();
+  plan_accept(p, sh, one, k, ok);
 }
 
 }  // namespace wisp
