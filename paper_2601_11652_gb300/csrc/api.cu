@@ -207,11 +207,9 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
     L.row_groups = kMaxRowsPerHead / (a->qkv_dtype == WISP_BF16 ? kTcRowsPerItem : kF32RowsPerItem);
     L.max_items = L.row_groups * ((int64_t)L.target_items + (int64_t)B * a->Hkv);
     L.partial_cap = (int64_t)2 * L.target_items * (kMaxRowsPerHead * (a->D + 2) + 4 * L.row_groups);
-    L.req_item_begin = take(sizeof(int32_t) * (size_t)B);
     L.req_chunks = take(sizeof(int32_t) * (size_t)B);
     L.pair_done = take(sizeof(int32_t) * (size_t)B * a->Hkv * L.row_groups);
     L.items = take(sizeof(WorkItem) * (size_t)L.max_items);
-    L.order = take(sizeof(int32_t) * (size_t)L.max_items);
     L.partials = take(sizeof(float) * (size_t)L.partial_cap);
   }
   if (c && c->B > 0) {
@@ -276,11 +274,9 @@ PlanParams plan_params(const wisp_attn_args *a, const wisp_accept_args *c, void 
     pp.kv_f32 = a->qkv_dtype == WISP_F32;
     pp.max_items = L.max_items;
     pp.partial_cap = L.partial_cap;
-    pp.req_item_begin = at<int32_t>(ws, L.req_item_begin);
     pp.req_chunks = at<int32_t>(ws, L.req_chunks);
     pp.pair_done = at<int32_t>(ws, L.pair_done);
     pp.items = at<WorkItem>(ws, L.items);
-    pp.order = at<int32_t>(ws, L.order);
   } else {
     pp.Hq = pp.Hkv = 1;
   }
@@ -320,12 +316,10 @@ wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L,
   ap.out = a->out;
   ap.status = at<DeviceStatus>(ws, L.status);
   ap.req_flag = at<int32_t>(ws, L.req_flag);
-  ap.req_item_begin = at<int32_t>(ws, L.req_item_begin);
   ap.req_chunks = at<int32_t>(ws, L.req_chunks);
   ap.header = at<PlanHeader>(ws, L.plan_header);
   ap.header_mut = at<PlanHeader>(ws, L.plan_header);
   ap.items = at<WorkItem>(ws, L.items);
-  ap.order = at<int32_t>(ws, L.order);
   ap.partials = at<float>(ws, L.partials);
   ap.pair_done = at<int32_t>(ws, L.pair_done);
   ap.row_groups = L.row_groups;

@@ -12,11 +12,10 @@ struct AttnParams {
   const void *q, *k_cache, *v_cache;
   void *out;
   DeviceStatus *status;
-  const int32_t *req_flag, *req_item_begin, *req_chunks;
+  const int32_t *req_flag, *req_chunks;
   const PlanHeader *header;
   PlanHeader *header_mut;  // same object: the work counter
-  const WorkItem *items;
-  const int32_t *order;  // dispatch order of the persistent kernel: item index per counter value
+  const WorkItem *items;  // in dispatch order
   float *partials;
   int row_groups;      // row groups per (request, head) at most
   int32_t *pair_done;  // [B * Hkv * row_groups] finished chunks of each split (request, head, row group), zeroed

@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_f32_kernel(const __grid_cons
       int it;
       do {
         it = atomicAdd(&p.header_mut->next_item, 1);
-        it = it < n_items ? p.order[it] : -1;
-      } while (it >= 0 && p.req_flag[p.items[it].r] != REQ_OK);
+        if (it >= n_items) it = -1;
+      } while (it >= 0 && p.items[it].t1 <= p.items[it].t0);  // (a refused request's items are empty)
       sh.item = it;
     }
     __syncthreads();  // (also: the previous item's shared memory is no longer read)

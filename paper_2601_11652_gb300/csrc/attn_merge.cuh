@@ -50,16 +50,15 @@ __device__ __forceinline__ void st_cols(float *dst, const float (&v)[CPL], float
 template <int D, typename T>
 __device__ __forceinline__ void merge_chunks(const AttnParams &p, const WorkItem &w, int g, int chunks, int wq, int nw) {
   const int lane = threadIdx.x & 31;
-  const WorkItem *ci = p.items + p.req_item_begin[w.r] + (w.h * w.nrg + w.rg) * chunks;
-  const float *base = p.partials + ci[0].poff;
-  const int64_t stride = ci[1].poff - ci[0].poff;
+  const float *base = p.partials + w.pbase;
+  const int stride = ((w.rg ? w.row0 / w.rg : w.rows) * (D + 2) + 3) / 4 * 4;  // (groups before the last have equal rows)
   constexpr int CPL = D / 32;  // columns per lane
   T *og = static_cast<T *>(p.out);
   for (int j0 = 2 * wq; j0 < w.rows; j0 += 2 * nw) {
     const int j1 = min(j0 + 1, w.rows - 1);  // an odd last row is merged twice, alike
     float m0 = -INFINITY, m1 = -INFINITY;
     for (int c = lane; c < chunks; c += 32) {
-      const float *pm = base + c * stride + w.rows * D;
+      const float *pm = base + (int64_t)c * stride + w.rows * D;
       m0 = fmaxf(m0, __ldcg(pm + j0));
       m1 = fmaxf(m1, __ldcg(pm + j1));
     }
@@ -74,7 +73,7 @@ __device__ __forceinline__ void merge_chunks(const AttnParams &p, const WorkItem
     for (int c0 = 0; c0 < chunks; c0 += 32) {
       float w0 = 0.0f, w1 = 0.0f;  // lane: chunk c0 + lane
       if (c0 + lane < chunks) {
-        const float *pm = base + (c0 + lane) * stride + w.rows * D;
+        const float *pm = base + (int64_t)(c0 + lane) * stride + w.rows * D;
         const float mc0 = __ldcg(pm + j0), mc1 = __ldcg(pm + j1);
         w0 = mc0 == -INFINITY ? 0.0f : ptx::ex2(mc0 - m0);
         w1 = mc1 == -INFINITY ? 0.0f : ptx::ex2(mc1 - m1);
@@ -87,7 +86,7 @@ __device__ __forceinline__ void merge_chunks(const AttnParams &p, const WorkItem
         float v0[4][CPL], v1[4][CPL];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const float *po = base + (c0 + min(c + u, nc - 1)) * stride + lane * CPL;
+          const float *po = base + (int64_t)(c0 + min(c + u, nc - 1)) * stride + lane * CPL;
           ld_cols<CPL>(po + (int64_t)j0 * D, v0[u]);
           ld_cols<CPL>(po + (int64_t)j1 * D, v1[u]);
         }

@@ -12,10 +12,10 @@
 //
 // Persistent CTAs (one per SM) take work items (request, KV head, key chunk, row group) from a
 // global counter, in the planner's longest-first order.  Warp roles in a CTA:
-//   * warp 2 (item loader) takes the next item just in time (when the K producer is three tiles
-//     from the end of the current one), publishes it to the other warps through a 4-slot shared
-//     ring, and copies its query rows into one of two shared Q buffers (128-byte-swizzled,
-//     K-major: the B operand of S^T);
+//   * warp 2 takes the next item just in time (when the K producer is three tiles from the end of what
+//     is published) and publishes it to the other warps through a 4-slot shared ring;
+//   * warp 17 copies an item's query rows into one of two shared Q buffers (128-byte-swizzled, K-major:
+//     the B operand of S^T);
 //   * warps 0 and 3 (K and V producers) stream the item's K and V tiles of 128 tokens with TMA
 //     tiled loads into two rings: one 16 KB box per 64-wide half of the head dim when the tile's
 //     eight 16-token blocks are consecutive in the pool, else one 2 KB box per block; blocks past
@@ -37,7 +37,9 @@
 // (read S^T, P, publish): 0.80 us a 128-key tile at 4 query rows and 1.06 us at 64 with K and V in L2,
 // against the 1.47 us that a tile's 64 KB take at an SM's share of the copy rate (D = 128).  With one
 // thread issuing both products, a vote of the softmax warps per tile and the barrier pointers in local
-// memory those were 1.42 and 1.78 us.
+// memory those were 1.42 and 1.78 us.  An item of one tile takes 4 us (its claim, Q copy, first-tile
+// references and epilogue overlap its neighbours'); with a division per query row in the Q copy and the
+// epilogue, and one warp for claims and Q, 7.5 us.
 //
 // Every mbarrier wait is bounded in time; an expired wait records WISP_DEV_TIMEOUT and the CTA
 // drains.  No named barrier is used: a warp that gives up cannot leave the others blocked, and the
@@ -58,7 +60,7 @@ constexpr int kBT = 128;            // KV tokens per tile (the M of S^T)
 constexpr int kNR = kTcRowsPerItem; // query rows per item at most (64: the planner cuts larger sets)
 constexpr int kThreads = 640;       // warps 0-3 K producer, S^T issuer, item loader and V producer; 4-7 softmax
                                     // (first half of the rows); 8-11 epilogue; 12-15 softmax (second half);
-                                    // 16 PV issuer (17-19 have no work: registers are allotted per four warps)
+                                    // 16 PV issuer; 17 Q loader (18, 19: registers are allotted per four warps)
 constexpr int kSoftmaxWarps = 8;
 constexpr uint32_t kTmemCols = 256; // S^T[2] at columns 0 / 64, O^T[2] at 128 / 192
 constexpr long long kWaitCycles = 4000000000LL;  // about two seconds: a wait that long is a failure
@@ -67,6 +69,8 @@ constexpr long long kWaitCycles = 4000000000LL;  // about two seconds: a wait th
 // 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it is
 // computed again by its epilogue warps (item_exact).
 constexpr float kMaxP = 0x1p64f;
+constexpr uint32_t kAhead = 3;      // the item loader takes the next item when the K producer is this many tiles from
+                                    // the end of what is published
 static_assert(kNR == 64, "TMEM and shared-memory layout assume 64 rows per item");
 
 template <int D>
@@ -87,7 +91,7 @@ struct Cfg {
   static constexpr int OFF_V = OFF_K + NSK * KV_TILE;
   static constexpr int OFF_P = OFF_V + NSV * KV_TILE;
   static constexpr int OFF_BAR = OFF_P + NP * P_BYTES;
-  static constexpr int N_BAR = 2 * NSK + 2 * NSV + 8 + 2 * NP + 6 + 1 + 2 * RING + 5;
+  static constexpr int N_BAR = 2 * NSK + 2 * NSV + 8 + 2 * NP + 6 + 1 + 2 * RING + 4;
   static constexpr int OFF_MW = (OFF_BAR + N_BAR * 8 + 15) / 16 * 16;  // float [8][32] per warp: minus the rows' references
   static constexpr int OFF_RED = OFF_MW + kSoftmaxWarps * 32 * 4;      // float [2][4][64] first-tile maxima per quadrant
   static constexpr int OFF_HL = OFF_RED + 2 * 4 * kNR * 4;             // float [2][4][64] row-sum shares per quadrant
@@ -118,8 +122,7 @@ struct Bars {
   static constexpr int EGRP = IT_EMPTY + C::RING; // the epilogue warps
   static constexpr int RED = EGRP + 1;            // [2] per softmax group: its four warps, once per item (first-tile maxima)
   static constexpr int FIN = RED + 2;             // every warp, once: its last access to TMEM is done
-  static constexpr int CLAIM = FIN + 1;           // the K producer, once per item, a few tiles before the item's end
-  static_assert(CLAIM + 1 <= C::N_BAR, "barrier count");
+  static_assert(FIN + 1 <= C::N_BAR, "barrier count");
   __device__ __forceinline__ uint32_t k_full(int i) const { return at(K_FULL + i); }
   __device__ __forceinline__ uint32_t k_empty(int i) const { return at(K_EMPTY + i); }
   __device__ __forceinline__ uint32_t v_full(int i) const { return at(V_FULL + i); }
@@ -139,7 +142,6 @@ struct Bars {
   __device__ __forceinline__ uint32_t mma_done() const { return at(MMA_DONE); }
   __device__ __forceinline__ uint32_t egrp() const { return at(EGRP); }
   __device__ __forceinline__ uint32_t fin() const { return at(FIN); }
-  __device__ __forceinline__ uint32_t claim() const { return at(CLAIM); }
 };
 
 __device__ __forceinline__ bool wait_bar(uint32_t b, uint32_t parity, volatile int *abort) {
@@ -156,7 +158,8 @@ __device__ __forceinline__ bool wait_bar(uint32_t b, uint32_t parity, volatile i
 }
 
 __device__ __forceinline__ bool item_ok(const AttnParams &p, const WorkItem &w) {
-  return w.r >= 0 && w.r < p.B && p.req_flag[w.r] == REQ_OK && w.t1 > w.t0 && w.rows > 0 && w.rows <= kNR &&
+  // (a refused request's items are empty)
+  return w.r >= 0 && w.r < p.B && w.t1 > w.t0 && w.rows > 0 && w.rows <= kNR &&
          w.row0 >= 0 && w.nrg >= 1 && w.nrg <= p.row_groups && w.rg >= 0 && w.rg < w.nrg;
 }
 
@@ -282,6 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + C::OFF_MISC);
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 4);
   volatile int *s_last = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 8);
+  volatile uint32_t *s_issued = reinterpret_cast<volatile uint32_t *>(smem + C::OFF_MISC + 12);  // K tiles issued
   volatile int *s_ovf = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 16);  // [2] per O buffer: P past kMaxP
   struct RingSlot {
     int it;
@@ -319,13 +323,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::mbar_init(B.mma_done(), 2);  // the two MMA issuers
     for (int i = 0; i < C::RING; ++i) {
       ptx::mbar_init(B.it_full(i), 1);
-      ptx::mbar_init(B.it_empty(i), 4 + kSoftmaxWarps + 4);  // KV producers, MMA issuers, softmax and epilogue warps
+      ptx::mbar_init(B.it_empty(i), 5 + kSoftmaxWarps + 4);  // KV producers, MMA issuers, Q loader, softmax and epilogue warps
     }
     ptx::mbar_init(B.egrp(), 4);      // the four epilogue warps
     ptx::mbar_init(B.red(0), 4);
     ptx::mbar_init(B.red(1), 4);
     ptx::mbar_init(B.fin(), kThreads / 32);
-    ptx::mbar_init(B.claim(), 1);
+    *s_issued = 0;
     *s_abort = 0;
     s_ovf[0] = s_ovf[1] = 0;
     ptx::fence_mbar_init();
@@ -356,6 +360,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
   const int g = p.Hq / p.Hkv;
+  // a query row's position and head: row / g for rows below 128 as a product (exact: 127 (g - 1) < 2^16)
+  const unsigned gm = (65536u + g - 1) / g;
+  auto div_g = [&](int row) -> int { return (int)(((unsigned)row * gm) >> 16); };
 
   if (warp == 0 || warp == 3) {
     // ------------------------------------------------------------------ K / V producers
@@ -386,11 +393,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       int cur = fetch(0), nxt = fetch(32);  // block ids of tiles t..t+3 and t+4..t+7
       const int ntiles = (w.t1 - w.t0 + kBT - 1) / kBT;
-      const int t_claim = ntiles > 3 ? ntiles - 3 : 0;
       for (int t = 0; t < ntiles; ++t, ++tile_n) {
-        // a few tiles before this item's end the loader may take the next one (items are taken
-        // just in time, so the work counter balances the CTAs to the end)
-        if (is_k && t == t_claim && lane == 0) ptx::mbar_arrive(B.claim());
+        if (is_k && lane == 0) *s_issued = tile_n;
         if (t > 0 && (t & 3) == 0) {
           cur = nxt;
           nxt = fetch(32 * ((t >> 2) + 1));
@@ -437,36 +441,63 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ item loader
-    int li = 0;
+    uint32_t published = 0;  // tiles of the items published so far
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
-      // next valid work item: publish it to the other warps, then load its query rows.  Item j is
-      // taken once the K producer is near the end of item j - 1 (the claim barrier completes once
-      // per item, and the producer cannot pass item j - 1 before item j is published: the parity
-      // is exact).
+      // next valid work item: publish it to the other warps.  Items are taken just in time, so the work
+      // counter balances the CTAs to the end, but early enough to hide the way from the claim to the first
+      // load: when the K producer is kAhead tiles from the end of what is published, which for items of
+      // a tile or two means several items ahead.
       const int slot = j % C::RING;
-      if (j > 0 && !wait_bar(B.claim(), (j - 1) & 1, s_abort)) { ok = false; break; }
+      for (const long long g0 = clock64(); published > *s_issued + kAhead;) {
+        if (*s_abort || clock64() - g0 > kWaitCycles) {
+          *s_abort = 1;
+          ok = false;
+          break;
+        }
+        __nanosleep(100);
+      }
+      if (!ok) break;
       if (!wait_bar(B.it_empty(slot), ((j / C::RING) & 1) ^ 1, s_abort)) { ok = false; break; }
-      int it = -1;
+      int tiles = 0;
       if (lane == 0) {
-        while (true) {
+        int it;
+        WorkItem w;
+        do {
           it = atomicAdd(&p.header_mut->next_item, 1);
           if (it >= n_items) { it = -1; break; }
-          it = p.order[it];
-          if (item_ok(p, p.items[it])) break;
-        }
+          w = p.items[it];
+        } while (!item_ok(p, w));
         s_ring[slot].it = it;
-        if (it >= 0) s_ring[slot].w = p.items[it];
+        if (it >= 0) {
+          s_ring[slot].w = w;
+          tiles = (w.t1 - w.t0 + kBT - 1) / kBT;
+        }
         ptx::mbar_arrive(B.it_full(slot));
       }
-      it = __shfl_sync(0xffffffffu, it, 0);
-      if (it < 0) {
+      tiles = __shfl_sync(0xffffffffu, tiles, 0);
+      if (tiles == 0) {
         // no item left for this CTA: a kernel launched after this one as a programmatic
-        // dependent (the acceptance walk) may be scheduled; it still waits for this grid to finish
+        // dependent may be scheduled; it still waits for this grid to finish
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
         break;
       }
-      const WorkItem w = p.items[it];
+      published += tiles;
+    }
+    if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
+  } else if (warp == 17) {
+    // ------------------------------------------------------------------ Q loader
+    // (a warp of its own: claiming an item and copying its rows in turn took 7.5 us, which bounded short items)
+    int li = 0;
+    bool ok = true;
+    for (uint32_t j = 0; ok; ++j) {
+      const int slot = j % C::RING;
+      if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
+      const int it = s_ring[slot].it;
+      const WorkItem w = s_ring[slot].w;
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
+      if (it < 0) break;
       const int qb = li % C::NQ;
       if (!wait_bar(B.q_empty(qb), ((li / C::NQ) & 1) ^ 1, s_abort)) { ok = false; break; }
       ++li;
@@ -475,28 +506,26 @@ __global__ void __launch_bounds__(kThreads, 1)
       // MMA's N only feed S^T columns that the softmax masks.
       const uint16_t *qg = static_cast<const uint16_t *>(p.q);
       uint8_t *qs = smem + C::OFF_Q + qb * C::Q_BYTES;
-      constexpr int CPR = D / 8;  // 16-byte chunks per row
+      constexpr int CPR = D / 8;       // 16-byte chunks per row: a lane keeps its chunk of every row it copies
+      constexpr int RPI = 32 / CPR;    // rows per warp load
       constexpr int QBATCH = 8;
-      const int nchunks = w.rows * CPR;
-      for (int base = 0; base < nchunks; base += 32 * QBATCH) {
+      const int cc = lane % CPR;
+      const uint16_t *qi = qg + ((int64_t)w.q0 * p.Hq + w.h * g) * D + cc * 8;
+      for (int base = lane / CPR; base < w.rows; base += RPI * QBATCH) {
         uint4 v[QBATCH];
 #pragma unroll
         for (int u = 0; u < QBATCH; ++u) {
-          const int c = base + u * 32 + lane;
-          if (c < nchunks) {
-            const int row = c / CPR, cc = c % CPR;
-            const int rj = w.row0 + row;
-            const int jj = rj / g, hh = rj % g;
-            v[u] = __ldg(reinterpret_cast<const uint4 *>(qg + ((int64_t)(w.q0 + jj) * p.Hq + w.h * g + hh) * D) + cc);
+          const int row = base + u * RPI;
+          if (row < w.rows) {
+            const int rj = w.row0 + row, jj = div_g(rj), hh = rj - jj * g;
+            v[u] = __ldg(reinterpret_cast<const uint4 *>(qi + (int64_t)(jj * p.Hq + hh) * D));
           }
         }
 #pragma unroll
         for (int u = 0; u < QBATCH; ++u) {
-          const int c = base + u * 32 + lane;
-          if (c < nchunks) {
-            const int row = c / CPR, cc = c % CPR;
+          const int row = base + u * RPI;
+          if (row < w.rows)
             *reinterpret_cast<uint4 *>(qs + (cc >> 3) * C::QHALF + row * 128 + (((cc & 7) ^ (row & 7)) << 4)) = v[u];
-          }
         }
       }
       ptx::fence_proxy_async_smem();
@@ -641,15 +670,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float lsum = hl[jl] + hl[kNR + jl] + hl[2 * kNR + jl] + hl[3 * kNR + jl];
         if (w.poff < 0) {
           const float linv = 1.0f / lsum;
-          uint16_t *og = static_cast<uint16_t *>(p.out);
+          // (row pointers stepped from row to row: with a division per row, the epilogue took 5-7 us an item and
+          // bounded items of a few tiles)
+          int hh = w.row0 + 32 * c - div_g(w.row0 + 32 * c) * g;
+          uint16_t *og = static_cast<uint16_t *>(p.out) +
+                         ((int64_t)(w.q0 + div_g(w.row0 + 32 * c)) * p.Hq + w.h * g + hh) * D + d;
+          const int wrap = (p.Hq - g + 1) * D;  // from a position's last head to the next one's first
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int jr = 32 * c + i;
-            const float inv = __shfl_sync(0xffffffffu, linv, i);
-            if (jr < w.rows && dval) {
-              const int rj = w.row0 + jr, jq = rj / g, hh = rj % g;
-              const float o = __uint_as_float(x[i]) * inv;
-              og[((int64_t)(w.q0 + jq) * p.Hq + w.h * g + hh) * D + d] = __bfloat16_as_ushort(__float2bfloat16_rn(o));
+          for (int i0 = 0; i0 < 32; i0 += 8) {
+            if (32 * c + i0 >= w.rows) break;
+#pragma unroll
+            for (int i = i0; i < i0 + 8; ++i) {
+              const float inv = __shfl_sync(0xffffffffu, linv, i);
+              if (32 * c + i < w.rows && dval) *og = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(x[i]) * inv));
+              const bool last_head = hh == g - 1;
+              og += last_head ? wrap : D;
+              hh = last_head ? 0 : hh + 1;
             }
           }
         } else {

@@ -251,11 +251,13 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   chunk = max64(chunk, kMinChunk);
   chunk = min64((chunk + kChunkAlign - 1) / kChunkAlign * kChunkAlign, (int64_t)1 << 30);  // (a sequence is shorter)
 
-  // pass 3: items and partial slots (request-major, then KV head, then row group, then chunk), and the
-  // histogram of their lengths.  Per chunk of kThreads requests: one thread per request sizes its items
-  // (block scans), then the chunk's items are written by consecutive threads (item i by thread
-  // i mod kThreads, its request found by binary search over the chunk's first items), so that the stores
-  // coalesce.
+  // pass 3: the requests' items and partial slots (request-major, then KV head, then row group, then chunk)
+  // and the histogram of the items' lengths; pass 4: the items, each written at its place in the dispatch
+  // order, longest first (counting sort on the tile count), so that the persistent kernel ends with its
+  // shortest items and its CTAs finish close together.  Per chunk of kThreads requests: one thread per
+  // request sizes its items (block scans into shared arrays), then consecutive threads take consecutive
+  // items (the request found by binary search over the chunk's first items).  With one chunk of requests
+  // pass 4 finds the shared arrays as pass 3 left them and its items' requests and buckets in registers.
   int32_t *s_first = sh.att.first;  // the chunk's requests' first items, relative
   // per request of the chunk: query rows, chunks (0: no items), first partial, context, first
   // query row, keys
@@ -264,11 +266,8 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     return kOrderBuckets - 1 - min((tokens + kOrderTile - 1) / kOrderTile, kOrderBuckets - 1);
   };
   int64_t item_carry = 0, poff_carry = 0;
-  int keep[kKeep];
-#pragma unroll
-  for (int x = 0; x < kKeep; ++x) keep[x] = 0;
-  unsigned long long my_tiles = 0;  // KV tiles (kOrderTile tokens) of this thread's items
-  for (int base = 0; base < p.B; base += kThreads) {
+  int ti = 0;  // items of the chunk of requests
+  auto size_requests = [&](int base, bool refuse) {
     const int r = base + tid;
     int n = 0, chunks = 0, rows = 0, nrg = 1, rows0 = 0, ctx_r = 0;
     if (r < p.B && (one ? my_ok : p.req_flag[r] == REQ_OK)) {
@@ -284,20 +283,17 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     // each split item's partials start on a 16-byte boundary (vector stores)
     const int slot = (rows0 * (p.D + 2) + 3) / 4 * 4;
     const int pfl = chunks > 1 ? nitems * slot : 0;
-    int ti, tp;  // (a batch's items and partials are bounded by max_items and partial_cap: 32 bits hold them)
+    int tp;  // (a batch's items and partials are bounded by max_items and partial_cap: 32 bits hold them)
     const int ii = block_scan(nitems, s_w[3], &ti), ip = block_scan(pfl, s_w[4], &tp);
     bool fits = false;
     if (r < p.B) {
-      const int64_t first = item_carry + ii - nitems;
-      const int64_t pfirst = poff_carry + ip - pfl;
-      fits = first + nitems <= p.max_items && pfirst + pfl <= p.partial_cap;
-      if (!fits && nitems > 0) {
+      fits = item_carry + ii <= p.max_items && poff_carry + ip <= p.partial_cap;
+      if (!fits && nitems > 0 && refuse) {
         // cannot happen with the host's bounds; refuse the request rather than overflow
         p.req_flag[r] = REQ_BAD;
         report(p.status, WISP_DEV_UNSUPPORTED, p.request_ids, r);
       }
-      p.req_item_begin[r] = (int32_t)first;
-      p.req_chunks[r] = fits ? chunks : 0;
+      if (refuse) p.req_chunks[r] = fits ? chunks : 0;
     }
     s_first[tid] = ii - nitems;
     if (tid == kThreads - 1) s_first[kThreads] = ti;
@@ -307,64 +303,53 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     s_ctx[tid] = ctx_r;
     s_q0[tid] = r < p.B ? (one ? my_q0 : p.q_row_start[r]) : 0;
     s_nn[tid] = n;
+    poff_carry += tp;
+    __syncthreads();
+  };
+  auto request_of = [&](int i) -> int {  // the last one whose first item is <= i
+    int lo = 0, hi = kThreads - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (s_first[mid] <= i) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  };
+  // item i's chunk of keys and its bucket (a refused request's items are empty and come last)
+  auto keys_of = [&](int i, int lo, int &t0, int &t1) -> int {
+    const int ch = s_ch[lo];
+    t0 = t1 = 0;
+    if (ch > 0) {
+      const int64_t c = (unsigned)(i - s_first[lo]) % (unsigned)ch;
+      t0 = (int)(c * chunk);
+      t1 = (int)min64(s_nn[lo], (c + 1) * chunk);
+    }
+    return bucket_of(t1 - t0);
+  };
+  int keep[kKeep];  // request and bucket of this thread's first items
+#pragma unroll
+  for (int x = 0; x < kKeep; ++x) keep[x] = 0;
+  unsigned long long my_tiles = 0;  // KV tiles (kOrderTile tokens) of this thread's items
+  for (int base = 0; base < p.B; base += kThreads) {
+    size_requests(base, one);
     // per (request, head, row group) finished-chunk counters of the chunk's requests: zeroed, coalesced
     const int64_t pd0 = (int64_t)base * p.Hkv * p.row_groups;
     const int64_t pd1 = (int64_t)min(p.B, base + kThreads) * p.Hkv * p.row_groups;
     for (int64_t x = pd0 + tid; x < pd1; x += kThreads) p.pair_done[x] = 0;
-    __syncthreads();
     int x = 0;
     for (int i = tid; i < ti; i += kThreads, ++x) {
-      // the request of item i: the last one whose first item is <= i
-      int lo = 0, hi = kThreads - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_first[mid] <= i) lo = mid;
-        else hi = mid - 1;
-      }
-      const int rr = base + lo;
-      const int ch = s_ch[lo];
-      if (item_carry + i >= p.max_items) continue;  // (a request refused for want of room)
-      int bucket = kOrderBuckets - 1;
-      if (ch == 0) {  // a refused request's slot: an empty item, listed last; the kernels skip it
-        WorkItem it = {};
-        it.r = rr;
-        p.items[item_carry + i] = it;
-      } else {
-        const int rws = s_rows[lo];
-        const int ng = (rws + p.max_rows_item - 1) / p.max_rows_item;
-        const int r0 = (rws + ng - 1) / ng;
-        const int j = i - s_first[lo];  // (head, row group, chunk) in that order
-        const int hg = j / ch, c = j - hg * ch;
-        const int h = hg / ng, rg = hg - h * ng;
-        const int slot_r = (r0 * (p.D + 2) + 3) / 4 * 4;
-        WorkItem it;
-        it.r = rr;
-        it.h = h;
-        it.t0 = (int32_t)(c * chunk);
-        it.t1 = (int32_t)min64(s_nn[lo], (c + 1) * chunk);
-        it.row0 = rg * r0;
-        it.rows = min(r0, rws - rg * r0);
-        it.rg = rg;
-        it.nrg = ng;
-        it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)j * slot_r) : -1;
-        it.q0 = s_q0[lo];
-        it.ctx = s_ctx[lo];
-        it.pad = 0;
-        p.items[item_carry + i] = it;
-        bucket = bucket_of(it.t1 - it.t0);
-        my_tiles += (unsigned)(it.t1 - it.t0 + kOrderTile - 1) / kOrderTile;
-      }
+      if (item_carry + i >= p.max_items) break;  // (a request refused for want of room)
+      int t0, t1;
+      const int lo = request_of(i), bucket = keys_of(i, lo, t0, t1);
+      my_tiles += (unsigned)(t1 - t0 + kOrderTile - 1) / kOrderTile;
       atomicAdd(&s_hist[bucket], 1);
 #pragma unroll
       for (int y = 0; y < kKeep; ++y)
-        if (y == x) keep[y] = bucket;
+        if (y == x) keep[y] = lo << 16 | bucket;
     }
     item_carry += ti;
-    poff_carry += tp;
     __syncthreads();  // the shared arrays are rewritten by the next chunk; the histogram is complete after the last
   }
-  // pass 4: dispatch order, longest items first (counting sort on the tile count), so that the
-  // persistent kernel ends with its shortest items and its CTAs finish close together
   const int n_items = (int)min64(item_carry, p.max_items);
   for (int o = 16; o > 0; o >>= 1) my_tiles += __shfl_xor_sync(0xffffffffu, my_tiles, o);
   if (lane == 0 && my_tiles) atomicAdd(&s_sum[1], my_tiles);
@@ -374,31 +359,48 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     s_hist[tid] = block_scan(h, s_w[5], &tot) - h;
   }
   __syncthreads();
-  int x = 0;
-  for (int i = tid; i < n_items; i += kThreads, ++x) {
-    int bucket = 0;
-    if (one && x < kKeep) {
+  item_carry = 0;
+  if (!one) poff_carry = 0;
+  for (int base = 0; base < p.B; base += kThreads) {
+    if (!one) size_requests(base, true);
+    int x = 0;
+    for (int i = tid; i < ti; i += kThreads, ++x) {
+      if (item_carry + i >= p.max_items) break;
+      int lo = -1, bucket = 0;
+      if (one) {
 #pragma unroll
-      for (int y = 0; y < kKeep; ++y)
-        if (y == x) bucket = keep[y];
-    } else if (one) {  // from the shared arrays, which still describe every request
-      int lo = 0, hi = kThreads - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_first[mid] <= i) lo = mid;
-        else hi = mid - 1;
+        for (int y = 0; y < kKeep; ++y)
+          if (y == x) {
+            lo = keep[y] >> 16;
+            bucket = keep[y] & 0xffff;
+          }
       }
-      const int ch = s_ch[lo];
-      bucket = kOrderBuckets - 1;
-      if (ch > 0) {
-        const int64_t t0 = (int64_t)((i - s_first[lo]) % ch) * chunk;
-        bucket = bucket_of((int)(min64(s_nn[lo], t0 + chunk) - t0));
-      }
-    } else {
-      const WorkItem &w = p.items[i];
-      bucket = bucket_of(w.t1 - w.t0);  // (an empty item: the last bucket)
+      if (lo < 0) lo = request_of(i);
+      WorkItem it;
+      const int b = keys_of(i, lo, it.t0, it.t1);
+      if (!one || x >= kKeep) bucket = b;
+      const int ch = max(1, s_ch[lo]);
+      const int rws = s_rows[lo];
+      const int ng = max(1, (rws + p.max_rows_item - 1) / p.max_rows_item);
+      const int r0 = (rws + ng - 1) / ng;
+      const int j = i - s_first[lo];  // (head, row group, chunk) in that order
+      const int hg = j / ch, c = j - hg * ch;
+      const int h = hg / ng, rg = hg - h * ng;
+      const int slot = (r0 * (p.D + 2) + 3) / 4 * 4;
+      it.r = base + lo;
+      it.h = h;
+      it.row0 = rg * r0;
+      it.rows = min(r0, rws - rg * r0);
+      it.rg = rg;
+      it.nrg = ng;
+      it.poff = ch > 1 ? (int32_t)(s_pf[lo] + (int64_t)j * slot) : -1;
+      it.pbase = it.poff - c * slot;
+      it.q0 = s_q0[lo];
+      it.ctx = s_ctx[lo];
+      p.items[atomicAdd(&s_hist[bucket], 1)] = it;
     }
-    p.order[atomicAdd(&s_hist[bucket], 1)] = i;
+    item_carry += ti;
+    if (!one) __syncthreads();  // the shared arrays are rewritten by the next chunk
   }
 
   if (tid == 0) {

@@ -18,7 +18,7 @@ struct alignas(16) WorkItem {  // 48 bytes: written and read as three 16-byte ve
   int32_t row0;   // first query row of the item within its (request, head)
   int32_t rg;     // row group of the item
   int32_t nrg;    // row groups of its (request, head)
-  int32_t pad;
+  int32_t pbase;  // offset of the partials of chunk 0 of its (request, head, row group)
 };
 static_assert(sizeof(WorkItem) == 48, "work item layout");
 
@@ -66,11 +66,9 @@ struct Layout {
   size_t draft_start = 0;     // int32 [B+1]
   size_t req_flag = 0;        // int32 [B]
   size_t plan_header = 0;     // PlanHeader
-  size_t req_item_begin = 0;  // int32 [B]  first item of request r
   size_t req_chunks = 0;      // int32 [B]  chunks per KV head of request r
   size_t pair_done = 0;       // int32 [B * Hkv * row_groups] finished chunks per split (request, head, row group)
-  size_t items = 0;           // WorkItem [max_items]
-  size_t order = 0;           // int32 [max_items]  dispatch order of the items (largest first)
+  size_t items = 0;           // WorkItem [max_items] in dispatch order (longest first)
   size_t partials = 0;        // float [partial_cap]
   // acceptance pass (sampling rule)
   size_t acc_ctr = 0;         // AccCounters
@@ -106,9 +104,8 @@ struct PlanParams {
   DeviceStatus *status;
   int32_t *q_row_start, *draft_start, *req_flag;
   PlanHeader *header;
-  int32_t *req_item_begin, *req_chunks, *pair_done;
+  int32_t *req_chunks, *pair_done;
   WorkItem *items;
-  int32_t *order;
   // acceptance pass: level-major dispatch order of the logit rows and the launch's state
   int with_accept;
   int split_sms;               // 1: the acceptance pass runs beside the attention (one step); the
