@@ -127,9 +127,9 @@ void greedy_slices(const wisp_accept_args *c, int sms, int *slices, int *vps) {
   *slices = (int)((nvec + v - 1) / v);
 }
 
-// Work shape of the acceptance kernel: statistics slices per row (about two items per resident
+// Work shape of the acceptance kernel: statistics slices per row (about one item per resident
 // CTA over the batch's rows: more, smaller items cost more in per-item set-up and bookkeeping than
-// they gain in balance; a slice is a whole number of 3-vector chunks per thread), draw tiles (64 vectors: one warp's share of a draw chunk; no tile records when they
+// they gain in balance: 16 requests 57 us against 62 with two items per CTA, 32 requests 68 against 71; a slice is a whole number of 3-vector chunks per thread), draw tiles (64 vectors: one warp's share of a draw chunk; no tile records when they
 // would exceed tile_budget bytes) and draw slices per row (one item per resident CTA over the batch
 // when it is small, up to two per CTA as it grows; whole chunks of 256 vectors).
 constexpr size_t kTileBudget = (size_t)256 << 20;
@@ -154,7 +154,7 @@ AcceptShape accept_shape(const wisp_accept_args *c, int sms, size_t tile_budget)
     *n = (int)((nvec + v - 1) / v);
   };
   AcceptShape sh;
-  cut(2 * ctas, c->total_q_rows > 0 ? c->total_q_rows : 1, (int64_t)kAcceptThreads * kStatsChunkVecs, &sh.sslices,
+  cut(ctas, c->total_q_rows > 0 ? c->total_q_rows : 1, (int64_t)kAcceptThreads * kStatsChunkVecs, &sh.sslices,
       &sh.svps);
   // a tile is one warp's 64 vectors of a draw chunk; without room for the records, none
   const int64_t nt = (nvec + 63) / 64;
@@ -226,11 +226,11 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
     L.tiles = take(sizeof(TileRec) * ((size_t)c->B * sh.ntiles + 1));
     L.tcache = c->logits_dtype == WISP_BF16 ? take((size_t)kTabCacheSlots * kExpTabBytes) : 0;
     // the greedy variant's argmax partials (8 bytes per row and warp slice) share the statistics'
-    // space when they fit, else get their own
+    // space when they fit, else get their own (not in the fixed scratch, where it does not run)
     int S = 1, vps = 0;
     greedy_slices(c, sms, &S, &vps);
     const size_t gbytes = 8 * T * S;
-    L.row_parts = gbytes <= sizeof(SlicePart) * T * sh.sslices ? L.sparts : take(gbytes);
+    L.row_parts = gbytes <= sizeof(SlicePart) * T * sh.sslices || tile_budget != kTileBudget ? L.sparts : take(gbytes);
   }
   L.total = off;
   return L;
