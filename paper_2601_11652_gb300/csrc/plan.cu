@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int kKeep = 4;  // items per thread whose bucket is kept in registers
   __shared__ int s_w[6][32];
-  __shared__ unsigned long long s_sum[2];  // keys of the valid requests; KV tiles of the items
+  __shared__ unsigned long long s_sum[2];  // keys of the valid requests; passes over their KV tiles per KV head
   __shared__ int32_t s_valid;
   __shared__ int32_t s_hist[kOrderBuckets];
   // the attention's per-request arrays (pass 3) come after the acceptance part is done with its own
@@ -209,6 +209,11 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
       atomicAdd(&s_sum[0], (unsigned long long)n_lo + ((unsigned long long)n_hi << 16));
       atomicAdd(&s_valid, __popc(vm));
     }
+    if (p.split_sms) {  // (at most 2^25 tiles and 4 row groups each: a warp's sum fits 32 bits)
+      const int nrg = n > 0 ? (g * ((int)k + 1) + p.max_rows_item - 1) / p.max_rows_item : 0;
+      const unsigned t = __reduce_add_sync(0xffffffffu, (unsigned)((n + kOrderTile - 1) / kOrderTile) * nrg);
+      if (lane == 0 && t) atomicAdd(&s_sum[1], (unsigned long long)t);
+    }
     if (r < p.B) {
       const int64_t d0 = carry_d + incl - k, q0 = d0 + r;
       // a request whose rows fall outside the caller's buffers is never touched
@@ -236,6 +241,28 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   if (!p.with_attention) return;
   __syncthreads();
 
+  // SMs for the attention in a step whose acceptance pass runs beside it.  Both kernels are
+  // persistent and each fills an SM's shared memory, so the acceptance CTAs start on the SMs the
+  // attention leaves, and the step ends with the later of the two: the split that lets both end
+  // together is the attention's share of the work.  Times on all SMs, in ns: 3.2 (D = 128; 2.7 at
+  // 64) per pass over a KV tile of 64 tokens, 47 with an fp32 cache; 35.5 us, 22.5 per logit row and
+  // 0.27 per 1000 logits.  The constants are a fit to the split measured best (32 to 152 of 152
+  // SMs, steps of 4) for 24 batches of 1 to 512 requests, contexts of 64 to 128K tokens and
+  // vocabularies of 4K to 152K: within 2.5% of the best for 23 of them, 5% for one.  Before, it was
+  // half the SMs + 4 or seven eighths of them, by the number of tiles.  Steps on GB300, before and
+  // now: 256 requests 635, 592 us; 512 requests 1238, 1189; 32 requests 114, 107; 16 requests 100,
+  // 88; 8 requests with an fp32 cache 136, 114; 512 short requests with 4K tokens of vocabulary 495,
+  // 372; 300 requests with 8K 858, 754; one request of 100K tokens 130, 93; the others as before or
+  // faster.  At least a quarter of the SMs: a small batch's step is bound by the acceptance's chain,
+  // which more SMs do not shorten.  The fp32 kernel's time is in proportion to 1 / SMs, so beside
+  // less than 1/16 of its work the acceptance waits (4 requests of 30-60K: 503 us; 538 with 146 SMs).
+  const int sms = max(1, p.target_items / kItemsPerSM);
+  int na = sms;
+  if (p.split_sms && s_sum[1] > 0) {
+    const float att = (p.kv_f32 ? 47.0f : 2.24f + 0.0075f * (float)p.D) * (float)s_sum[1] * (float)p.Hkv;
+    const float acc = 35500.0f + (22.5f + 0.27e-3f * (float)p.V) * (float)p.total_q_rows;
+    if (!p.kv_f32 || att < 16.0f * acc) na = max((sms + 3) / 4, min(sms, (int)((float)sms * (att / (att + acc)) + 0.5f)));
+  }
   // pass 2: chunk length.  With at least as many (request, head) pairs as SMs, a longest-first
   // order balances whole sequences: only a sequence longer than 5/4 of the average work per SM
   // is cut (a split costs a merge of its chunks).  With fewer pairs than SMs, sequences are cut
@@ -243,9 +270,8 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // the order does not see, so it gets items of at most 2/3 of the average (32 requests of 512-4096
   // tokens: 307 us at 5/4, 290 at 2/3, 302 at 1/2; the tensor-core kernel there: 68, 80, 83 us).
   const int64_t work = (int64_t)s_sum[0] * p.Hkv;
-  const int64_t sms = max(1, p.target_items / kItemsPerSM);
-  const bool many_pairs = (int64_t)s_valid * p.Hkv >= sms;
-  const int64_t goal = many_pairs ? sms : (int64_t)p.target_items;
+  const bool many_pairs = (int64_t)s_valid * p.Hkv >= na;
+  const int64_t goal = many_pairs ? na : (int64_t)na * kItemsPerSM;
   int64_t chunk = ceil_div(work, goal);
   if (many_pairs) chunk = p.kv_f32 ? chunk - chunk / 3 : chunk + chunk / 4;
   chunk = max64(chunk, kMinChunk);
@@ -329,7 +355,6 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   int keep[kKeep];  // request and bucket of this thread's first items
 #pragma unroll
   for (int x = 0; x < kKeep; ++x) keep[x] = 0;
-  unsigned long long my_tiles = 0;  // KV tiles (kOrderTile tokens) of this thread's items
   for (int base = 0; base < p.B; base += kThreads) {
     size_requests(base, one);
     // per (request, head, row group) finished-chunk counters of the chunk's requests: zeroed, coalesced
@@ -341,7 +366,6 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
       if (item_carry + i >= p.max_items) break;  // (a request refused for want of room)
       int t0, t1;
       const int lo = request_of(i), bucket = keys_of(i, lo, t0, t1);
-      my_tiles += (unsigned)(t1 - t0 + kOrderTile - 1) / kOrderTile;
       atomicAdd(&s_hist[bucket], 1);
 #pragma unroll
       for (int y = 0; y < kKeep; ++y)
@@ -351,8 +375,6 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     __syncthreads();  // the shared arrays are rewritten by the next chunk; the histogram is complete after the last
   }
   const int n_items = (int)min64(item_carry, p.max_items);
-  for (int o = 16; o > 0; o >>= 1) my_tiles += __shfl_xor_sync(0xffffffffu, my_tiles, o);
-  if (lane == 0 && my_tiles) atomicAdd(&s_sum[1], my_tiles);
   {
     const int h = s_hist[tid];
     int tot;
@@ -404,21 +426,6 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   }
 
   if (tid == 0) {
-    const int64_t tiles = (int64_t)s_sum[1];
-    // SMs for the attention in a step whose acceptance pass runs beside it.  Both kernels are
-    // persistent and each fills an SM's shared memory, so the acceptance CTAs start on the SMs the
-    // attention leaves.  Measured on GB300 (bf16, D = 128): with few KV tiles per SM (under ~200
-    // of 64 tokens) the attention is latency-bound and about half the SMs stream its keys as fast
-    // as all of them (32 requests with 0.5-4K contexts: step 0.156 -> 0.129 ms with 80 attention
-    // CTAs of 152); with more it is bound by each SM's streaming rate, and only a few SMs (an
-    // eighth) pay off by starting the acceptance early (2-3% at 256-512 requests; a quarter or
-    // more is slower).  When the acceptance has little vocabulary work per KV tile (under 50
-    // elements: a few requests with long contexts) every SM stays with the attention.  The fp32
-    // kernel is bound by arithmetic, so every SM taken from it costs.
-    const int sms = p.target_items / kItemsPerSM;
-    int na = sms;
-    if (p.with_accept && p.split_sms && tiles > 0 && (int64_t)p.B * p.V >= 50 * tiles)
-      na = !p.kv_f32 && tiles < (int64_t)200 * sms ? sms / 2 + 4 : sms - sms / 8;
     PlanHeader hd;
     hd.n_items = n_items;
     hd.chunk_len = (int32_t)chunk;
