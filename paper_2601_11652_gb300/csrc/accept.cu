@@ -475,7 +475,6 @@ struct Item {
   U96 ea, ep;
   ff qp;
   int n_amb;
-  AmbElem amb[kAmbPerSlice];
 };
 
 // The draw's per-CTA exp table (dynamic shared memory): the fixed-point value as two 32-bit words,
@@ -499,7 +498,6 @@ struct Sm {
   int tab_valid;
   int tab_mode;
   int amb_n;
-  AmbElem amb[kAmbPerSlice];
   int keeper_done;
   int abort_;
 };
@@ -880,10 +878,11 @@ __device__ void c_draw(Sm &sm, Item &it, Tab tab, const char *ring, int &c, uint
           const float qi = q[h][i], fl = fix_to_float(fx[i]);
           if (!(fl > qi * zhi) && fl > qi * zlo) {
             const int a = atomicAdd(&sm.amb_n, 1);
-            if (a < kAmbPerSlice) {
-              sm.amb[a].e = fx[i];
-              sm.amb[a].q = qi;
-              sm.amb[a].v = (int)((cv0 + wi * TV + h * 32 + lane) * E + i);
+            if (a < p.amb_cap) {
+              AmbElem *el = p.damb + ((int64_t)it.r * p.dslices + it.s) * p.amb_cap + a;
+              el->e = fx[i];
+              el->q = qi;
+              el->v = (int)((cv0 + wi * TV + h * 32 + lane) * E + i);
             }
           }
         }
@@ -926,10 +925,8 @@ __device__ void c_draw(Sm &sm, Item &it, Tab tab, const char *ring, int &c, uint
     it.ea = a;
     it.ep = b;
     it.qp = t;
-    const int na = sm.amb_n;
-    it.n_amb = na;
-    for (int x = 0; x < na && x < kAmbPerSlice; ++x) it.amb[x] = sm.amb[x];
-    __threadfence();  // the tile records before the keeper's completion count
+    it.n_amb = sm.amb_n;
+    __threadfence();  // the tile records and undecided elements before the keeper's completion count
   }
 }
 
@@ -1243,7 +1240,6 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
     out->q_hi = it.qp.hi;
     out->q_lo = it.qp.lo;
     out->n_amb = it.n_amb;
-    for (int x = 0; x < it.n_amb && x < kAmbPerSlice; ++x) out->amb[x] = it.amb[x];
     __threadfence();
     last = atomicAdd(p.req_dcnt + r, 1) == Sd - 1;
   }
@@ -1271,10 +1267,11 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
   bool over = false;
   if (resid) {
     sd = u96_to_double(ep) - Zu * qp;
-    if (na > kAmbPerSlice) {
+    if (na > p.amb_cap) {
       over = true;
     } else {
-      for (int j = 0; j < na; ++j) sd += weight_d(__ldcg(&dp->amb[j].e), __ldcg(&dp->amb[j].q), true, Zu);
+      const AmbElem *el = p.damb + ((int64_t)r * Sd + lane) * p.amb_cap;
+      for (int j = 0; j < na; ++j) sd += weight_d(__ldcg(&el[j].e), __ldcg(&el[j].q), true, Zu);
     }
   }
   // slices with more undecided elements than their record holds: their mass by an exact pass
@@ -1335,7 +1332,7 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
   double thr_t = thr_d;
   const bool d_over = (ov >> d) & 1u;
   const int nad = resid && !d_over ? __shfl_sync(0xffffffffu, na, d) : 0;
-  const DrawPart *dd = p.dparts + (int64_t)r * Sd + d;
+  const AmbElem *dd = p.damb + ((int64_t)r * Sd + d) * p.amb_cap;
   const TileRec *tr = p.tiles + (int64_t)r * p.ntiles;
   run = 0.0;
   int64_t lastpos = -1;
@@ -1348,8 +1345,8 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
       } else if (resid) {
         w = u96_to_double(tile_u96(tr + t, true)) - Zu * ((double)__ldcg(&tr[t].q_hi) + (double)__ldcg(&tr[t].q_lo));
         for (int j = 0; j < nad; ++j) {
-          const int64_t vt = (int64_t)(__ldcg(&dd->amb[j].v) / E) / p.tile_vecs;
-          if (vt == t) w += weight_d(__ldcg(&dd->amb[j].e), __ldcg(&dd->amb[j].q), true, Zu);
+          const unsigned vt = (unsigned)__ldcg(&dd[j].v) / E / (unsigned)p.tile_vecs;  // (v < 2^24)
+          if (vt == t) w += weight_d(__ldcg(&dd[j].e), __ldcg(&dd[j].q), true, Zu);
         }
       } else {
         w = u96_to_double(tile_u96(tr + t, false));

@@ -8,7 +8,8 @@ namespace wisp {
 constexpr int kAcceptThreads = 256;  // consumer threads of an acceptance CTA (8 warps; plus a producer and a keeper warp)
 constexpr int kAcceptCtasPerSM = 2;  // resident CTAs per SM of the persistent acceptance kernel
 constexpr int kStatsChunkVecs = 3;   // 16-byte vectors per consumer thread in one chunk of the statistics stream
-constexpr int kAmbPerSlice = 8;      // residual elements per draw slice whose sign is left to the finisher
+constexpr int kAmbPerSlice = 64;     // residual elements per draw slice whose sign is left to the finisher
+constexpr int kAmbNoAlloc = 8;       // as many of them in the fixed scratch of wisp_verify_accept_noalloc
 constexpr int kMaxSlices = 32;       // warp slices per row of the greedy variant
 constexpr int kGreedyCtasPerSM = 3;  // resident CTAs (of kAcceptThreads) per SM of the greedy variant
 
@@ -65,13 +66,12 @@ struct AmbElem {
 
 // Totals of one draw slice of row L: sum of exp(z - m) over all elements (fixed point); over the
 // elements with p > q (certainly), the sum of exp(z - m) (fixed point) and of q (double-float);
-// the undecided elements.
+// the number of undecided elements.
 struct DrawPart {
   U96 e_all, e_p;
   float q_hi, q_lo;
-  int n_amb;     // > kAmbPerSlice: overflowed (the finisher rescans the slice)
+  int n_amb;     // more than were kept: overflowed (the finisher rescans the slice)
   int pad;
-  AmbElem amb[kAmbPerSlice];
 };
 
 // Sums of one tile (tile_vecs consecutive vectors of row L) written by the draw: over all elements
@@ -109,6 +109,8 @@ struct AcceptParams {
   int32_t *req_dcnt;       // [B] finished draw slices
   int32_t *queue;          // [B] requests ready to draw (-1: not yet written)
   DrawPart *dparts;        // [B, dslices]
+  AmbElem *damb;           // [B, dslices, amb_cap] undecided elements of the slices
+  int amb_cap;
   TileRec *tiles;          // [B, ntiles]
   uint32_t *tcache;        // [kTabCacheSlots, 2 * kExpTabEntries] exp tables by row maximum (bf16 logits)
   AccCounters *ctr;

@@ -135,7 +135,7 @@ void greedy_slices(const wisp_accept_args *c, int sms, int *slices, int *vps) {
 constexpr size_t kTileBudget = (size_t)256 << 20;
 constexpr size_t kNoAllocTileBudget = (size_t)4 << 20;
 struct AcceptShape {
-  int sslices, svps, dslices, vpd, tile_vecs, ntiles;
+  int sslices, svps, dslices, vpd, tile_vecs, ntiles, amb_cap;
 };
 AcceptShape accept_shape(const wisp_accept_args *c, int sms, size_t tile_budget) {
   const int E = c->logits_dtype == WISP_BF16 ? 8 : 4;
@@ -162,8 +162,11 @@ AcceptShape accept_shape(const wisp_accept_args *c, int sms, size_t tile_budget)
   sh.tile_vecs = tiles ? 64 : 0;
   sh.ntiles = tiles ? (int)nt : 0;
   // draw slices: one wave of items over the CTAs when the batch is small, up to two waves (and
-  // about three slices per row) as it grows, and at least two per row (a slice keeps at most
-  // kAmbPerSlice undecided elements; past that the bookkeeper weighs the slice exactly alone)
+  // about three slices per row) as it grows, and at least two per row.  A slice keeps at most
+  // amb_cap undecided elements; past that the bookkeeper weighs the slice exactly alone, which
+  // takes over a millisecond (512 requests, one of whose slices had 9: 1977 us with room for 8,
+  // 291 with room for 64)
+  sh.amb_cap = tile_budget == kTileBudget ? kAmbPerSlice : kAmbNoAlloc;
   cut(std::max<int64_t>(2 * B, std::max<int64_t>(ctas, std::min<int64_t>(2 * ctas, 3 * B))), B, kAcceptThreads,
       &sh.dslices, &sh.vpd);
   return sh;
@@ -223,6 +226,7 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
     L.sparts = take(sizeof(SlicePart) * T * sh.sslices);
     L.req_state = take(sizeof(int32_t) * 5 * (size_t)c->B);
     L.dparts = take(sizeof(DrawPart) * (size_t)c->B * sh.dslices);
+    L.damb = take(sizeof(AmbElem) * (size_t)c->B * sh.dslices * sh.amb_cap);
     L.tiles = take(sizeof(TileRec) * ((size_t)c->B * sh.ntiles + 1));
     L.tcache = c->logits_dtype == WISP_BF16 ? take((size_t)kTabCacheSlots * kExpTabBytes) : 0;
     // the greedy variant's argmax partials (8 bytes per row and warp slice) share the statistics'
@@ -363,6 +367,8 @@ AcceptParams accept_params(const wisp_accept_args *c, void *ws, const Layout &L,
   ap.req_dcnt = rs + 3 * (size_t)c->B;
   ap.queue = rs + 4 * (size_t)c->B;
   ap.dparts = at<DrawPart>(ws, L.dparts);
+  ap.damb = at<AmbElem>(ws, L.damb);
+  ap.amb_cap = sh.amb_cap;
   ap.ctr = at<AccCounters>(ws, L.acc_ctr);
   ap.tcache = bf ? at<uint32_t>(ws, L.tcache) : nullptr;
   ap.request_ids = c->request_ids;

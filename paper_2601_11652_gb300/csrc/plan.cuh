@@ -79,6 +79,7 @@ struct Layout {
   size_t sparts = 0;          // SlicePart [total_q_rows, sslices]
   size_t req_state = 0;       // int32 [5, B]: lowest rejecting row, claim, L, finished draw slices, queue
   size_t dparts = 0;          // DrawPart [B, dslices]
+  size_t damb = 0;            // AmbElem [B, dslices, amb_cap]
   size_t tiles = 0;           // TileRec [B, ntiles]
   size_t tcache = 0;          // uint32 [kTabCacheSlots, 2 * kExpTabEntries]: the draw's exp tables
   // greedy variant
