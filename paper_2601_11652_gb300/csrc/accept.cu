@@ -166,17 +166,13 @@ __device__ __forceinline__ unsigned long long ff_to_fix(ff a) {
   return r > 0 ? (unsigned long long)r : 0ull;
 }
 
-// A draw weight: round(2^56 exp(z - m)) and exp(z - m) rounded to float.
-struct Wt {
-  unsigned long long fix;
-  float f;
-};
-
-// exp(z - m), z <= m, computed directly (double-float, Tang's method).
-__device__ __noinline__ Wt exp_fix_direct(float z, float m, const float *th, const float *tl) {
+// round(2^56 exp(z - m)), z <= m, computed directly (double-float, Tang's method).
+__device__ __forceinline__ unsigned long long exp_fix_inline(float z, float m, const float *th, const float *tl) {
   const ff x = ff_two_sum(z, -m);
-  const ff e = ff_exp_nonpos(x.hi, x.lo, th, tl);
-  return Wt{ff_to_fix(e), e.hi};
+  return ff_to_fix(ff_exp_nonpos(x.hi, x.lo, th, tl));
+}
+__device__ __noinline__ unsigned long long exp_fix_direct(float z, float m, const float *th, const float *tl) {
+  return exp_fix_inline(z, m, th, tl);
 }
 
 // s += q exactly as a double-float without renormalisation (Knuth's TwoSum; the low part collects
@@ -600,7 +596,7 @@ __device__ void ensure_table(float m, Sm &sm, Tab tab, uint32_t &ph, const Accep
     } else {
       for (int idx = threadIdx.x; idx < kExpTabSize; idx += kConsumers) {
         const float u = bf16_bits_to_float(exp_tab_bits(idx));
-        const unsigned long long fx = u <= m ? exp_fix_direct(u, m, sm.th, sm.tl).fix : 0ull;
+        const unsigned long long fx = u <= m ? exp_fix_direct(u, m, sm.th, sm.tl) : 0ull;
         tab.lo[exp_tab_entry_of(idx)] = (uint32_t)fx;
         tab.hi[exp_tab_entry_of(idx)] = (uint32_t)(fx >> 32);
       }
@@ -636,7 +632,7 @@ template <typename LT>
 __device__ __forceinline__ void weights(const uint4 &w, float m, const Sm &sm, Tab tab,
                                         unsigned long long (&fx)[LTraits<LT>::E]);
 __device__ __noinline__ unsigned long long weight_direct1(uint32_t bits, float m, const Sm &sm) {
-  return bits == 0xFF80u ? 0ull : exp_fix_direct(__uint_as_float(bits << 16), m, sm.th, sm.tl).fix;
+  return bits == 0xFF80u ? 0ull : exp_fix_direct(__uint_as_float(bits << 16), m, sm.th, sm.tl);
 }
 template <>
 __device__ __forceinline__ void weights<uint16_t>(const uint4 &w, float m, const Sm &sm, Tab tab,
@@ -669,7 +665,7 @@ template <>
 __device__ __forceinline__ void weights<float>(const uint4 &w, float m, const Sm &sm, Tab,
                                                unsigned long long (&fx)[4]) {
   #pragma unroll
-  for (int i = 0; i < 4; ++i) fx[i] = exp_fix_direct(vec_elem<float>(w, i), m, sm.th, sm.tl).fix;
+  for (int i = 0; i < 4; ++i) fx[i] = exp_fix_direct(vec_elem<float>(w, i), m, sm.th, sm.tl);
 }
 
 // A fixed-point weight (units 2^-56, at most 2^56) as a float, within 2^-23 of its value relative:
@@ -681,9 +677,31 @@ __device__ __forceinline__ float fix_to_float(unsigned long long x) {
 __device__ __forceinline__ double ff_to_double_(ff a) { return (double)a.hi + (double)a.lo; }
 
 // Draw weight of one element in units of 2^-56, in double: the residual max(0, e - q Z) (Z = Zu in
-// the same units) or e itself.  fmax drops a NaN q (no mass), as max(0, p - q) does.
+// the same units) or e itself.  A NaN q has no mass, as in max(0, p - q).
 __device__ __forceinline__ double weight_d(unsigned long long e, float q, bool residual, double Zu) {
-  return residual ? fmax(0.0, (double)e - (double)q * Zu) : (double)e;
+  const double w = residual ? (double)e - (double)q * Zu : (double)e;
+  // negative or NaN: zero (by the bits: an FP64 comparison takes as long as an FP64 addition)
+  return (unsigned long long)__double_as_longlong(w) > 0x7FF0000000000000ull ? 0.0 : w;
+}
+
+// An FP64 operation of the bookkeeping warp takes about 120 cycles on GB300 and everything it runs is run
+// seldom enough to be fetched anew, so the draw's last chain (k_draw, keeper_finish) keeps FP64 operations
+// few and its code short and shared: comparisons on the bits, one scan function, loops not unrolled.
+
+// Orders doubles as integers (NaN above every number if positive; no -0 is compared).
+__device__ __forceinline__ long long dkey(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll);
+}
+// Inclusive sums over the lanes.
+__device__ __noinline__ double warp_scan(double v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const double t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
 }
 
 // Exact draw weight (units 2^-56, double) of one vector once the normaliser Zu is known: the sign of
@@ -930,102 +948,101 @@ __device__ void c_draw(Sm &sm, Item &it, Tab tab, const char *ring, int &c, uint
   }
 }
 
-// The exp table for row maximum m from the launch's global cache, if a CTA has published it
-// (bit-identical to a table built here); else none (the direct exp is then used).
-__device__ Tab cached_table(const AcceptParams &p, float m) {
-  const unsigned mb = __float_as_uint(m);
-  if (!p.tcache) return Tab{nullptr, nullptr};
-  const int slot = (int)((mb >> 16) & (kTabCacheSlots - 1));
-  if (ptx::ld_acquire_gpu(&p.ctr->tab_state[slot]) != 2 || ld_vol((const int32_t *)&p.ctr->tab_m[slot]) != (int32_t)mb)
-    return Tab{nullptr, nullptr};
-  uint32_t *t = p.tcache + (size_t)slot * 2 * kExpTabEntries;
-  return Tab{t, t + kExpTabEntries};
+// The token of the crossing of r2 (or, past the last, the last with weight; -1 without one) among the
+// elements of two vectors from vector g on: one lane per element, its exact weight, a scan.
+template <typename LT>
+__device__ __noinline__ int pair_token(const AcceptParams &p, const Sm &sm, const LT *row, const float *qrow, float m,
+                                       double Zu, int64_t g, int64_t v1, double r2) {
+  constexpr int E = LTraits<LT>::E;
+  const int lane = threadIdx.x & 31;
+  const int64_t v = g * E + lane;
+  double wt = 0.0;
+  if (lane < 2 * E && v < p.V && v < v1 * E)
+    wt = weight_d(exp_fix_inline(load_scalar(row, v), m, sm.th, sm.tl), qrow ? __ldg(qrow + v) : 0.0f, qrow != nullptr, Zu);
+  const double acc = warp_scan(wt);
+  const unsigned some = __ballot_sync(0xffffffffu, dkey(wt) > 0);
+  const unsigned over = __ballot_sync(0xffffffffu, dkey(acc) > dkey(r2)) & some;
+  return over ? (int)(g * E + __ffs(over) - 1) : some ? (int)(g * E + 31 - __clz(some)) : -1;
 }
 
 // The extra token (Eq. 3) from vectors [v0, v1) of row L, which hold the crossing of thr (the
 // share of u * total left at v0), by the bookkeeping warp right after it has located them: exact
-// weights of 32 vectors at a time, a warp scan in token order, then the element of the crossing
-// within its vector; with take_last, or when rounding leaves no crossing, the last element with
-// weight.  Writes the request's outputs.
+// weights of 64 vectors at a time (a tile; two neighbouring vectors per lane, one element of each at a
+// time), a warp scan in token order, then the elements of the crossing's two vectors, one lane each; with
+// take_last, or when rounding leaves no crossing, the last element with weight.  Writes the request's
+// outputs.  Against one vector per lane in two turns (weights from a table in L2, the crossing vector's E
+// double-precision weights by one lane in a row), acceptance on GB300: 32 requests 66 -> 60 us, 256 requests
+// 177 -> 166 us, 512 requests with 4K tokens of vocabulary 175 -> 135 us.  Unrolled, with the exps of both
+// vectors side by side, it was slower than before (32 requests 68 us): code run once is fetched at about 100
+// cycles per 8 instructions.
 template <typename LT>
 __device__ void keeper_finish(const AcceptParams &p, const Sm &sm, int r, int i, bool resid, int64_t Q0, int64_t D0,
                               float m, double Zu, int64_t v0, int64_t v1, double thr, bool take_last) {
   constexpr int E = LTraits<LT>::E;
   const int lane = threadIdx.x & 31;
+  const uint32_t ni = LTraits<LT>::NEG_INF2;
   const LT *row = static_cast<const LT *>(p.logits) + (Q0 + i) * (int64_t)p.V;
-  const float *qrow = p.draft_probs + (D0 + i) * (int64_t)p.V;
-  const Tab tab = std::is_same<LT, uint16_t>::value ? cached_table(p, m) : Tab{nullptr, nullptr};
+  const float *qrow = resid ? p.draft_probs + (D0 + i) * (int64_t)p.V : nullptr;
+  const float Zf = (float)(Zu * 0x1p-56);
+  const float zh = Zf * (1.0f + 0x1p-20f), zl = Zf * (1.0f - 0x1p-20f);
   double carry = 0.0;
   int tok = -1;
-  int64_t last_vec = -1;  // the last vector with weight so far
-  for (int64_t base = v0; base < v1 && tok < 0; base += 32) {
-    const int64_t vi = base + lane;
-    const bool have = vi < v1;
-    uint4 w = make_uint4(0, 0, 0, 0);
-    float q[E];
+  int64_t last = -1;  // the last pair of vectors with weight so far
+  for (int64_t base = v0; base < v1 && tok < 0; base += 64) {
+    uint4 w[2];
+    float q[2][E];
 #pragma unroll
-    for (int x = 0; x < E; ++x) q[x] = 0.0f;
-    if (have) {
-      w = load_vec<LT>(row, vi, p.V, p.vec_z != 0);
-      if (resid) load_q<E>(qrow, vi * E, p.V, p.vec_q != 0, q);
+    for (int h = 0; h < 2; ++h) {
+      const int64_t vi = base + 2 * lane + h;
+      w[h] = make_uint4(ni, ni, ni, ni);
+#pragma unroll
+      for (int x = 0; x < E; ++x) q[h][x] = 0.0f;
+      if (vi < v1) {
+        w[h] = load_vec<LT>(row, vi, p.V, p.vec_z != 0);
+        if (resid) load_q<E>(qrow, vi * E, p.V, p.vec_q != 0, q[h]);
+      }
     }
-    const double wv = have ? vec_weight<LT>(w, q, resid, m, Zu, sm, tab) : 0.0;
-    double incl = wv;
-    for (int o = 1; o < 32; o <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+    // the two vectors' mass: integer sums of the weights, double-float sums of q over the elements with
+    // p > q for certain (an fp32 test with a 2^-20 margin), the others in double
+    unsigned long long sp = 0;
+    ff sq[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
+    double ad = 0.0;
+#pragma unroll 1
+    for (int x = 0; x < E; ++x) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const unsigned long long fx = exp_fix_inline(__uint_as_float(E == 4 ? w[h].x : w[h].x << 16), m, sm.th, sm.tl);
+        const float qx = q[h][0], fl = fix_to_float(fx);
+        const bool sure = qx >= 0.0f && fl > qx * zh;
+        sp += sure ? fx : 0ull;
+        ff_acc(sq[h], sure ? qx : 0.0f);
+        if (!sure && fl > qx * zl) ad += weight_d(fx, qx, true, Zu);
+        // on to the next element
+        if (E == 4) {
+          w[h] = make_uint4(w[h].y, w[h].z, w[h].w, 0u);
+        } else {
+          w[h] = make_uint4(__funnelshift_r(w[h].x, w[h].y, 16), __funnelshift_r(w[h].y, w[h].z, 16),
+                            __funnelshift_r(w[h].z, w[h].w, 16), w[h].w >> 16);
+        }
+#pragma unroll
+        for (int y = 0; y + 1 < E; ++y) q[h][y] = q[h][y + 1];
+      }
     }
-    incl += carry;
-    const unsigned pos = __ballot_sync(0xffffffffu, have && wv > 0.0);
-    if (pos) last_vec = base + 31 - __clz(pos);
-    const unsigned hit = take_last ? 0u : __ballot_sync(0xffffffffu, have && incl > thr);
+    double t = (double)sp + ad;
+    if (resid) t -= Zu * (ff_to_double_(sq[0]) + ff_to_double_(sq[1]));
+    const double incl = warp_scan(t) + carry;
+    const unsigned pos = __ballot_sync(0xffffffffu, dkey(t) > 0);
+    if (pos) last = base + 2 * (31 - __clz(pos));
+    const unsigned hit = take_last ? 0u : __ballot_sync(0xffffffffu, dkey(incl) > dkey(thr)) & pos;
     if (hit) {
       const int l0 = __ffs(hit) - 1;
-      int t_ = -1;
-      if (lane == l0) {
-        // this lane's elements in order, with exact weights
-        unsigned long long fx[E];
-        weights<LT>(w, m, sm, tab, fx);
-        double wt[E];
-#pragma unroll
-        for (int x = 0; x < E; ++x) wt[x] = vi * E + x < p.V ? weight_d(fx[x], q[x], resid, Zu) : 0.0;
-        const double r2 = thr - (incl - wv);
-        double acc = 0.0;
-        int lastv = -1;
-#pragma unroll
-        for (int x = 0; x < E; ++x) {
-          if (t_ < 0) {
-            if (wt[x] > 0.0) lastv = (int)(vi * E + x);
-            acc += wt[x];
-            if (acc > r2) t_ = (int)(vi * E + x);
-          }
-        }
-        if (t_ < 0) t_ = lastv;
-      }
-      tok = __shfl_sync(0xffffffffu, t_, l0);
-      if (tok < 0) tok = -2;  // the crossing vector had no element with weight after all
+      tok = pair_token<LT>(p, sm, row, qrow, m, Zu, base + 2 * l0, v1, __shfl_sync(0xffffffffu, thr - (incl - t), l0));
       break;
     }
     carry = __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (tok < 0) {
-    // no crossing (take_last, or rounding): the last element with weight
-    tok = -1;
-    if (last_vec >= 0 && lane == 0) {
-      const uint4 w = load_vec<LT>(row, last_vec, p.V, p.vec_z != 0);
-      float q[E];
-#pragma unroll
-      for (int x = 0; x < E; ++x) q[x] = 0.0f;
-      if (resid) load_q<E>(qrow, last_vec * E, p.V, p.vec_q != 0, q);
-      unsigned long long fx[E];
-      weights<LT>(w, m, sm, tab, fx);
-#pragma unroll
-      for (int x = 0; x < E; ++x) {
-        const int64_t v = last_vec * E + x;
-        if (v < p.V && weight_d(fx[x], q[x], resid, Zu) > 0.0) tok = (int)v;
-      }
-    }
-  }
+  if (tok < 0 && last >= 0)  // no crossing (take_last, or rounding): the last element with weight
+    tok = pair_token<LT>(p, sm, row, qrow, m, Zu, last, v1, INFINITY);
   if (lane == 0) {
     p.accepted_len[r] = i;
     p.next_token[r] = tok;
@@ -1251,6 +1268,7 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
   U96 ea = u96_zero(), ep = u96_zero();
   double qp = 0.0;
   int na = 0;
+  const float u = __ldg(p.sample_u + r);
   const DrawPart *dp = p.dparts + (int64_t)r * Sd + lane;
   if (lane < Sd) {
     ea.lo = __ldcg(&dp->e_all.lo);
@@ -1284,26 +1302,18 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
   }
   // the slices' masses in slice order: an inclusive warp scan (lane d: slices 0..d), the total from
   // the last lane, so that the crossing search below reads the same prefix sums as the total
-  auto slice_scan = [&](double v) {
-    double incl = lane < Sd ? v : 0.0;
-    for (int o = 1; o < 32; o <<= 1) {
-      const double t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    return incl;
-  };
-  double incl = slice_scan(sd);
+  double incl = warp_scan(lane < Sd ? sd : 0.0);
   double S = __shfl_sync(0xffffffffu, incl, 31);
   if (resid && !(S > 0.0)) {
     // the residual has no mass (only through rounding): draw from p_L instead
     resid = false;
     sd = se;
-    incl = slice_scan(sd);
+    incl = warp_scan(lane < Sd ? sd : 0.0);
     S = __shfl_sync(0xffffffffu, incl, 31);
   }
-  const double thr = (double)__ldg(p.sample_u + r) * S;
-  const unsigned hitd = __ballot_sync(0xffffffffu, lane < Sd && incl > thr);
-  const unsigned massd = __ballot_sync(0xffffffffu, lane < Sd && sd > 0.0);
+  const double thr = (double)u * S;
+  const unsigned massd = __ballot_sync(0xffffffffu, lane < Sd && dkey(sd) > 0);
+  const unsigned hitd = __ballot_sync(0xffffffffu, dkey(incl) > dkey(thr)) & massd;
   const int owner = hitd ? __ffs(hitd) - 1 : -1;
   const int lastd = massd ? 31 - __clz(massd) : -1;
   // the share of thr left at the owner's first element: thr minus the scan's prefix before it
@@ -1325,35 +1335,46 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
     keeper_finish<LT>(p, sm, r, it.i, resid, it.Q0, it.D0, it.rec.m, Zu, s0, s1, thr_d, take_last != 0);
     return;
   }
-  // the tile within slice d
-  const int64_t tlo = (int64_t)d * p.vpd / p.tile_vecs;
-  const int64_t thi = min((int64_t)p.ntiles, (min(nvec, (int64_t)(d + 1) * p.vpd) + p.tile_vecs - 1) / p.tile_vecs);
-  int64_t tile = -1;
+  // the tile within slice d, 32 records at a time, the next 32 loaded ahead
+  const int tlo = (int)((unsigned)(d * p.vpd) / (unsigned)p.tile_vecs);
+  const int thi = min(p.ntiles, (int)((unsigned)(s1 + p.tile_vecs - 1) / (unsigned)p.tile_vecs));
+  int tile = -1;
   double thr_t = thr_d;
   const bool d_over = (ov >> d) & 1u;
   const int nad = resid && !d_over ? __shfl_sync(0xffffffffu, na, d) : 0;
   const AmbElem *dd = p.damb + ((int64_t)r * Sd + d) * p.amb_cap;
   const TileRec *tr = p.tiles + (int64_t)r * p.ntiles;
   run = 0.0;
-  int64_t lastpos = -1;
-  for (int64_t t0 = tlo; t0 < thi && tile < 0; t0 += 32) {
-    const int64_t t = t0 + lane;
-    double w = 0.0;
+  int lastpos = -1;
+  U96 nx = u96_zero();
+  float nqh = 0.0f, nql = 0.0f;
+  auto ahead = [&](int t) {
+    nx = u96_zero();
+    nqh = nql = 0.0f;
     if (t < thi) {
-      if (d_over) {
-        w = 0.0;  // filled below, one tile at a time, by the whole warp
-      } else if (resid) {
-        w = u96_to_double(tile_u96(tr + t, true)) - Zu * ((double)__ldcg(&tr[t].q_hi) + (double)__ldcg(&tr[t].q_lo));
-        for (int j = 0; j < nad; ++j) {
-          const unsigned vt = (unsigned)__ldcg(&dd[j].v) / E / (unsigned)p.tile_vecs;  // (v < 2^24)
-          if (vt == t) w += weight_d(__ldcg(&dd[j].e), __ldcg(&dd[j].q), true, Zu);
-        }
-      } else {
-        w = u96_to_double(tile_u96(tr + t, false));
+      nx = tile_u96(tr + t, resid);
+      if (resid) {
+        nqh = __ldcg(&tr[t].q_hi);
+        nql = __ldcg(&tr[t].q_lo);
       }
     }
+  };
+  ahead(tlo + lane);
+#pragma unroll 1
+  for (int t0 = tlo; t0 < thi && tile < 0; t0 += 32) {
+    const int t = t0 + lane;
+    const U96 x = nx;
+    const float qh = nqh, ql = nql;
+    ahead(t + 32);
+    double w = u96_to_double(x);
+    if (resid) w -= Zu * ((double)qh + (double)ql);
+    for (int j = 0; j < nad; ++j) {
+      const unsigned vt = (unsigned)__ldcg(&dd[j].v) / E / (unsigned)p.tile_vecs;  // (v < 2^24)
+      if (vt == (unsigned)t) w += weight_d(__ldcg(&dd[j].e), __ldcg(&dd[j].q), true, Zu);
+    }
     if (d_over) {
-      // the slice's tile sums miss undecided elements: exact tile masses
+      // the slice's tile sums miss undecided elements: exact tile masses, by the whole warp
+      w = 0.0;
       for (int x = 0; x < 32 && t0 + x < thi; ++x) {
         const int64_t tt = t0 + x;
         const double m_ = warp_range_weight<LT>(p, sm, row, resid ? qrow : nullptr, it.rec.m, Zu,
@@ -1361,21 +1382,14 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
         if (lane == x) w = m_;
       }
     }
-    double incl = w;
-    for (int o = 1; o < 32; o <<= 1) {
-      const double u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
-    }
-    incl += run;
-    const unsigned pos = __ballot_sync(0xffffffffu, t < thi && w > 0.0);
+    const double incl = warp_scan(w) + run;
+    const unsigned pos = __ballot_sync(0xffffffffu, dkey(w) > 0);
     if (pos) lastpos = t0 + 31 - __clz(pos);
-    if (!take_last) {
-      const unsigned hit = __ballot_sync(0xffffffffu, t < thi && incl > thr_d);
-      if (hit) {
-        const int l0 = __ffs(hit) - 1;
-        tile = t0 + l0;
-        thr_t = thr_d - __shfl_sync(0xffffffffu, incl - w, l0);
-      }
+    const unsigned hit = take_last ? 0u : __ballot_sync(0xffffffffu, dkey(incl) > dkey(thr_d)) & pos;
+    if (hit) {
+      const int l0 = __ffs(hit) - 1;
+      tile = t0 + l0;
+      thr_t = thr_d - __shfl_sync(0xffffffffu, incl - w, l0);
     }
     run = __shfl_sync(0xffffffffu, incl, 31);
   }
@@ -1390,7 +1404,7 @@ __device__ void k_draw(const AcceptParams &p, Sm &sm, const Item &it) {
     }
     return;
   }
-  const int64_t t0v = tile * p.tile_vecs;
+  const int64_t t0v = (int64_t)tile * p.tile_vecs;
   keeper_finish<LT>(p, sm, r, it.i, resid, it.Q0, it.D0, it.rec.m, Zu, t0v, min(nvec, t0v + p.tile_vecs), thr_t,
                     take_last != 0);
 }
