@@ -143,20 +143,13 @@ __device__ __forceinline__ uint32_t exp_tab_entry(uint32_t b, uint32_t &d) {
 __device__ __forceinline__ int exp_tab_entry_of(int idx) { return idx + (idx >= kExpTabHalf ? 1 : 0); }
 
 // round(2^56 x) for |x| <= 1 from the bits of x (integer operations only: 64-bit conversions run
-// on the slow FP64 pipe); zero below 2^-126.
+// on the slow FP64 pipe; selects, not branches, which the lanes of a warp would take in turn).
 __device__ __forceinline__ long long f32_to_fix(float x) {
   const uint32_t b = __float_as_uint(x);
-  const int e = (int)((b >> 23) & 0xFFu);
-  if (e == 0) return 0;
-  const unsigned long long mant = (unsigned long long)((b & 0x7FFFFFu) | 0x800000u);  // x = mant 2^(e - 150)
-  const int sh = e - 150 + kFixShift;
-  unsigned long long v;
-  if (sh >= 0)
-    v = mant << sh;
-  else if (sh > -40)
-    v = (mant + (1ull << (-sh - 1))) >> (-sh);
-  else
-    v = 0;
+  const uint32_t mant = (b & 0x7FFFFFu) | 0x800000u;  // x = mant 2^(e - 150), e its exponent field
+  const int sh = (int)((b >> 23) & 0xFFu) - 150 + kFixShift;
+  const int s = min(max(-sh, 1), 26);  // (from 25 places on nothing is left, a subnormal's included)
+  const unsigned long long v = sh >= 0 ? (unsigned long long)mant << sh : (unsigned long long)((mant + (1u << (s - 1))) >> s);
   return (b >> 31) ? -(long long)v : (long long)v;
 }
 // round(2^56 a) for a double-float a in [0, 1] (the two parts converted exactly up to the last

@@ -132,7 +132,8 @@ __device__ __forceinline__ ff ff_exp_nonpos(float xh, float xl, const float *tab
   constexpr float C_HI = 0x1.62p-9f;        // ln2/256 rounded to 8 significant bits
   constexpr float C_MID = 0x1.c85fep-18f;   // next 24 bits
   constexpr float C_LO = -0x1.718432p-43f;  // next 24 bits
-  if (!(xh > -87.0f)) return {0.0f, 0.0f};  // exp(x) < 1.7e-38: below ff resolution of any sum >= 1
+  const bool none = !(xh > -87.0f);  // exp(x) < 1.7e-38: below ff resolution of any sum >= 1
+  xh = fmaxf(xh, -87.0f);
   const float Nf = rintf(xh * kInvC);
   const int N = (int)Nf;
   const float r1 = __fmaf_rn(-Nf, C_HI, xh);  // exact
@@ -151,7 +152,7 @@ __device__ __forceinline__ ff ff_exp_nonpos(float xh, float xl, const float *tab
   const int kexp = (N - j) >> 8;  // in [-126, 0] since x > -87
   e = ff_mul(e, ff{tab_hi[j], tab_lo[j]});
   const float scale = __int_as_float((127 + kexp) << 23);
-  return {__fmul_rn(e.hi, scale), __fmul_rn(e.lo, scale)};
+  return {none ? 0.0f : __fmul_rn(e.hi, scale), none ? 0.0f : __fmul_rn(e.lo, scale)};
 }
 
 }  // namespace wisp
