@@ -658,7 +658,7 @@ template <>
 __device__ __forceinline__ void weights<float>(const uint4 &w, float m, const Sm &sm, Tab,
                                                unsigned long long (&fx)[4]) {
   #pragma unroll
-  for (int i = 0; i < 4; ++i) fx[i] = exp_fix_direct(vec_elem<float>(w, i), m, sm.th, sm.tl);
+  for (int i = 0; i < 4; ++i) fx[i] = exp_fix_inline(vec_elem<float>(w, i), m, sm.th, sm.tl);
 }
 
 // A fixed-point weight (units 2^-56, at most 2^56) as a float, within 2^-23 of its value relative:
@@ -1110,8 +1110,8 @@ __device__ void try_determine(const AcceptParams &p, int r, int k, int64_t Q0) {
     return;
   }
   st_vol(p.req_L + r, L);
-  __threadfence();
   const int pos = atomicAdd(&p.ctr->q_reserve, 1);  // reserve a queue entry
+  __threadfence();                                  // L before the entry
   st_vol(p.queue + pos, r);
   __threadfence();
   atomicAdd(&p.ctr->n_claimed, 1);  // after the queue entry: a CTA that sees every request claimed sees it
@@ -1432,14 +1432,16 @@ namespace {
 // Lane 0: the next statistics item in the level-major order (skipping rows past a known rejection and rows of
 // decided requests), if one is left.
 template <typename LT>
-__device__ bool pick_stats(const AcceptParams &p, Item &d) {
+__device__ bool pick_stats(const AcceptParams &p, Item &d, bool &left) {
   constexpr int E = LTraits<LT>::E;
   const int64_t nvec = (p.V + E - 1) / E;
   AccCounters *c = p.ctr;
-  const int n_items = __ldcg(&c->n_items);
-  while (ld_vol(&c->stats_next) < n_items) {
+  while (left) {
     const int t = atomicAdd(&c->stats_next, 1);
-    if (t >= n_items) break;
+    if (t >= __ldcg(&c->n_items)) {
+      left = false;  // (a producer takes at most one past the end)
+      break;
+    }
     const int2 ent = __ldcg(p.row_order + t / p.sslices);
     const int r = ent.x, i = ent.y;
     if (i > ld_vol(p.req_rej + r)) continue;  // past a rejection, or the request is decided
@@ -1513,7 +1515,7 @@ __device__ bool pick_draw(const AcceptParams &p, Sm &sm, Item &d, int &pend) {
 // Lane 0: the next work item of this CTA.  WORK_EXIT once every valid request is decided, every draw ticket
 // taken and this CTA's keeper is done with everything issued; WORK_WAIT otherwise.
 template <typename LT>
-__device__ int pick(const AcceptParams &p, Sm &sm, Item &d, long long &idle_since, int issued, int &pend) {
+__device__ int pick(const AcceptParams &p, Sm &sm, Item &d, long long &idle_since, int issued, int &pend, bool &left) {
   AccCounters *c = p.ctr;
   const int Sd = p.dslices;
   if (vload(sm.abort_)) return WORK_EXIT;
@@ -1523,7 +1525,7 @@ __device__ int pick(const AcceptParams &p, Sm &sm, Item &d, long long &idle_sinc
   const bool draws_first = blockIdx.x * 8 >= gridDim.x * 3;
   int kind = WORK_WAIT;
   if (draws_first && pick_draw<LT>(p, sm, d, pend)) kind = WORK_DRAW;
-  if (kind == WORK_WAIT && pick_stats<LT>(p, d)) kind = WORK_STATS;
+  if (kind == WORK_WAIT && pick_stats<LT>(p, d, left)) kind = WORK_STATS;
   if (kind == WORK_WAIT && !draws_first && pick_draw<LT>(p, sm, d, pend)) kind = WORK_DRAW;
   if (kind != WORK_WAIT) {
     idle_since = -1;
@@ -1585,13 +1587,14 @@ template <typename LT>
 __device__ void producer(const AcceptParams &p, Sm &sm, char *ring) {
   const int lane = threadIdx.x & 31;
   long long idle_since = -1;
-  int pend = -1;  // lane 0: a draw ticket taken but not yet usable
+  int pend = -1;     // lane 0: a draw ticket taken but not yet usable
+  bool left = true;  // statistics items may be left
   int n = 0, c = 0;
   bool ok = true;
   for (;;) {
     Item d;
     int kind = WORK_WAIT;
-    if (lane == 0) kind = pick<LT>(p, sm, d, idle_since, n, pend);
+    if (lane == 0) kind = pick<LT>(p, sm, d, idle_since, n, pend, left);
     kind = __shfl_sync(0xffffffffu, kind, 0);
     if (kind == WORK_WAIT) {
       __nanosleep(256);
@@ -1662,8 +1665,6 @@ __global__ void __launch_bounds__(kCtaThreads, kAcceptCtasPerSM) accept_kernel(c
   char *ring = reinterpret_cast<char *>(s_dyn);
   const Tab tab{reinterpret_cast<uint32_t *>(s_dyn + kRingBytes),
                 reinterpret_cast<uint32_t *>(s_dyn + kRingBytes + kExpTabEntries * sizeof(uint32_t))};
-  // launched as a programmatic dependent of the planner: read nothing before it has completed
-  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int tid = threadIdx.x, warp = tid >> 5;
   for (int j = tid; j < 256; j += kCtaThreads) {
     sm.th[j] = p.tab.hi[j];
@@ -1685,6 +1686,9 @@ __global__ void __launch_bounds__(kCtaThreads, kAcceptCtasPerSM) accept_kernel(c
     sm.keeper_done = 0;
     sm.abort_ = 0;
   }
+  // launched as a programmatic dependent of the planner: only the kernel's own arguments are read
+  // before it has completed
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __syncthreads();  // the only CTA-wide barrier: set-up
   if (warp < kCW)
     consumers<LT>(p, sm, ring, tab);
