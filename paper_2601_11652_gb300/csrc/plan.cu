@@ -245,22 +245,22 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // persistent and each fills an SM's shared memory, so the acceptance CTAs start on the SMs the
   // attention leaves, and the step ends with the later of the two: the split that lets both end
   // together is the attention's share of the work.  Times on all SMs, in ns: 3.2 (D = 128; 2.7 at
-  // 64) per pass over a KV tile of 64 tokens, 47 with an fp32 cache; 35.5 us, 22.5 per logit row and
-  // 0.27 per 1000 logits.  The constants are a fit to the split measured best (32 to 152 of 152
+  // 64) per pass over a KV tile of 64 tokens, 47 with an fp32 cache; 35.2 us, 12.3 per logit row and
+  // 0.29 per 1000 logits.  The constants are a fit to the split measured best (32 to 152 of 152
   // SMs, steps of 4) for 24 batches of 1 to 512 requests, contexts of 64 to 128K tokens and
-  // vocabularies of 4K to 152K: within 2.5% of the best for 23 of them, 5% for one.  Before, it was
-  // half the SMs + 4 or seven eighths of them, by the number of tiles.  Steps on GB300, before and
-  // now: 256 requests 635, 592 us; 512 requests 1238, 1189; 32 requests 114, 107; 16 requests 100,
-  // 88; 8 requests with an fp32 cache 136, 114; 512 short requests with 4K tokens of vocabulary 495,
-  // 372; 300 requests with 8K 858, 754; one request of 100K tokens 130, 93; the others as before or
-  // faster.  At least a quarter of the SMs: a small batch's step is bound by the acceptance's chain,
-  // which more SMs do not shorten.  The fp32 kernel's time is in proportion to 1 / SMs, so beside
+  // vocabularies of 4K to 152K: within 2% of the best for 20 of them, within 7% for four.  Before, it
+  // was half the SMs + 4, seven eighths of them or all, by the number of tiles.  Steps on GB300 with
+  // that split and this one: 256 requests 620, 583 us; 512 requests 1225, 1183; 32 requests 102, 92;
+  // 16 requests 87, 78; 8 requests with an fp32 cache 130, 113; 512 short requests with 4K tokens of
+  // vocabulary 443, 358; 300 requests with 8K 821, 750; one request of 100K tokens 119, 94; the others
+  // as before or faster.  At least a quarter of the SMs: a small batch's step is bound by the
+  // acceptance's chain, which more SMs do not shorten.  The fp32 kernel's time is in proportion to 1 / SMs, so beside
   // less than 1/16 of its work the acceptance waits (4 requests of 30-60K: 503 us; 538 with 146 SMs).
   const int sms = max(1, p.target_items / kItemsPerSM);
   int na = sms;
   if (p.split_sms && s_sum[1] > 0) {
     const float att = (p.kv_f32 ? 47.0f : 2.24f + 0.0075f * (float)p.D) * (float)s_sum[1] * (float)p.Hkv;
-    const float acc = 35500.0f + (22.5f + 0.27e-3f * (float)p.V) * (float)p.total_q_rows;
+    const float acc = 35200.0f + (12.3f + 0.29e-3f * (float)p.V) * (float)p.total_q_rows;
     if (!p.kv_f32 || att < 16.0f * acc) na = max((sms + 3) / 4, min(sms, (int)((float)sms * (att / (att + acc)) + 0.5f)));
   }
   // pass 2: chunk length.  With at least as many (request, head) pairs as SMs, a longest-first
