@@ -127,11 +127,13 @@ void greedy_slices(const wisp_accept_args *c, int sms, int *slices, int *vps) {
   *slices = (int)((nvec + v - 1) / v);
 }
 
-// Work shape of the acceptance kernel: statistics slices per row (about one item per resident
-// CTA over the batch's rows: more, smaller items cost more in per-item set-up and bookkeeping than
-// they gain in balance: 16 requests 57 us against 62 with two items per CTA, 32 requests 68 against 71; a slice is a whole number of 3-vector chunks per thread), draw tiles (64 vectors: one warp's share of a draw chunk; no tile records when they
-// would exceed tile_budget bytes) and draw slices per row (one item per resident CTA over the batch
-// when it is small, up to two per CTA as it grows; whole chunks of 256 vectors).
+// Work shape of the acceptance kernel: statistics slices per row (about one item per resident CTA
+// over the batch's rows: more, smaller items cost more in per-item set-up and bookkeeping than they
+// gain in balance: 16 requests 57 us against 62 with two items per CTA, 32 requests 68 against 71; a
+// slice is a whole number of 3-vector chunks per thread), draw tiles (64 vectors: one warp's share of
+// a draw chunk; no tile records when they would exceed tile_budget bytes) and draw slices per row (one
+// item per resident CTA over the batch when it is small, up to two per CTA as it grows; whole chunks
+// of 256 vectors).
 constexpr size_t kTileBudget = (size_t)256 << 20;
 constexpr size_t kNoAllocTileBudget = (size_t)4 << 20;
 struct AcceptShape {
@@ -154,21 +156,25 @@ AcceptShape accept_shape(const wisp_accept_args *c, int sms, size_t tile_budget)
     *n = (int)((nvec + v - 1) / v);
   };
   AcceptShape sh;
-  cut(ctas, c->total_q_rows > 0 ? c->total_q_rows : 1, (int64_t)kAcceptThreads * kStatsChunkVecs, &sh.sslices,
-      &sh.svps);
+  // One wave exactly once a row has two slices anyway (three for fp32 rows, whose items take twice as
+  // long): bf16, 16 requests 51.7 -> 49.8 us, fp32 16 requests with two slices 57.1 -> 58.5.
+  const int64_t T = c->total_q_rows > 0 ? c->total_q_rows : 1;
+  cut(ctas / T >= (E == 8 ? 2 : 3) ? ctas / T * T : ctas, T, (int64_t)kAcceptThreads * kStatsChunkVecs, &sh.sslices, &sh.svps);
   // a tile is one warp's 64 vectors of a draw chunk; without room for the records, none
   const int64_t nt = (nvec + 63) / 64;
   const bool tiles = B * nt * (int64_t)sizeof(TileRec) <= (int64_t)tile_budget;
   sh.tile_vecs = tiles ? 64 : 0;
   sh.ntiles = tiles ? (int)nt : 0;
-  // draw slices: one wave of items over the CTAs when the batch is small, up to two waves (and
-  // about three slices per row) as it grows, and at least two per row.  A slice keeps at most
+  // draw slices: one wave of items over the CTAs when the batch is small (rounded down: a few items
+  // more than CTAs take as long as two waves; 20 requests 58 -> 53 us, 64 requests 90 -> 86, 100 requests
+  // 103 -> 96), up to two waves (and about three slices per row) as it grows, and at least two per
+  // row.  A slice keeps at most
   // amb_cap undecided elements; past that the bookkeeper weighs the slice exactly alone, which
   // takes over a millisecond (512 requests, one of whose slices had 9: 1977 us with room for 8,
   // 291 with room for 64)
   sh.amb_cap = tile_budget == kTileBudget ? kAmbPerSlice : kAmbNoAlloc;
-  cut(std::max<int64_t>(2 * B, std::max<int64_t>(ctas, std::min<int64_t>(2 * ctas, 3 * B))), B, kAcceptThreads,
-      &sh.dslices, &sh.vpd);
+  cut(std::max<int64_t>(2 * B, std::max<int64_t>(ctas / B * B, std::min<int64_t>(2 * ctas, 3 * B))), B,
+      kAcceptThreads, &sh.dslices, &sh.vpd);
   return sh;
 }
 
