@@ -1943,7 +1943,7 @@ cudaError_t set_attr() {
 }
 
 template <typename LT>
-cudaError_t launch_t(const AcceptParams &ap, int sms, cudaStream_t s, bool pdl) {
+cudaError_t launch_t(const AcceptParams &ap, int sms, cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3((unsigned)(sms * kAcceptCtasPerSM));
@@ -1956,7 +1956,7 @@ cudaError_t launch_t(const AcceptParams &ap, int sms, cudaStream_t s, bool pdl) 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, accept_kernel<LT>, ap);
 }
 
@@ -1993,8 +1993,8 @@ cudaError_t accept_setup() {
   return e;
 }
 
-cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_t s, bool pdl) {
-  return bf16 ? launch_t<uint16_t>(p, sms, s, pdl) : launch_t<float>(p, sms, s, pdl);
+cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_t s) {
+  return bf16 ? launch_t<uint16_t>(p, sms, s) : launch_t<float>(p, sms, s);
 }
 
 cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, bool level_major, int sms, cudaStream_t s) {

@@ -128,7 +128,7 @@ struct AcceptParams {
 
 cudaError_t accept_setup();  // once per device: kernel attributes, the exp table of the draw
 // the acceptance pass (one persistent kernel; needs the planner's offsets and dispatch order)
-cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_t s, bool pdl);
+cudaError_t accept_launch(const AcceptParams &p, bool bf16, int sms, cudaStream_t s);
 // greedy (temperature 0) variant: one persistent kernel in the planner's dispatch order, or argmax partials of
 // every row and then the walk (two launches; needs only the planner's offsets)
 cudaError_t accept_greedy_launch(const AcceptParams &p, bool bf16, bool level_major, int sms, cudaStream_t s);

@@ -417,7 +417,7 @@ wisp_status launch_accept(const wisp_accept_args *c, void *ws, const Layout &L, 
   wisp_status st = launch_plan(nullptr, c, ws, L, sms, true, s);
   if (st != WISP_OK || c->B == 0) return st;
   const AcceptParams ap = accept_params(c, ws, L, sms, tile_budget);
-  return accept_launch(ap, c->logits_dtype == WISP_BF16, sms, s, true) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
+  return accept_launch(ap, c->logits_dtype == WISP_BF16, sms, s) == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
 }
 
 }  // namespace
@@ -528,7 +528,7 @@ wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args 
   ok = ok && launch_attention(attn, ws, L, s, true) == WISP_OK;
   const bool forked = ok && cudaStreamWaitEvent(sl->side, sl->ev_fork, 0) == cudaSuccess;
   ok = forked && launch_plan_accept(attn, acc, ws, L, sms, sl->side) == WISP_OK;
-  ok = ok && accept_launch(ap, bf, sms, sl->side, false) == cudaSuccess;
+  ok = ok && accept_launch(ap, bf, sms, sl->side) == cudaSuccess;
   // join what was forked even after a failed launch, so that `s` never runs ahead of `side`
   const bool joined = !forked || (cudaEventRecord(sl->ev_join, sl->side) == cudaSuccess &&
                                   cudaStreamWaitEvent(s, sl->ev_join, 0) == cudaSuccess);

@@ -1,6 +1,6 @@
 // attn_tc.cu -- tensor-core paged GQA attention for the verification forward (bf16 KV).
 //
-// Same contract as attn_simt.cu (Sec. 4.4-4.5: request r's k+1 new queries over its
+// Same contract as attn_f32.cu (Sec. 4.4-4.5: request r's k+1 new queries over its
 // L_total = L_cached + L_new paged keys, query j seeing keys 0..c_r + j), built for sm_103a.
 //
 // A verification item has few query rows (g * (k+1), at most 64 per item) and many keys, so the

@@ -441,6 +441,8 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
 // that the attention, which waits for the whole planner grid, does not wait for it).  Reads what
 // plan_kernel's first pass wrote (flags and offsets).
 __global__ void __launch_bounds__(kThreads, 1) plan_accept_kernel(const PlanParams p) {
+  // the acceptance kernel may be placed and set itself up now (it waits for this grid)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ AcceptPlan sh;
   plan_accept_clear(sh);
   const int r = threadIdx.x;
