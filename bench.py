@@ -71,8 +71,8 @@ def accept_bytes(b, L) -> int:
 
 def _launches_per_step(b) -> int:
     """Kernels of this library one wisp_verify_step launches: planner, attention (tensor-core
-    kernel for bf16; SIMT kernel + combine for fp32), acceptance (one persistent kernel)."""
-    return 3 if b.dtype == "bf16" else 4
+    kernel for bf16, CUDA-core kernel for fp32), the acceptance part of the plan, acceptance."""
+    return 4
 
 
 def _peaks():
