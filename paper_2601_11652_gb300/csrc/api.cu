@@ -231,8 +231,10 @@ Layout make_layout(const wisp_attn_args *a, const wisp_accept_args *c, int sms, 
     L.row_rec = take(sizeof(RowRec) * T);
     L.sparts = take(sizeof(SlicePart) * T * sh.sslices);
     L.req_state = take(sizeof(int32_t) * 5 * (size_t)c->B);
-    L.dparts = take(sizeof(DrawPart) * (size_t)c->B * sh.dslices);
-    L.damb = take(sizeof(AmbElem) * (size_t)c->B * sh.dslices * sh.amb_cap);
+    // (one piece: no room is lost between the two in the fixed scratch)
+    const size_t slices = (size_t)c->B * sh.dslices;
+    L.dparts = take((sizeof(DrawPart) + sizeof(AmbElem) * sh.amb_cap) * slices);
+    L.damb = L.dparts + sizeof(DrawPart) * slices;
     L.tiles = take(sizeof(TileRec) * ((size_t)c->B * sh.ntiles + 1));
     L.tcache = c->logits_dtype == WISP_BF16 ? take((size_t)kTabCacheSlots * kExpTabBytes) : 0;
     // the greedy variant's argmax partials (8 bytes per row and warp slice) share the statistics'
