@@ -177,10 +177,10 @@ wisp_status wisp_verify_accept_greedy(const wisp_accept_args *acc, void *workspa
  * acceptance part of the plan) runs on a side stream owned by the library, forked from and
  * joined back into `stream` with events, so work queued on `stream` afterwards sees the whole step
  * finished.  The planner gives the attention its share of the SMs, from the batch's estimated work:
- * the other attention CTAs exit at once and the acceptance pass starts on their SMs (the tokens do not
- * depend on it; attention outputs may differ in their last bits where sequences are cut elsewhere).  Each caller stream gets its own side stream (created on its
- * first step: make that first call before any stream capture), so steps on different streams,
- * with different workspaces, run independently. */
+ * the other attention CTAs exit at once and the acceptance pass starts on their SMs (the results are
+ * those of the two entry points either way, to the bit).  Each caller stream gets its own side stream
+ * (created on its first step: make that first call before any stream capture), so steps on different
+ * streams, with different workspaces, run independently. */
 wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args *acc, void *workspace,
                              size_t workspace_bytes, void *stream);
 

@@ -246,20 +246,24 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // attention leaves, and the step ends with the later of the two: the split that lets both end
   // together is the attention's share of the work.  Times on all SMs, in ns: 3.2 (D = 128; 2.7 at
   // 64) per pass over a KV tile of 64 tokens, 47 with an fp32 cache; 35.2 us, 12.3 per logit row and
-  // 0.29 per 1000 logits.  The constants are a fit to the split measured best (32 to 152 of 152
-  // SMs, steps of 4) for 24 batches of 1 to 512 requests, contexts of 64 to 128K tokens and
-  // vocabularies of 4K to 152K: within 2% of the best for 20 of them, within 7% for four.  Before, it
-  // was half the SMs + 4, seven eighths of them or all, by the number of tiles.  Steps on GB300 with
-  // that split and this one: 256 requests 620, 583 us; 512 requests 1225, 1183; 32 requests 102, 92;
-  // 16 requests 87, 78; 8 requests with an fp32 cache 130, 113; 512 short requests with 4K tokens of
-  // vocabulary 443, 358; 300 requests with 8K 821, 750; one request of 100K tokens 119, 94; the others
-  // as before or faster.  At least a quarter of the SMs: a small batch's step is bound by the
-  // acceptance's chain, which more SMs do not shorten.  The fp32 kernel's time is in proportion to 1 / SMs, so beside
-  // less than 1/16 of its work the acceptance waits (4 requests of 30-60K: 503 us; 538 with 146 SMs).
+  // 0.29 per 1000 logits.  The constants are a fit to the split measured best (32 to 152 of 152 SMs) for
+  // 24 batches of 1 to 512 requests, contexts of 64 to 128K tokens and vocabularies of 4K to 152K.  With
+  // fewer (request, head) pairs than SMs the tensor-core kernel's tiles count 3/2 times and 10 us more: its
+  // sequences are cut into a fixed number of items (pass 2), which cost a merge each and fill a small
+  // share in more rounds (fitted to the best share of 14 such batches).
+  // Steps on GB300 with all SMs for the attention first and with this split: 256 requests 653, 588 us; 512
+  // requests 1266, 1183; 32 requests 116, 92; 16 requests 94, 82; 8 requests with an fp32 cache 123, 109;
+  // 512 short requests with 4K tokens of vocabulary 437, 360; 300 requests with 8K 823, 758; one
+  // request of 100K tokens 123, 103.  At least a quarter of the SMs: a small batch's step is bound by
+  // the acceptance's chain, which more SMs do not shorten.  The fp32 kernel's time is in proportion to
+  // 1 / SMs, so beside less than 1/16 of its work the acceptance waits (4 requests of 30-60K: 503 us; 524
+  // with 144 SMs).
   const int sms = max(1, p.target_items / kItemsPerSM);
+  const bool many_pairs = (int64_t)s_valid * p.Hkv >= sms;
   int na = sms;
   if (p.split_sms && s_sum[1] > 0) {
-    const float att = (p.kv_f32 ? 47.0f : 2.24f + 0.0075f * (float)p.D) * (float)s_sum[1] * (float)p.Hkv;
+    float att = (p.kv_f32 ? 47.0f : 2.24f + 0.0075f * (float)p.D) * (float)s_sum[1] * (float)p.Hkv;
+    if (!p.kv_f32 && !many_pairs) att = 1.5f * att + 10000.0f;
     const float acc = 35200.0f + (12.3f + 0.29e-3f * (float)p.V) * (float)p.total_q_rows;
     if (!p.kv_f32 || att < 16.0f * acc) na = max((sms + 3) / 4, min(sms, (int)((float)sms * (att / (att + acc)) + 0.5f)));
   }
@@ -268,10 +272,11 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // is cut (a split costs a merge of its chunks).  With fewer pairs than SMs, sequences are cut
   // into about kItemsPerSM items per SM.  The fp32 kernel's time also grows with the item's rows, which
   // the order does not see, so it gets items of at most 2/3 of the average (32 requests of 512-4096
-  // tokens: 307 us at 5/4, 290 at 2/3, 302 at 1/2; the tensor-core kernel there: 68, 80, 83 us).
+  // tokens: 307 us at 5/4, 290 at 2/3, 302 at 1/2; the tensor-core kernel there: 68, 80, 83 us).  All SMs
+  // count, also in a step that gives the attention a share of them: where a sequence is cut decides the
+  // last bits of its outputs, and those do not depend on the acceptance's sizes.
   const int64_t work = (int64_t)s_sum[0] * p.Hkv;
-  const bool many_pairs = (int64_t)s_valid * p.Hkv >= na;
-  const int64_t goal = many_pairs ? na : (int64_t)na * kItemsPerSM;
+  const int64_t goal = many_pairs ? sms : p.target_items;
   int64_t chunk = ceil_div(work, goal);
   if (many_pairs) chunk = p.kv_f32 ? chunk - chunk / 3 : chunk + chunk / 4;
   chunk = max64(chunk, kMinChunk);
