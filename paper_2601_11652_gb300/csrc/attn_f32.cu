@@ -150,9 +150,10 @@ __device__ __forceinline__ void item_rows(const AttnParams &p, const WorkItem &w
       }
     }
     // ---- weights against the running maxima; row rho sees key t iff t <= ctx + (row0 + rho) / g
+    // (every row if t <= ctx: no product of g and a whole context, which 32 bits may not hold)
     const int tok = w.t0 + pg * kPage + lb;
-    const int vis0 = tok < w.t1 ? g * (tok - w.ctx) - w.row0 : 0x7fffffff;  // rows >= vis see the key
-    const int vis1 = tok + 8 < w.t1 ? g * (tok + 8 - w.ctx) - w.row0 : 0x7fffffff;
+    const int vis0 = tok < w.t1 ? g * max(tok - w.ctx, 0) - w.row0 : 0x7fffffff;  // rows >= vis see the key
+    const int vis1 = tok + 8 < w.t1 ? g * max(tok + 8 - w.ctx, 0) - w.row0 : 0x7fffffff;
     float pw[RL][2], alpha[RL];
     bool moved = false;
 #pragma unroll

@@ -11,6 +11,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 import oracle  # noqa: E402
+from paper_2601_11652_gb300 import binding as wb  # noqa: E402
 from paper_2601_11652_gb300 import workload as wl  # noqa: E402
 from paper_2601_11652_gb300.device_batch import DeviceBatch  # noqa: E402
 
@@ -52,3 +53,32 @@ def test_step_beside_the_acceptance():
     assert np.max(np.abs(got["out"] - oracle.attention(b))) <= 1e-4
     near = (ref["accept_margin"] < 1e-6) | (ref["sample_margin"] < 1e-9)
     assert np.all(near | ((got["accepted_len"] == ref["accepted_len"]) & (got["next_token"] == ref["next_token"])))
+
+
+def test_group_times_context_past_31_bits():
+    """128 query heads on one KV head and over 2^24 tokens of context: the product of the two does not fit 32
+    bits.  The first 4096 keys carry half of every row's weight and a V of their own."""
+    heads, D, first, rest = 128, 64, 256, 1 << 20  # pages: `first` times block 0, then the blocks 1 .. 63 in turn
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    kc = torch.randn((64, 1, 16, D), generator=gen, device="cuda") * 0.25
+    vc = torch.randn((64, 1, 16, D), generator=gen, device="cuda")
+    q = torch.randn((1, heads, D), generator=gen, device="cuda")
+    q[:, :, 0] = 8.0  # (a score is q k / 8)
+    kc[..., 0] = 0.0
+    kc[0, ..., 0] = float(np.log(rest / first))
+    vc[0] += 1.0
+    table = torch.cat([torch.zeros(first, dtype=torch.int32), 1 + torch.arange(rest, dtype=torch.int32) % 63]).cuda()[None].contiguous()
+    i32 = lambda x: torch.tensor([x], dtype=torch.int32, device="cuda")  # noqa: E731
+    out = torch.empty_like(q)
+    a = wb.make_attn_args(draft_lens=i32(0), context_lens=i32(16 * (first + rest) - 1), block_tables=table, q=q, k_cache=kc,
+                          v_cache=vc, out=out)
+    ws = wb.alloc_workspace(wb.wisp_verify_workspace_size(a, None))
+    wb.wisp_verify_attention(a, ws)
+    torch.cuda.synchronize()
+    assert wb.wisp_verify_get_device_status(ws) == (0, -1)
+    count = torch.bincount(table[0].long(), minlength=64).double().repeat_interleave(16)  # of every key of the pool
+    s = q[0].double() @ kc.view(-1, D).double().T / 8.0
+    w = torch.exp(s - s.max()) * count
+    ref = (w / w.sum(dim=1, keepdim=True)) @ vc.view(-1, D).double()
+    assert float((out[0].double() - ref).abs().max()) <= 1e-4
