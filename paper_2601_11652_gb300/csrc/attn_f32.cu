@@ -168,9 +168,9 @@ __device__ __forceinline__ void item_rows(const AttnParams &p, const WorkItem &w
       alpha[j] = mn == m[j] ? 1.0f : exp2f(m[j] - mn);
       moved |= mn != m[j];
       m[j] = mn;
-      // (a row that sees no key yet has mn = -inf: its weights are zero)
-      pw[j][0] = rho >= vis0 ? exp2f(a - mn) : 0.0f;
-      pw[j][1] = rho >= vis1 ? exp2f(b - mn) : 0.0f;
+      // a key not seen, or with a score of -inf, has weight zero (also while mn is -inf)
+      pw[j][0] = a == -INFINITY ? 0.0f : exp2f(a - mn);
+      pw[j][1] = b == -INFINITY ? 0.0f : exp2f(b - mn);
       l[j] = fmaf(l[j], alpha[j], pw[j][0] + pw[j][1]);
     }
     if (__any_sync(0xffffffffu, moved)) {

@@ -55,6 +55,20 @@ def test_step_beside_the_acceptance():
     assert np.all(near | ((got["accepted_len"] == ref["accepted_len"]) & (got["next_token"] == ref["next_token"])))
 
 
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("B, ctx", [(40, 700), (1, 9000)])  # whole sequences, and chunks whose partials are merged
+def test_keys_of_minus_infinity(D, B, ctx):
+    """Keys whose scores are -inf have weight zero: the first page of every warp, a whole chunk, single keys."""
+    b = wl.make_batch_from_lengths("inf", draft_lens=[5] * B, context_lens=[ctx + i for i in range(B)], Hq=8, Hkv=4, D=D, V=64,
+                                   dtype="f32", sigma=0.5, key=(240, D, B), shuffle_blocks=True)
+    b.q[:, :, 0] = np.abs(b.q[:, :, 0]) + np.float32(0.1)
+    for r in range(B):
+        n = int(b.context_lens[r]) + 6
+        for t in [*range(min(640, n // 2)), n // 2 + 1, n - 20]:
+            b.k_cache[b.block_tables[r, t // 16], :, t % 16, 0] = -np.inf
+    _check(b)
+
+
 def test_group_times_context_past_31_bits():
     """128 query heads on one KV head and over 2^24 tokens of context: the product of the two does not fit 32
     bits.  The first 4096 keys carry half of every row's weight and a V of their own."""
