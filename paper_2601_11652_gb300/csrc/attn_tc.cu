@@ -28,7 +28,8 @@
 //     second the rest; within a group one warp per TMEM lane quadrant, i.e. 32 keys of each tile per
 //     warp: a thread holds one key's scores for the group's rows.  The rows' reference maxima are
 //     those of the item's first tile and stay fixed.  Each thread writes its key's part of the P row
-//     (bf16, MN-major, swizzled: the B operand of the PV product) and keeps its share of every row sum;
+//     (bf16, MN-major, swizzled: the B operand of the PV product) and keeps its share of every row sum.
+//     An item with a P past kMaxP is taken again, its true maxima first: see kMaxP;
 //   * warps 8-11 (epilogue) add the row-sum shares, read O^T from TMEM and write the normalised
 //     output or, for a split item, the (O, m, l) partials; the last chunk of a split
 //     (request, head, row group) to finish merges all its chunks.  This runs while the softmax
@@ -66,9 +67,13 @@ constexpr uint32_t kTmemCols = 256; // S^T[2] at columns 0 / 64, O^T[2] at 128 /
 constexpr long long kWaitCycles = 4000000000LL;  // about two seconds: a wait that long is a failure
 // Largest P = 2^(s - m) an item may hold: m is the maximum of a row's first tile, so later scores may
 // exceed it.  P (bf16), its row sums and O (fp32) keep their relative precision at any exponent; up to
-// 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it is
-// computed again by its epilogue warps (item_exact).
+// 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it
+// writes nothing: the epilogue hands it back to the item loader, which publishes it again for two passes over its keys, S^T alone for the rows' true
+// maxima and then the ordinary one against those: 24 requests of 8192 tokens at 64 query rows, every item taken
+// again, 389 us against 164 (D = 64: 290 against 117).  Whether an item is taken again follows from its
+// own scores alone, so outputs repeat to the bit.
 constexpr float kMaxP = 0x1p64f;
+constexpr int kRedo = 8;            // items waiting to be taken again, at most: those published and undecided, RING + 1
 constexpr uint32_t kAhead = 3;      // the item loader takes the next item when the K producer is this many tiles from
                                     // the end of what is published
 static_assert(kNR == 64, "TMEM and shared-memory layout assume 64 rows per item");
@@ -96,11 +101,11 @@ struct Cfg {
   static constexpr int OFF_RED = OFF_MW + kSoftmaxWarps * 32 * 4;      // float [2][4][64] first-tile maxima per quadrant
   static constexpr int OFF_HL = OFF_RED + 2 * 4 * kNR * 4;             // float [2][4][64] row-sum shares per quadrant
   static constexpr int OFF_HM = OFF_HL + 2 * 4 * kNR * 4;              // float [2][64] row reference maxima
-  static constexpr int OFF_EX = OFF_HM + 2 * kNR * 4;                  // float [128 + 4] item_exact: a block's weights
-  static constexpr int OFF_MISC = OFF_EX + (kBT + 4) * 4;              // tmem base, flags
-  static constexpr int OFF_RING = OFF_MISC + 64;                       // RING x (index, WorkItem)
+  static constexpr int OFF_MISC = OFF_HM + 2 * kNR * 4;                // tmem base, flags, counters
+  static constexpr int OFF_RING = OFF_MISC + 80;                       // RING x (index, passes, WorkItem)
   static constexpr int SMEM = OFF_RING + RING * 64 + 1024;             // + slack to align the base to 1024
   static_assert(SMEM <= 227 * 1024, "shared memory of one CTA on sm_103a");
+  static_assert(RING + 1 <= kRedo && OFF_RING % 16 == 0, "item ring");
   static_assert(OFF_K % 1024 == 0 && OFF_V % 1024 == 0 && OFF_P % 1024 == 0, "swizzled buffers need 1 KB alignment");
 };
 
@@ -185,85 +190,6 @@ __device__ __forceinline__ uint32_t bmax2(uint32_t a, uint32_t b) {  // NaN neve
   return r;
 }
 
-// The whole item again, by the four epilogue warps on the CUDA cores with a running row maximum: the
-// way out for an item whose scores grow past kMaxP times its first tile's maximum (no input of an
-// ordinary model does; one such item takes about a millisecond).  Same output or partials as the main
-// path; a key whose block id is invalid reads as zero, as in the TMA loads.  s_p: kBT + 4 floats.
-// `bar`, `ph`: the epilogue warps' barrier and its phase count; returns the new count, or -1 if a wait
-// gave up.
-template <int D>
-__device__ __noinline__ int item_exact(const AttnParams &p, int it, float *s_p, uint32_t bar, int ph,
-                                       volatile int *abort) {
-  const WorkItem w = p.items[it];
-  const int g = p.Hq / p.Hkv;
-  auto sync = [&]() -> bool {
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(bar);
-    return wait_bar(bar, (ph++) & 1, abort);
-  };
-  const int tid = threadIdx.x & 127, lane = tid & 31, wq = tid >> 5;
-  float *s_w = s_p + kBT;
-  const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
-  const uint16_t *kc = static_cast<const uint16_t *>(p.k_cache), *vc = static_cast<const uint16_t *>(p.v_cache);
-  const int32_t *bt = p.block_tables + (int64_t)w.r * p.max_blocks_per_seq;
-  auto key_at = [&](int t) -> int64_t {
-    const int32_t b = __ldg(bt + t / 16);
-    return b < 0 || b >= p.num_blocks ? -1 : (((int64_t)b * p.Hkv + w.h) * 16 + t % 16) * D;
-  };
-  for (int jr = 0; jr < w.rows; ++jr) {
-    const int rj = w.row0 + jr, jq = rj / g, hh = rj % g;
-    const int64_t o_at = ((int64_t)(w.q0 + jq) * p.Hq + w.h * g + hh) * D;
-    const uint16_t *qr = static_cast<const uint16_t *>(p.q) + o_at;
-    const int end = min(w.t1, w.ctx + jq + 1);
-    float m = -INFINITY, l = 0.0f, acc = 0.0f;
-    for (int t0 = w.t0; t0 < end; t0 += kBT) {
-      float s = -INFINITY;
-      if (t0 + tid < end) {
-        const int64_t at = key_at(t0 + tid);
-        float a = 0.0f;
-        if (at >= 0)
-          for (int d = 0; d < D; ++d) a = fmaf(bf16_bits_to_float(__ldg(qr + d)), bf16_bits_to_float(__ldg(kc + at + d)), a);
-        s = a * scale_log2;
-      }
-      float mx = s;
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      if (lane == 0) s_w[wq] = mx;
-      if (!sync()) return -1;
-      mx = fmaxf(m, fmaxf(fmaxf(s_w[0], s_w[1]), fmaxf(s_w[2], s_w[3])));
-      const float f = m == mx ? 1.0f : ptx::ex2(m - mx);
-      const float e = t0 + tid < end ? ptx::ex2(s - mx) : 0.0f;
-      m = mx;
-      l = fmaf(l, f, e);
-      s_p[tid] = e;
-      if (!sync()) return -1;
-      acc *= f;
-      if (tid < D) {
-        for (int i = 0; i < kBT && t0 + i < end; ++i) {
-          const int64_t at = key_at(t0 + i);
-          if (at >= 0) acc = fmaf(s_p[i], bf16_bits_to_float(__ldg(vc + at + tid)), acc);
-        }
-      }
-      if (!sync()) return -1;
-    }
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (lane == 0) s_w[wq] = l;
-    if (!sync()) return -1;
-    l = s_w[0] + s_w[1] + s_w[2] + s_w[3];
-    if (!sync()) return -1;
-    if (tid < D) {
-      if (w.poff < 0)
-        static_cast<uint16_t *>(p.out)[o_at + tid] = __bfloat16_as_ushort(__float2bfloat16_rn(acc / l));
-      else
-        __stcg(p.partials + w.poff + (int64_t)jr * D + tid, acc);
-    }
-    if (w.poff >= 0 && tid == 0) {
-      __stcg(p.partials + w.poff + w.rows * D + jr, m);
-      __stcg(p.partials + w.poff + w.rows * D + w.rows + jr, l);
-    }
-  }
-  return ph;
-}
-
 }  // namespace
 
 template <int D>
@@ -279,17 +205,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   const Bars<D> B{sbase + C::OFF_BAR};
   float *s_mw = reinterpret_cast<float *>(smem + C::OFF_MW);
   float *s_red = reinterpret_cast<float *>(smem + C::OFF_RED);
-  float *s_ex = reinterpret_cast<float *>(smem + C::OFF_EX);
   float *s_hl = reinterpret_cast<float *>(smem + C::OFF_HL);
   float *s_hm = reinterpret_cast<float *>(smem + C::OFF_HM);
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + C::OFF_MISC);
   volatile int *s_abort = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 4);
   volatile int *s_last = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 8);
   volatile uint32_t *s_issued = reinterpret_cast<volatile uint32_t *>(smem + C::OFF_MISC + 12);  // K tiles issued
-  volatile int *s_ovf = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 16);  // [2] per O buffer: P past kMaxP
+  // items decided by the epilogue (to be taken again, or not), and those to be taken again: their number and a ring
+  // of their indexes.  Written by one lane of warp 8, read by one lane of warp 2.
+  volatile uint32_t *s_decided = reinterpret_cast<volatile uint32_t *>(smem + C::OFF_MISC + 16);
+  volatile uint32_t *s_nredo = reinterpret_cast<volatile uint32_t *>(smem + C::OFF_MISC + 20);
+  volatile int *s_redo = reinterpret_cast<volatile int *>(smem + C::OFF_MISC + 24);
+  volatile uint8_t *s_ovf = smem + C::OFF_MISC + 64;  // [2][8] per O buffer and softmax warp: the item must be taken again
   struct RingSlot {
     int it;
-    int pad[3];
+    int passes;  // over the keys: 1, or 2 for an item that is taken again
+    int pad[2];
     WorkItem w;
   };
   static_assert(sizeof(RingSlot) <= 64, "item ring slot");
@@ -331,7 +262,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::mbar_init(B.fin(), kThreads / 32);
     *s_issued = 0;
     *s_abort = 0;
-    s_ovf[0] = s_ovf[1] = 0;
+    *s_decided = 0;
+    *s_nredo = 0;
     ptx::fence_mbar_init();
   }
   if (warp == 0 && lane == 0) {
@@ -382,6 +314,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const WorkItem w = s_ring[slot].w;
+      const int passes = is_k ? s_ring[slot].passes : 1;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
@@ -393,9 +326,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       int cur = fetch(0), nxt = fetch(32);  // block ids of tiles t..t+3 and t+4..t+7
       const int ntiles = (w.t1 - w.t0 + kBT - 1) / kBT;
-      for (int t = 0; t < ntiles; ++t, ++tile_n) {
+      for (int t = 0, left = passes * ntiles; left > 0; ++t, --left, ++tile_n) {
         if (is_k && lane == 0) *s_issued = tile_n;
-        if (t > 0 && (t & 3) == 0) {
+        if (t == ntiles) {  // the keys once more
+          t = 0;
+          cur = fetch(0);
+          nxt = fetch(32);
+        } else if (t > 0 && (t & 3) == 0) {
           cur = nxt;
           nxt = fetch(32 * ((t >> 2) + 1));
         }
@@ -441,13 +378,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp == 2) {
     // ------------------------------------------------------------------ item loader
-    uint32_t published = 0;  // tiles of the items published so far
+    uint32_t published = 0;           // K tiles of the items published so far
+    uint32_t items = 0, redone = 0;   // (lane 0) items published, and those of them taken again
+    bool left = true;                 // (lane 0) the plan may have items left
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
       // next valid work item: publish it to the other warps.  Items are taken just in time, so the work
       // counter balances the CTAs to the end, but early enough to hide the way from the claim to the first
       // load: when the K producer is kAhead tiles from the end of what is published, which for items of
-      // a tile or two means several items ahead.
+      // a tile or two means several items ahead.  Items to be taken again go first.  The end is published
+      // once every item is decided, before the last one's epilogue.
       const int slot = j % C::RING;
       for (const long long g0 = clock64(); published > *s_issued + kAhead;) {
         if (*s_abort || clock64() - g0 > kWaitCycles) {
@@ -461,17 +401,45 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!wait_bar(B.it_empty(slot), ((j / C::RING) & 1) ^ 1, s_abort)) { ok = false; break; }
       int tiles = 0;
       if (lane == 0) {
-        int it;
+        int it = -1, passes = 1;
         WorkItem w;
-        do {
-          it = atomicAdd(&p.header_mut->next_item, 1);
-          if (it >= n_items) { it = -1; break; }
-          w = p.items[it];
-        } while (!item_ok(p, w));
+        uint32_t seen = *s_decided;
+        for (long long g0 = clock64();;) {
+          const uint32_t decided = *s_decided;
+          __threadfence_block();  // what was decided before it, too
+          if (redone != *s_nredo) {
+            __threadfence_block();
+            it = s_redo[redone++ % kRedo];
+            w = p.items[it];
+            passes = 2;
+            break;
+          }
+          if (left) {
+            do {
+              it = atomicAdd(&p.header_mut->next_item, 1);
+              if (it >= n_items) { it = -1; break; }
+              w = p.items[it];
+            } while (!item_ok(p, w));
+            if (it >= 0) break;
+            left = false;
+          } else if (decided == items) {
+            break;
+          } else {
+            if (decided != seen) g0 = clock64();
+            seen = decided;
+            if (*s_abort || clock64() - g0 > kWaitCycles) {
+              *s_abort = 1;
+              break;
+            }
+            __nanosleep(32);
+          }
+        }
         s_ring[slot].it = it;
         if (it >= 0) {
           s_ring[slot].w = w;
-          tiles = (w.t1 - w.t0 + kBT - 1) / kBT;
+          s_ring[slot].passes = passes;
+          tiles = passes * ((w.t1 - w.t0 + kBT - 1) / kBT);
+          ++items;
         }
         ptx::mbar_arrive(B.it_full(slot));
       }
@@ -480,6 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // no item left for this CTA: a kernel launched after this one as a programmatic
         // dependent may be scheduled; it still waits for this grid to finish
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        ok = !*s_abort;
         break;
       }
       published += tiles;
@@ -547,10 +516,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const int rows = s_ring[slot].w.rows, ntok = s_ring[slot].w.t1 - s_ring[slot].w.t0;
+      const int passes = is_s ? s_ring[slot].passes : 1;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
-      const int nt = (ntok + kBT - 1) / kBT;
+      const int nt = passes * ((ntok + kBT - 1) / kBT);
       const int nrow = (rows + 15) / 16 * 16;  // the MMA's N: rows rounded up to 16
       if (is_s) {
         // S^T(n): K(n) has landed, the item's Q is loaded, the TMEM tile has been read
@@ -642,6 +612,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const WorkItem w = s_ring[slot].w;
+      const int passes = s_ring[slot].passes;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
@@ -649,18 +620,22 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t o_col = 128 + ob * kNR;
       // the softmax warps' hand-over and the item's last PV
       if (!wait_bar(B.ep_full(ob), (li >> 1) & 1, s_abort)) { ok = false; break; }
+      const bool again = passes == 1 && *reinterpret_cast<volatile unsigned long long *>(s_ovf + 8 * ob) != 0;
+      if (warp == 8 && lane == 0) {
+        const uint32_t nr = *s_nredo;
+        if (again) {
+          s_redo[nr % kRedo] = it;
+          __threadfence_block();
+          *s_nredo = nr + 1;
+          __threadfence_block();
+        }
+        *s_decided = *s_decided + 1;
+      }
       if (!wait_bar(B.o_done(ob), (li >> 1) & 1, s_abort)) { ok = false; break; }
       ++li;
       ptx::tc_fence_after();
       const int nc = (w.rows + 31) / 32;
-      const bool ovf = s_ovf[ob] != 0;
-      if (ovf) {  // (uniform over the four warps: set before the hand-over, cleared below)
-        const int ph = item_exact<D>(p, it, s_ex, B.egrp(), (int)(gph & 1), s_abort);
-        if (ph < 0) { ok = false; break; }
-        gph = (uint32_t)ph;
-        if (warp == 8 && lane == 0) s_ovf[ob] = 0;
-      }
-      for (int c = 0; c < nc && !ovf; ++c) {
+      for (int c = 0; c < nc && !again; ++c) {
         uint32_t x[32];  // O^T[d][rows 32c..]
         ptx::tmem_ld32(tmem + lane_addr + o_col + 32 * c, x);
         ptx::tmem_wait_ld();
@@ -706,7 +681,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) ptx::mbar_arrive(B.o_empty(ob));
 
       // ---- split item: the last chunk of this (request, head, row group) to finish merges all ----
-      if (w.poff >= 0) {
+      if (w.poff >= 0 && !again) {
         __threadfence();
         if (!group_sync()) { ok = false; break; }
         if (warp == 8 && lane == 0) {
@@ -739,7 +714,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
     const float2 scale2 = make_float2(scale_log2, scale_log2);
     float *mw = s_mw + (grp * 4 + qd) * 32;   // minus the rows' references, this warp's copy
-    uint32_t n = 0;                           // tiles so far
+    uint32_t n = 0;                           // P tiles so far
+    uint32_t ns = 0;                          // S^T tiles so far: an item that is taken again has two per P tile
     int li = 0;                               // items so far: item li accumulates into O buffer li & 1
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
@@ -747,7 +723,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!wait_bar(B.it_full(slot), (j / C::RING) & 1, s_abort)) { ok = false; break; }
       const int it = s_ring[slot].it;
       const int t0 = s_ring[slot].w.t0, t1 = s_ring[slot].w.t1, rows = s_ring[slot].w.rows;
-      const int ctx = s_ring[slot].w.ctx, row0 = s_ring[slot].w.row0;
+      const int ctx = s_ring[slot].w.ctx, row0 = s_ring[slot].w.row0, passes = s_ring[slot].passes;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(B.it_empty(slot));
       if (it < 0) break;
@@ -761,16 +737,19 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int i = 0; i < 16; ++i) lp[i] = make_float2(0.0f, 0.0f);
       uint32_t pmax = 0;        // largest P so far (two bf16 lanes)
-      float mref = -INFINITY;   // lane i: row r0 + i's reference (-inf: no key visible)
-      for (int t = 0; t < ntiles && ok; ++t, ++n) {
-        const int sb = n & 1;
-        if (!wait_bar(B.s_full(sb), (n >> 1) & 1, s_abort)) { ok = false; break; }
+      float mref = -INFINITY;   // lane i: row r0 + i's maximum so far, then its reference (-inf: no key visible)
+      // tiles whose maxima are still to be taken: 1, the first, or for an item that is taken again all of them,
+      // counted up to 0, in a pass of their own
+      int pre = passes == 2 ? -ntiles : 1;
+      for (int t = 0; t < ntiles; ++ns) {
+        const int sb = ns & 1;
+        if (!wait_bar(B.s_full(sb), (ns >> 1) & 1, s_abort)) { ok = false; break; }
         ptx::tc_fence_after();
         uint32_t x[2][16];
         ptx::tmem_ld16(tmem + lane_addr + sb * kNR + r0, x[0]);
         if (nu > 2) ptx::tmem_ld16(tmem + lane_addr + sb * kNR + r0 + 16, x[1]);
         ptx::tmem_wait_ld();
-        // S^T(n) is in registers: its TMEM tile may be overwritten by S^T(n + 2)
+        // the tile is in registers: it may be overwritten by the S^T after next
         ptx::tc_fence_before();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(B.s_empty(sb));
@@ -785,31 +764,39 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 32; ++i)
             if (!(seen & (1u << i))) x[i >> 4][i & 15] = 0xff800000u;
         }
-        if (t == 0) {
-          // references: exact row maxima of the tile, over this warp's 32 keys, then over the group's
-          // four quadrants.  Padding rows get +inf (P = 0), rows without a visible key 0 (P = 0: all
-          // their scores are -inf).  s_red alternates between items: a warp that writes it for item
+        if (pre != 0) {
+          const bool apart = pre < 0;
+          // exact row maxima over this warp's 32 keys, and after the last such tile over the group's four
+          // quadrants: the references.  Padding rows get +inf (P = 0), rows without a visible key 0 (P = 0:
+          // all their scores are -inf).  s_red alternates between items: a warp that writes it for item
           // li + 2 has passed the barrier of item li + 1, where every reader of item li has arrived.
-          float wm = -INFINITY;  // lane i: row r0 + i's maximum over this warp's keys
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             if (u < nu) {
 #pragma unroll
               for (int i = 8 * u; i < 8 * u + 8; ++i) {
                 const float rm = ptx::warp_max(__uint_as_float(x[i >> 4][i & 15]));
-                if (lane == i) wm = rm;
+                if (lane == i) mref = fmaxf(mref, rm);
               }
             }
           }
-          float *red = s_red + (li & 1) * 4 * kNR + r0 + lane;
-          if (lane < half) red[qd * kNR] = wm;
-          __syncwarp();
-          if (lane == 0) ptx::mbar_arrive(B.red(grp));
-          if (!wait_bar(B.red(grp), li & 1, s_abort)) { ok = false; break; }
-          if (lane < half)
-            mref = fmaxf(fmaxf(red[0], red[kNR]), fmaxf(red[2 * kNR], red[3 * kNR])) * scale_log2;
-          mw[lane] = r0 + lane >= rows || lane >= half ? -INFINITY : mref == -INFINITY ? 0.0f : -mref;
-          __syncwarp();
+          pre += apart ? 1 : -1;
+          if (pre == 0) {
+            float *red = s_red + (li & 1) * 4 * kNR + r0 + lane;
+            if (lane < half) red[qd * kNR] = mref;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(B.red(grp));
+            if (!wait_bar(B.red(grp), li & 1, s_abort)) { ok = false; break; }
+            if (lane < half)
+              mref = fmaxf(fmaxf(red[0], red[kNR]), fmaxf(red[2 * kNR], red[3 * kNR])) * scale_log2;
+            const bool pad = r0 + lane >= rows || lane >= half;
+            mw[lane] = pad ? -INFINITY : mref == -INFINITY ? 0.0f : -mref;
+            __syncwarp();
+          }
+          if (apart) {
+            t = pre == 0 ? 0 : t + 1;
+            continue;
+          }
         }
         // P buffer n % NP is free again once PV(n - NP) is done; PV(n) needs the P(n) about to be
         // published, so the parity is exact
@@ -848,6 +835,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(B.p_full(pbuf));
+        ++t;
+        ++n;
       }
       if (!ok) break;
       // ---- hand the item over to the epilogue warps: this quadrant's share of each row sum of
@@ -860,13 +849,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         ls[2 * i + 1] = lp[i].y;
       }
       const float lsh = warp_transpose_sum(ls, lane);
-      const bool ovf = __any_sync(0xffffffffu, fmaxf(__uint_as_float(pmax << 16), __uint_as_float(pmax & 0xffff0000u)) > kMaxP);
+      const bool ovf =
+          __any_sync(0xffffffffu, fmaxf(__uint_as_float(pmax << 16), __uint_as_float(pmax & 0xffff0000u)) > kMaxP);
       if (!wait_bar(B.o_empty(ob), ((li >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
       if (lane < half) {
         s_hl[(ob * 4 + qd) * kNR + r0 + lane] = lsh;
         if (qd == 0) s_hm[ob * kNR + r0 + lane] = mref;
       }
-      if (ovf && lane == 0) s_ovf[ob] = 1;
+      if (lane == 0) s_ovf[8 * ob + 4 * grp + qd] = ovf ? 1 : 0;
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(B.ep_full(ob));
       ++li;
