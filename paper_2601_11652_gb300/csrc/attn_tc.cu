@@ -67,8 +67,9 @@ constexpr uint32_t kTmemCols = 256; // S^T[2] at columns 0 / 64, O^T[2] at 128 /
 constexpr long long kWaitCycles = 4000000000LL;  // about two seconds: a wait that long is a failure
 // Largest P = 2^(s - m) an item may hold: m is the maximum of a row's first tile, so later scores may
 // exceed it.  P (bf16), its row sums and O (fp32) keep their relative precision at any exponent; up to
-// 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it
-// writes nothing: the epilogue hands it back to the item loader, which publishes it again for two passes over its keys, S^T alone for the rows' true
+// 2^64 nothing comes near the fp32 range (2^64 x 2^30 keys x |V| < 2^33).  An item that goes past it, or
+// that has a row whose first tile scores -inf throughout, writes nothing: the epilogue hands it back to
+// the item loader, which publishes it again for two passes over its keys, S^T alone for the rows' true
 // maxima and then the ordinary one against those: 24 requests of 8192 tokens at 64 query rows, every item taken
 // again, 389 us against 164 (D = 64: 290 against 117).  Whether an item is taken again follows from its
 // own scores alone, so outputs repeat to the bit.
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float2 lp[16];  // this thread's (key's) share of every row sum of the group
 #pragma unroll
       for (int i = 0; i < 16; ++i) lp[i] = make_float2(0.0f, 0.0f);
-      uint32_t pmax = 0;        // largest P so far (two bf16 lanes)
+      uint32_t pmax = 0;        // largest P so far (two bf16 lanes); +inf too for a row that sees keys of -inf only so far
       float mref = -INFINITY;   // lane i: row r0 + i's maximum so far, then its reference (-inf: no key visible)
       // tiles whose maxima are still to be taken: 1, the first, or for an item that is taken again all of them,
       // counted up to 0, in a pass of their own
@@ -791,6 +792,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               mref = fmaxf(fmaxf(red[0], red[kNR]), fmaxf(red[2 * kNR], red[3 * kNR])) * scale_log2;
             const bool pad = r0 + lane >= rows || lane >= half;
             mw[lane] = pad ? -INFINITY : mref == -INFINITY ? 0.0f : -mref;
+            if (!pad && mref == -INFINITY && g * max(t0 - ctx, 0) <= row0 + r0 + lane) pmax = 0x7F80u;
             __syncwarp();
           }
           if (apart) {

@@ -122,6 +122,20 @@ def test_chunks_on_both_sides_of_the_limit(D):
 
 
 @pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("B, ctx", [(40, 700), (1, 9000)])
+def test_keys_of_minus_infinity(D, B, ctx):
+    """Keys whose scores are -inf have weight zero, also where an item's first 128 keys or all of them are such."""
+    b = wl.make_batch_from_lengths("inf", draft_lens=[5] * B, context_lens=[ctx + i for i in range(B)], Hq=8, Hkv=4, D=D, V=64,
+                                   dtype="bf16", sigma=0.5, key=(241, D, B), shuffle_blocks=True)
+    b.q[:, :, 0] = wl.f32_to_bf16_bits(np.abs(wl.bf16_bits_to_f32(b.q[:, :, 0])) + np.float32(0.1))
+    for r in range(B):
+        n = int(b.context_lens[r]) + 6
+        for t in [*range(min(640, n // 2)), n // 2 + 1, n - 20]:
+            b.k_cache[b.block_tables[r, t // 16], :, t % 16, 0] = 0xFF80
+    _check(b)
+
+
+@pytest.mark.parametrize("D", [64, 128])
 @pytest.mark.parametrize("B, ctx", [(24, 8192), (2, 60000)])
 def test_growing_scores_cost_a_few_passes(D, B, ctx):
     """Every item's scores pass the limit: 64 query rows, 64 tiles an item (25 where sequences are cut).  Three
