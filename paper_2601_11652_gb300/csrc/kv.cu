@@ -181,6 +181,9 @@ __global__ void __launch_bounds__(kThreads) __cluster_dims__(kReserveCtas, 1, 1)
     }
     __syncthreads();  // s_before and s_q0 are rewritten by the next 1024 requests
   }
+  // rows past the requests' (total_rows larger than the sum of the lengths): nobody's
+  for (int64_t x = carry_rows + blockIdx.x * kThreads + threadIdx.x; x < p.total_rows; x += kReserveCtas * kThreads)
+    p.row_req[x] = -1;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *p.free_count = (int32_t)(F - taken);
     if (carry_rows != p.total_rows) atomicCAS(&p.status->code, 0, (int32_t)WISP_DEV_BAD_LENGTH);
