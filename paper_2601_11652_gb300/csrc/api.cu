@@ -426,7 +426,8 @@ wisp_status launch_accept(const wisp_accept_args *c, void *ws, const Layout &L, 
 
 // Workspace of wisp_verify_accept_noalloc: status word, per-request offsets, flags and state,
 // planner header, the dispatch order and statistics of every logit row, the draw's slice totals.
-// 16 MiB holds them for batches of up to kNoAllocMaxBatch requests and kNoAllocMaxRows logit rows.
+// 16 MiB holds them for batches of up to kNoAllocMaxBatch requests and kNoAllocMaxRows logit rows
+// (about 13 MB at both limits); the tile records get what is left, or none.
 constexpr size_t kNoAllocScratchBytes = 16 << 20;
 constexpr int kNoAllocMaxBatch = 8192;
 constexpr int kNoAllocMaxRows = 131072;
@@ -435,6 +436,12 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 namespace {
 
 void *g_noalloc_ptr[kMaxDevices];  // device address of g_noalloc_scratch, per device
+
+// Room for the tile records in the scratch (without them the draw's finish scans its whole slice).
+size_t noalloc_tile_budget(const wisp_accept_args *c, int sms) {
+  const size_t rest = make_layout(nullptr, c, sms, 0).total;
+  return rest < kNoAllocScratchBytes ? std::min(kNoAllocTileBudget, kNoAllocScratchBytes - rest) : 0;
+}
 
 // Address of the scratch array on the current device `dev`, looked up once (under g_mu).
 wisp_status noalloc_scratch(int dev, void **out) {
@@ -560,13 +567,14 @@ wisp_status wisp_verify_accept_noalloc(const wisp_accept_args *acc, void *stream
   if (acc->B > kNoAllocMaxBatch || acc->total_q_rows > kNoAllocMaxRows) return WISP_ERR_UNSUPPORTED;
   int dev = 0, sms = 0;
   if ((st = device_setup(&dev, &sms)) != WISP_OK) return st;
-  const Layout L = make_layout(nullptr, acc, sms, kNoAllocTileBudget);
+  const size_t tile_budget = noalloc_tile_budget(acc, sms);
+  const Layout L = make_layout(nullptr, acc, sms, tile_budget);
   if (L.total > kNoAllocScratchBytes) return WISP_ERR_UNSUPPORTED;
   void *ws = nullptr;
   if ((st = noalloc_scratch(dev, &ws)) != WISP_OK) return st;
   // the planner clears the status word and the launch's counters and per-row / per-request state
   // (everything that must start at zero) on `stream` first
-  return launch_accept(acc, ws, L, sms, static_cast<cudaStream_t>(stream), kNoAllocTileBudget);
+  return launch_accept(acc, ws, L, sms, static_cast<cudaStream_t>(stream), tile_budget);
 }
 
 const char *wisp_verify_status_string(wisp_status s) {
