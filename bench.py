@@ -87,7 +87,7 @@ def _peaks():
 
 # the sources each profiled kernel is built from (its launch set-up in api.cu included)
 KERNEL_SOURCES = {
-    "attention": ("api.cu", "attn.cuh", "attn_tc.cu", "common.cuh", "plan.cu", "plan.cuh", "sm100_ptx.cuh"),
+    "attention": ("api.cu", "attn.cuh", "attn_merge.cuh", "attn_tc.cu", "common.cuh", "plan.cu", "plan.cuh", "sm100_ptx.cuh"),
     "accept": ("accept.cu", "accept.cuh", "api.cu", "common.cuh", "plan.cu", "plan.cuh", "sm100_ptx.cuh"),
 }
 

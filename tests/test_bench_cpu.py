@@ -2,9 +2,11 @@
 that decide whether a committed ncu summary still describes the sources, the clock summary -- and
 the reference arm's JSON line."""
 import os
+import re
 import shutil
 
 import numpy as np
+import pytest
 
 import bench
 from paper_2601_11652_gb300 import workload as wl
@@ -35,6 +37,21 @@ def _copy_sources(tmp_path):
     shutil.copytree(os.path.join(bench.ROOT, "paper_2601_11652_gb300", "csrc"),
                     root / "paper_2601_11652_gb300" / "csrc")
     return root
+
+
+@pytest.mark.parametrize("kernel, unit", [("attention", "attn_tc.cu"), ("accept", "accept.cu")])
+def test_kernel_sources_cover_every_include(kernel, unit):
+    """A change in any header of csrc/ that a profiled kernel or its planner includes makes its summary stale."""
+    csrc = os.path.join(bench.ROOT, "paper_2601_11652_gb300", "csrc")
+    seen, todo = set(), [unit, "plan.cu"]
+    while todo:
+        name = todo.pop()
+        if name in seen or not os.path.exists(os.path.join(csrc, name)):
+            continue
+        seen.add(name)
+        with open(os.path.join(csrc, name)) as f:
+            todo += re.findall(r'#include "([^"]+)"', f.read())
+    assert seen <= set(bench.KERNEL_SOURCES[kernel])
 
 
 def test_kernel_sources_exist():
