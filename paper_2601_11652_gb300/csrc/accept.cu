@@ -619,8 +619,8 @@ __device__ void ensure_table(float m, Sm &sm, Tab tab, uint32_t &ph, const Accep
 }
 
 // The E weights of one vector: round(2^56 exp(z - m)).  From the table for bf16 values in its
-// range (almost every logit); the others (|z| < 2^-16, |z| >= 64, +-0, a table not given) directly,
-// entered once per vector that needs it.
+// range (almost every logit); the others (|z| < 2^-16, |z| >= 64, +-0) directly, entered once per
+// vector that needs it.
 template <typename LT>
 __device__ __forceinline__ void weights(const uint4 &w, float m, const Sm &sm, Tab tab,
                                         unsigned long long (&fx)[LTraits<LT>::E]);
@@ -630,18 +630,15 @@ __device__ __noinline__ unsigned long long weight_direct1(uint32_t bits, float m
 template <>
 __device__ __forceinline__ void weights<uint16_t>(const uint4 &w, float m, const Sm &sm, Tab tab,
                                                   unsigned long long (&fx)[8]) {
-  uint32_t dmax = 0xFFFFFFFFu;
-  if (tab.lo) {
-    dmax = 0;
+  uint32_t dmax = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint32_t u = (i >> 1) == 0 ? w.x : (i >> 1) == 1 ? w.y : (i >> 1) == 2 ? w.z : w.w;
-      const uint32_t bits = (i & 1) ? (u >> 16) : (u & 0xFFFFu);
-      uint32_t d;
-      const uint32_t e = exp_tab_entry(bits, d);
-      dmax = max(dmax, d);
-      fx[i] = ((unsigned long long)tab.hi[e] << 32) | tab.lo[e];
-    }
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t u = (i >> 1) == 0 ? w.x : (i >> 1) == 1 ? w.y : (i >> 1) == 2 ? w.z : w.w;
+    const uint32_t bits = (i & 1) ? (u >> 16) : (u & 0xFFFFu);
+    uint32_t d;
+    const uint32_t e = exp_tab_entry(bits, d);
+    dmax = max(dmax, d);
+    fx[i] = ((unsigned long long)tab.hi[e] << 32) | tab.lo[e];
   }
   if (dmax >= (uint32_t)kExpTabHalf) {
 #pragma unroll
@@ -650,7 +647,7 @@ __device__ __forceinline__ void weights<uint16_t>(const uint4 &w, float m, const
       const uint32_t bits = (i & 1) ? (u >> 16) : (u & 0xFFFFu);
       uint32_t d;
       exp_tab_entry(bits, d);
-      if (!tab.lo || d >= (uint32_t)kExpTabHalf) fx[i] = weight_direct1(bits, m, sm);
+      if (d >= (uint32_t)kExpTabHalf) fx[i] = weight_direct1(bits, m, sm);
     }
   }
 }
@@ -659,6 +656,12 @@ __device__ __forceinline__ void weights<float>(const uint4 &w, float m, const Sm
                                                unsigned long long (&fx)[4]) {
   #pragma unroll
   for (int i = 0; i < 4; ++i) fx[i] = exp_fix_inline(vec_elem<float>(w, i), m, sm.th, sm.tl);
+}
+// The same without a table.
+template <typename LT>
+__device__ __forceinline__ void weights_direct(const uint4 &w, float m, const Sm &sm, unsigned long long (&fx)[LTraits<LT>::E]) {
+#pragma unroll
+  for (int i = 0; i < LTraits<LT>::E; ++i) fx[i] = exp_fix_direct(vec_elem<LT>(w, i), m, sm.th, sm.tl);
 }
 
 // A fixed-point weight (units 2^-56, at most 2^56) as a float, within 2^-23 of its value relative:
@@ -701,10 +704,10 @@ __device__ __noinline__ double warp_scan(double v) {
 // p - q by an fp32 test with a 2^-20 margin, else in double.
 template <typename LT>
 __device__ __forceinline__ double vec_weight(const uint4 &w, const float *q, bool residual, float m, double Zu,
-                                             const Sm &sm, Tab tab) {
+                                             const Sm &sm) {
   constexpr int E = LTraits<LT>::E;
   unsigned long long fx[E];
-  weights<LT>(w, m, sm, tab, fx);
+  weights_direct<LT>(w, m, sm, fx);
   const float Zf = (float)(Zu * 0x1p-56);
   const float zh = Zf * (1.0f + 0x1p-20f), zl = Zf * (1.0f - 0x1p-20f);
   unsigned long long sp = 0;
@@ -1132,7 +1135,7 @@ __device__ double warp_range_weight(const AcceptParams &p, const Sm &sm, const L
     #pragma unroll
     for (int i = 0; i < E; ++i) q[i] = 0.0f;
     if (qrow) load_q<E>(qrow, vi * E, p.V, p.vec_q != 0, q);
-    acc += vec_weight<LT>(w, q, qrow != nullptr, m, Zu, sm, Tab{nullptr, nullptr});
+    acc += vec_weight<LT>(w, q, qrow != nullptr, m, Zu, sm);
   }
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   return acc;

@@ -312,7 +312,7 @@ PlanParams plan_params(const wisp_attn_args *a, const wisp_accept_args *c, void 
   return pp;
 }
 
-wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L, cudaStream_t s, bool pdl) {
+wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L, cudaStream_t s) {
   AttnParams ap;
   ap.B = a->B;
   ap.Hq = a->Hq;
@@ -327,7 +327,6 @@ wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L,
   ap.v_cache = a->v_cache;
   ap.out = a->out;
   ap.status = at<DeviceStatus>(ws, L.status);
-  ap.req_flag = at<int32_t>(ws, L.req_flag);
   ap.req_chunks = at<int32_t>(ws, L.req_chunks);
   ap.header = at<PlanHeader>(ws, L.plan_header);
   ap.header_mut = at<PlanHeader>(ws, L.plan_header);
@@ -338,7 +337,7 @@ wisp_status launch_attention(const wisp_attn_args *a, void *ws, const Layout &L,
   // persistent kernels, one CTA per SM: the work counter lives in the plan header written by the planner
   // on this stream, and split items are merged inside the kernel by the last chunk to finish
   const int grid = (int)(L.max_items < L.target_items / kItemsPerSM ? L.max_items : L.target_items / kItemsPerSM);
-  const cudaError_t e = a->qkv_dtype == WISP_BF16 ? attn_tc_launch(ap, grid, s, pdl) : attn_f32_launch(ap, grid, s, pdl);
+  const cudaError_t e = a->qkv_dtype == WISP_BF16 ? attn_tc_launch(ap, grid, s) : attn_f32_launch(ap, grid, s);
   return e == cudaSuccess ? WISP_OK : WISP_ERR_CUDA;
 }
 
@@ -480,7 +479,7 @@ wisp_status wisp_verify_attention(const wisp_attn_args *attn, void *ws, size_t w
   if ((st = launch_plan(attn, nullptr, ws, L, sms, false, s)) != WISP_OK) return st;
   if (attn->B == 0) return WISP_OK;
   // alone on the stream after the planner: the attention CTAs set up while the planner runs
-  return launch_attention(attn, ws, L, s, true);
+  return launch_attention(attn, ws, L, s);
 }
 
 wisp_status wisp_verify_accept(const wisp_accept_args *acc, void *ws, size_t ws_bytes, void *stream) {
@@ -534,7 +533,7 @@ wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args 
   // the attention is enqueued first, so that its CTAs take the SMs first; the acceptance part of
   // the plan and the acceptance CTAs follow on the side stream, on the SMs the attention leaves
   bool ok = cudaEventRecord(sl->ev_fork, s) == cudaSuccess;
-  ok = ok && launch_attention(attn, ws, L, s, true) == WISP_OK;
+  ok = ok && launch_attention(attn, ws, L, s) == WISP_OK;
   const bool forked = ok && cudaStreamWaitEvent(sl->side, sl->ev_fork, 0) == cudaSuccess;
   ok = forked && launch_plan_accept(attn, acc, ws, L, sms, sl->side) == WISP_OK;
   ok = ok && accept_launch(ap, bf, sms, sl->side) == cudaSuccess;

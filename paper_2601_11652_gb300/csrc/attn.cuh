@@ -12,7 +12,7 @@ struct AttnParams {
   const void *q, *k_cache, *v_cache;
   void *out;
   DeviceStatus *status;
-  const int32_t *req_flag, *req_chunks;
+  const int32_t *req_chunks;
   const PlanHeader *header;
   PlanHeader *header_mut;  // same object: the work counter
   const WorkItem *items;  // in dispatch order
@@ -22,15 +22,13 @@ struct AttnParams {
                        // by the planner
 };
 
-// Host launchers (defined next to their kernels).
+// Host launchers (defined next to their kernels): programmatic dependents of the planner, which they wait for
+// before they read the plan.
 // CUDA-core kernel for fp32 KV, D in {64, 128}; `grid` persistent CTAs
 cudaError_t attn_f32_setup();  // once per device: shared-memory attributes
-cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s, bool pdl);
+cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s);
 // tcgen05 / TMA kernel for bf16 KV, D in {64, 128}; `grid` persistent CTAs
 cudaError_t attn_tc_setup();
-// pdl: programmatic dependent launch (the CTAs' set-up overlaps the previous kernel on `s`, which
-// the kernel waits for before it reads the plan); off where another stream's kernel should get the
-// SMs first
-cudaError_t attn_tc_launch(const AttnParams &p, int grid, cudaStream_t s, bool pdl);
+cudaError_t attn_tc_launch(const AttnParams &p, int grid, cudaStream_t s);
 
 }  // namespace wisp

@@ -355,7 +355,7 @@ cudaError_t attn_f32_setup() {
   return e;
 }
 
-cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s, bool pdl) {
+cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof cfg);
   cudaLaunchAttribute attr[1];
@@ -365,7 +365,7 @@ cudaError_t attn_f32_launch(const AttnParams &p, int grid, cudaStream_t s, bool 
   cfg.blockDim = dim3(kThreads);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 1;
   cfg.dynamicSmemBytes = p.D == 128 ? Cfg<128>::SMEM : Cfg<64>::SMEM;
   return p.D == 128 ? cudaLaunchKernelEx(&cfg, attn_f32_kernel<128>, p) : cudaLaunchKernelEx(&cfg, attn_f32_kernel<64>, p);
 }

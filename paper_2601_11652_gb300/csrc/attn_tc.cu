@@ -966,7 +966,7 @@ cudaError_t pool_maps(const AttnParams &p, PoolMaps *out) {
 
 }  // namespace
 
-cudaError_t attn_tc_launch(const AttnParams &p, int grid, cudaStream_t s, bool pdl) {
+cudaError_t attn_tc_launch(const AttnParams &p, int grid, cudaStream_t s) {
   PoolMaps m;
   const cudaError_t e = pool_maps(p, &m);
   if (e != cudaSuccess) return e;
@@ -982,7 +982,7 @@ cudaError_t attn_tc_launch(const AttnParams &p, int grid, cudaStream_t s, bool p
   cfg.blockDim = dim3(kThreads);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 1;
   if (p.D == 128) {
     cfg.dynamicSmemBytes = Cfg<128>::SMEM;
     return cudaLaunchKernelEx(&cfg, attn_tc_kernel<128>, p, tk, tv, tk8, tv8);

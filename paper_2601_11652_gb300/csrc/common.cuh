@@ -50,10 +50,6 @@ enum : int32_t { REQ_OK = 0, REQ_BAD = 1 };
 __device__ __forceinline__ float bf16_bits_to_float(uint32_t bits16) {
   return __uint_as_float(bits16 << 16);
 }
-__device__ __forceinline__ float load_elem(const float *p, int64_t i) { return __ldg(p + i); }
-__device__ __forceinline__ float load_elem(const __nv_bfloat16 *p, int64_t i) {
-  return __bfloat162float(p[i]);
-}
 
 // ---------------------------------------------------------------------------
 // Double-float ("ff") arithmetic: a value is hi + lo with |lo| <= ulp(hi)/2.
@@ -94,7 +90,6 @@ __device__ __forceinline__ ff ff_add_f(ff a, float b) {
   s.lo = __fadd_rn(s.lo, a.lo);
   return ff_fast_two_sum(s.hi, s.lo);
 }
-__device__ __forceinline__ ff ff_neg(ff a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ ff ff_mul(ff a, ff b) {
   ff p = ff_two_prod(a.hi, b.hi);
   p.lo = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
@@ -105,15 +100,8 @@ __device__ __forceinline__ ff ff_mul_f(ff a, float b) {
   p.lo = __fmaf_rn(a.lo, b, p.lo);
   return ff_fast_two_sum(p.hi, p.lo);
 }
-__device__ __forceinline__ bool ff_gt(ff a, ff b) {  // a > b
-  return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo);
-}
-__device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ ff ff_shfl_xor(ff a, int m) {
   return {__shfl_xor_sync(0xffffffffu, a.hi, m), __shfl_xor_sync(0xffffffffu, a.lo, m)};
-}
-__device__ __forceinline__ ff ff_shfl_up(ff a, int d) {
-  return {__shfl_up_sync(0xffffffffu, a.hi, d), __shfl_up_sync(0xffffffffu, a.lo, d)};
 }
 
 // 2^(j/256), j = 0..255, as double-float pairs; filled by the host from exp2 in double.

@@ -129,14 +129,14 @@ __device__ void plan_accept(const PlanParams &p, AcceptPlan &sh, bool one, int m
 }  // namespace
 
 // One CTA, bound by latency: global loads of the lengths, then barriers.  So: 32-bit scans with one barrier
-// each, each item's bucket kept from the pass that writes it, and no 64-bit division where 32 bits hold the
+// each, each item's request kept from pass to pass, and no 64-bit division where 32 bits hold the
 // operands.  With 64-bit scans of three barriers, separate passes and a binary search per pass, one request
 // took 9.7 us here and 256 requests 18.4 us (cold caches, launch included); now 8.6 and 15 us.
 __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // a kernel launched after this one with programmatic stream serialization (the attention) may
   // start its own set-up now; it reads the plan only after waiting for this grid to complete
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  constexpr int kKeep = 4;  // items per thread whose bucket is kept in registers
+  constexpr int kKeep = 4;  // items per thread whose request is kept in registers
   __shared__ int s_w[6][32];
   __shared__ unsigned long long s_sum[2];  // keys of the valid requests; passes over their KV tiles per KV head
   __shared__ int32_t s_valid;
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // shortest items and its CTAs finish close together.  Per chunk of kThreads requests: one thread per
   // request sizes its items (block scans into shared arrays), then consecutive threads take consecutive
   // items (the request found by binary search over the chunk's first items).  With one chunk of requests
-  // pass 4 finds the shared arrays as pass 3 left them and its items' requests and buckets in registers.
+  // pass 4 finds the shared arrays as pass 3 left them and its items' requests in registers.
   int32_t *s_first = sh.att.first;  // the chunk's requests' first items, relative
   // per request of the chunk: query rows, chunks (0: no items), first partial, context, first
   // query row, keys
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     }
     return bucket_of(t1 - t0);
   };
-  int keep[kKeep];  // request and bucket of this thread's first items
+  int keep[kKeep];  // the requests of this thread's first items
 #pragma unroll
   for (int x = 0; x < kKeep; ++x) keep[x] = 0;
   for (int base = 0; base < p.B; base += kThreads) {
@@ -370,11 +370,11 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     for (int i = tid; i < ti; i += kThreads, ++x) {
       if (item_carry + i >= p.max_items) break;  // (a request refused for want of room)
       int t0, t1;
-      const int lo = request_of(i), bucket = keys_of(i, lo, t0, t1);
-      atomicAdd(&s_hist[bucket], 1);
+      const int lo = request_of(i);
+      atomicAdd(&s_hist[keys_of(i, lo, t0, t1)], 1);
 #pragma unroll
       for (int y = 0; y < kKeep; ++y)
-        if (y == x) keep[y] = lo << 16 | bucket;
+        if (y == x) keep[y] = lo;
     }
     item_carry += ti;
     __syncthreads();  // the shared arrays are rewritten by the next chunk; the histogram is complete after the last
@@ -393,19 +393,15 @@ __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
     int x = 0;
     for (int i = tid; i < ti; i += kThreads, ++x) {
       if (item_carry + i >= p.max_items) break;
-      int lo = -1, bucket = 0;
+      int lo = -1;
       if (one) {
 #pragma unroll
         for (int y = 0; y < kKeep; ++y)
-          if (y == x) {
-            lo = keep[y] >> 16;
-            bucket = keep[y] & 0xffff;
-          }
+          if (y == x) lo = keep[y];
       }
       if (lo < 0) lo = request_of(i);
       WorkItem it;
-      const int b = keys_of(i, lo, it.t0, it.t1);
-      if (!one || x >= kKeep) bucket = b;
+      const int bucket = keys_of(i, lo, it.t0, it.t1);
       const int ch = max(1, s_ch[lo]);
       const int rws = s_rows[lo];
       const int ng = max(1, (rws + p.max_rows_item - 1) / p.max_rows_item);
