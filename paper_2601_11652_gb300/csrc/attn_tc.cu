@@ -404,28 +404,27 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) {
         int it = -1, passes = 1;
         WorkItem w;
-        uint32_t seen = *s_decided;
-        for (long long g0 = clock64();;) {
-          const uint32_t decided = *s_decided;
-          __threadfence_block();  // what was decided before it, too
-          if (redone != *s_nredo) {
-            __threadfence_block();
-            it = s_redo[redone++ % kRedo];
+        if (left && redone == *s_nredo) {
+          do {
+            it = atomicAdd(&p.header_mut->next_item, 1);
+            if (it >= n_items) { it = -1; break; }
             w = p.items[it];
-            passes = 2;
-            break;
-          }
-          if (left) {
-            do {
-              it = atomicAdd(&p.header_mut->next_item, 1);
-              if (it >= n_items) { it = -1; break; }
+          } while (!item_ok(p, w));
+          left = it >= 0;
+        }
+        if (it < 0) {  // an item to be taken again, or the end
+          uint32_t seen = 0;
+          for (long long g0 = clock64();;) {
+            const uint32_t decided = *s_decided;
+            __threadfence_block();  // and with them what they ask for
+            if (redone != *s_nredo) {
+              __threadfence_block();
+              it = s_redo[redone++ % kRedo];
               w = p.items[it];
-            } while (!item_ok(p, w));
-            if (it >= 0) break;
-            left = false;
-          } else if (decided == items) {
-            break;
-          } else {
+              passes = 2;
+              break;
+            }
+            if (decided == items) break;
             if (decided != seen) g0 = clock64();
             seen = decided;
             if (*s_abort || clock64() - g0 > kWaitCycles) {
@@ -771,16 +770,18 @@ __global__ void __launch_bounds__(kThreads, 1)
           // quadrants: the references.  Padding rows get +inf (P = 0), rows without a visible key 0 (P = 0:
           // all their scores are -inf).  s_red alternates between items: a warp that writes it for item
           // li + 2 has passed the barrier of item li + 1, where every reader of item li has arrived.
+          float wm = -INFINITY;
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             if (u < nu) {
 #pragma unroll
               for (int i = 8 * u; i < 8 * u + 8; ++i) {
                 const float rm = ptx::warp_max(__uint_as_float(x[i >> 4][i & 15]));
-                if (lane == i) mref = fmaxf(mref, rm);
+                if (lane == i) wm = rm;
               }
             }
           }
+          mref = fmaxf(mref, wm);
           pre += apart ? 1 : -1;
           if (pre == 0) {
             float *red = s_red + (li & 1) * 4 * kNR + r0 + lane;
