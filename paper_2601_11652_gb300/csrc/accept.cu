@@ -966,11 +966,8 @@ __device__ __noinline__ int pair_token(const AcceptParams &p, const Sm &sm, cons
 // weights of 64 vectors at a time (a tile; two neighbouring vectors per lane, one element of each at a
 // time), a warp scan in token order, then the elements of the crossing's two vectors, one lane each; with
 // take_last, or when rounding leaves no crossing, the last element with weight.  Writes the request's
-// outputs.  Against one vector per lane in two turns (weights from a table in L2, the crossing vector's E
-// double-precision weights by one lane in a row), acceptance on GB300: 32 requests 66 -> 60 us, 256 requests
-// 177 -> 166 us, 512 requests with 4K tokens of vocabulary 175 -> 135 us.  Unrolled, with the exps of both
-// vectors side by side, it was slower than before (32 requests 68 us): code run once is fetched at about 100
-// cycles per 8 instructions.
+// outputs.  Not unrolled: code that runs once is fetched at about 100 cycles per 8 instructions, and with the
+// exps of both vectors side by side 32 requests took 68 us against 60.
 template <typename LT>
 __device__ void keeper_finish(const AcceptParams &p, const Sm &sm, int r, int i, bool resid, int64_t Q0, int64_t D0,
                               float m, double Zu, int64_t v0, int64_t v1, double thr, bool take_last) {

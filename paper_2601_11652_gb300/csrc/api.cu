@@ -521,8 +521,9 @@ wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args 
   if (attn->B == 0) return launch_plan(attn, acc, ws, L, sms, true, s);
   // One planner for both parts.  The attention follows it on `s` as its programmatic dependent
   // (persistent, one CTA per SM); the acceptance pass reads only the logits and the planner's
-  // state, so it runs on the library's side stream, forked after the planner and joined back: its
-  // CTAs take the SMs the attention's CTAs leave as they finish.
+  // state, so it runs on the library's side stream, forked after the planner and joined back.  The
+  // planner gives the attention a share of the SMs: its other CTAs exit at once, and the acceptance
+  // CTAs start there.
   DeviceInfo &d = g_dev[dev];
   std::lock_guard<std::mutex> lk(d.step_mu);
   SideSlot *sl = side_slot(d, s);
@@ -531,7 +532,7 @@ wisp_status wisp_verify_step(const wisp_attn_args *attn, const wisp_accept_args 
   const AcceptParams ap = accept_params(acc, ws, L, sms);
   const bool bf = acc->logits_dtype == WISP_BF16;
   // the attention is enqueued first, so that its CTAs take the SMs first; the acceptance part of
-  // the plan and the acceptance CTAs follow on the side stream, on the SMs the attention leaves
+  // the plan and the acceptance CTAs follow on the side stream
   bool ok = cudaEventRecord(sl->ev_fork, s) == cudaSuccess;
   ok = ok && launch_attention(attn, ws, L, s) == WISP_OK;
   const bool forked = ok && cudaStreamWaitEvent(sl->side, sl->ev_fork, 0) == cudaSuccess;

@@ -20,12 +20,14 @@
 // At the item's end the warps' (O, m, l) are merged in shared memory; the last chunk of a split merges
 // the chunks' partials.
 //
-// What bounds it: fp32 multiply-adds at 32 rows (two per key, row and head-dim element; about 74 TFLOP/s
-// on 152 SMs), of which it reaches half: the scores read RL + 2 floats per lane for 2 RL products, and
-// shared memory delivers one float a lane per four multiply-adds.  Below about 8 rows, the K / V stream
-// (4.7 TB/s at 4 rows).  With the previous kernel (32-token tiles staged through scalar loads, one warp
-// shuffle per key and row, accumulators in shared memory) 32 requests of 512-4096 tokens, 32 query and 8
-// KV heads, D = 128 took 5870 us; now 290 us.
+// What bounds it: at full items the reads that feed the score loop (RL + 2 16-byte loads for 4 RL packed
+// multiply-adds, at RL = 8 about 40 cycles of the shared-memory return path against 16 of arithmetic)
+// and the two warps a scheduler has to hide its latencies with; at few rows the K / V stream.  38
+// requests of 8192 tokens, 8 KV heads, D = 128: 38.7 TFLOP/s at 32 rows (about half of the fp32
+// rate), 29.0 at 16, 4.4 TB/s at 8, 4.8 TB/s at 4.  32 requests of 512-4096 tokens with 8 to 36 rows:
+// 285 us, 26.6 TFLOP/s; shared memory is busy 51% of the time there, issue 38%, DRAM 29%.  At RL = 8 and
+// D = 128 the 255 registers do not hold everything: 116 bytes of spills a thread (none at D = 64), 0.2%
+// of its instructions.
 #include "attn_merge.cuh"
 
 #include <cstring>

@@ -35,12 +35,10 @@
 //     (request, head, row group) to finish merges all its chunks.  This runs while the softmax
 //     warps are already on the next item.
 // What bounds it: the K and V stream (HBM).  An SM's own limit is the softmax warps' chain per tile
-// (read S^T, P, publish): 0.80 us a 128-key tile at 4 query rows and 1.06 us at 64 with K and V in L2,
-// against the 1.47 us that a tile's 64 KB take at an SM's share of the copy rate (D = 128).  With one
-// thread issuing both products, a vote of the softmax warps per tile and the barrier pointers in local
-// memory those were 1.42 and 1.78 us.  An item of one tile takes 4 us (its claim, Q copy, first-tile
-// references and epilogue overlap its neighbours'); with a division per query row in the Q copy and the
-// epilogue, and one warp for claims and Q, 7.5 us.
+// (read S^T, P, publish): 0.77 us a 128-key tile up to 32 query rows and 0.90 us at 64 with K and V in L2,
+// against the 1.47 us that a tile's 64 KB take at an SM's share of the copy rate (D = 128; at 64 the
+// tile's 32 KB take 0.74).  An item of one tile takes 4 us (its claim, Q copy, first-tile references and
+// epilogue overlap its neighbours').
 //
 // Every mbarrier wait is bounded in time; an expired wait records WISP_DEV_TIMEOUT and the CTA
 // drains.  No named barrier is used: a warp that gives up cannot leave the others blocked, and the
@@ -456,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
   } else if (warp == 17) {
     // ------------------------------------------------------------------ Q loader
-    // (a warp of its own: claiming an item and copying its rows in turn took 7.5 us, which bounded short items)
+    // (a warp of its own: in the item loader, the copy would delay the next claim, which bounds short items)
     int li = 0;
     bool ok = true;
     for (uint32_t j = 0; ok; ++j) {
@@ -504,9 +502,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!ok && lane == 0) report(p.status, WISP_DEV_TIMEOUT, p.request_ids, 0);
   } else if (warp == 1 || warp == 16) {
     // ------------------------------------------------------------------ MMA issuers
-    // One warp issues S^T, another PV, so that neither waits behind the other's barriers: one thread
-    // for both took 2400-2900 cycles a tile (about 45-90 per MMA, 100 per commit, and the polling of
-    // both queues), which bounded every item whatever its rows; the two run side by side.
+    // One warp issues S^T, another PV, so that neither waits behind the other's barriers: an MMA takes
+    // its issuer 45-90 cycles and a commit 100, and one thread for both would bound every item.
     const bool is_s = warp == 1;
     uint32_t n = 0;
     int li = 0;
@@ -645,8 +642,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const float lsum = hl[jl] + hl[kNR + jl] + hl[2 * kNR + jl] + hl[3 * kNR + jl];
         if (w.poff < 0) {
           const float linv = 1.0f / lsum;
-          // (row pointers stepped from row to row: with a division per row, the epilogue took 5-7 us an item and
-          // bounded items of a few tiles)
+          // (row pointers stepped from row to row: a division per row would bound items of a few tiles)
           int hh = w.row0 + 32 * c - div_g(w.row0 + 32 * c) * g;
           uint16_t *og = static_cast<uint16_t *>(p.out) +
                          ((int64_t)(w.q0 + div_g(w.row0 + 32 * c)) * p.Hq + w.h * g + hh) * D + d;
@@ -705,9 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // work).  Within a group, one warp per TMEM lane quadrant, i.e. 32 keys of each tile: a thread holds
     // one key's scores for the group's rows.  The rows' reference maxima are those of the item's first
     // tile (its four warps exchange them once per item): a key of the item that a row can see at all is
-    // preceded by one in the first tile, and later tiles then need no agreement between warps.  (A vote
-    // of the eight warps on every tile, with a second pass over tiles that moved a reference, took
-    // 700-1000 of about 2900 cycles a tile.)
+    // preceded by one in the first tile, and later tiles then need no agreement between warps.
     const int qd = warp & 3;                  // TMEM lane quadrant: keys 32*qd .. 32*qd + 31 of a tile
     const int grp = warp >= 12 ? 1 : 0;
     const uint32_t lane_addr = (uint32_t)(qd * 32) << 16;

@@ -80,10 +80,9 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Bound by the latency of reading the block tables (4 bytes a page, 0.1-1 MB a batch).  A warp reads one
-// request's row, lanes side by side and four loads ahead.  With a thread per request walking its row, in
-// one CTA, a served round of 64 requests of up to 2048 pages took 431 us (this kernel 196 us of it in a
-// cold-cache profile); now the round takes 289 us.
+// Bound by the latency of reading the block tables (4 bytes a page, 0.1-1 MB a batch) and of its barriers.  A
+// warp reads one request's row, lanes side by side and four loads ahead.  64 requests of up to 2048
+// pages: 16 us with cold caches.
 __global__ void __launch_bounds__(kThreads) __cluster_dims__(kReserveCtas, 1, 1) kv_reserve_kernel(const KvParams p) {
   // the append kernel may be placed now; it waits for this grid before it reads anything
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -130,8 +130,7 @@ __device__ void plan_accept(const PlanParams &p, AcceptPlan &sh, bool one, int m
 
 // One CTA, bound by latency: global loads of the lengths, then barriers.  So: 32-bit scans with one barrier
 // each, each item's request kept from pass to pass, and no 64-bit division where 32 bits hold the
-// operands.  With 64-bit scans of three barriers, separate passes and a binary search per pass, one request
-// took 9.7 us here and 256 requests 18.4 us (cold caches, launch included); now 8.6 and 15 us.
+// operands.  One request takes 8.6 us here and 256 requests 15 us (cold caches, launch included).
 __global__ void __launch_bounds__(kThreads, 1) plan_kernel(const PlanParams p) {
   // a kernel launched after this one with programmatic stream serialization (the attention) may
   // start its own set-up now; it reads the plan only after waiting for this grid to complete
